@@ -17,40 +17,86 @@ constexpr int kBlock = 256;
 constexpr int kWarps = kBlock / 32;
 constexpr int kViewChunk = 256;   // views whose partial results a block keeps in shared memory at once
 
-// Camera constants of the visibility test: rotation, centre, intrinsics, image size.
-struct VisCam {
-  float R[9];
-  float T[3];
-  float fx, fy, cx, cy;
-  float W, H;
+// Camera constants of the visibility test, as seven 16-byte vectors (a stride of 28 words:
+// lanes reading different cameras with 16-byte loads meet no bank conflict).
+struct __align__(16) VisCam {
+  float4 a;   // T, R2
+  float4 b;   // R5, R8, R0, R3
+  float4 c;   // R6, R1, R4, R7
+  float4 k;   // fx, fy, cx, cy
+  float4 w;   // W, H, |dt_z/dmu|, scale of the rounding margin
+  float4 g;   // |d(fx t_x + cx t_z)/dmu|, the same with cx - W, and both for y
+  float4 e;   // 1e-6 (|cx| + |W|), 1e-6 (|cy| + |H|), cx - W, cy - H
 };
 
 __device__ inline void load_vis_cam(const gs_camera& g, VisCam& c) {
-#pragma unroll
-  for (int i = 0; i < 9; ++i) c.R[i] = g.R[i];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) c.T[i] = g.T[i];
-  c.fx = g.fx;
-  c.fy = g.fy;
-  c.cx = g.cx;
-  c.cy = g.cy;
-  c.W = (float)g.width;
-  c.H = (float)g.height;
+  const float* R = g.R;
+  const float W = (float)g.width, H = (float)g.height;
+  c.a = make_float4(g.T[0], g.T[1], g.T[2], R[2]);
+  c.b = make_float4(R[5], R[8], R[0], R[3]);
+  c.c = make_float4(R[6], R[1], R[4], R[7]);
+  c.k = make_float4(g.fx, g.fy, g.cx, g.cy);
+  const float n0 = norm3df(R[0], R[3], R[6]), n1 = norm3df(R[1], R[4], R[7]), n2 = norm3df(R[2], R[5], R[8]);
+  auto plane = [&](int j, float f, float k) {   // norm of the gradient of f t_j + k t_z
+    return norm3df(f * R[j] + k * R[2], f * R[3 + j] + k * R[5], f * R[6 + j] + k * R[8]);
+  };
+  c.g = make_float4(plane(0, g.fx, g.cx), plane(0, g.fx, g.cx - W), plane(1, g.fy, g.cy), plane(1, g.fy, g.cy - H));
+  const float mx = fabsf(g.fx) * n0 + (fabsf(g.cx) + fabsf(W)) * n2;
+  const float my = fabsf(g.fy) * n1 + (fabsf(g.cy) + fabsf(H)) * n2;
+  c.w = make_float4(W, H, n2, 1e-4f * fmaxf(mx, my));
+  c.e = make_float4(1e-6f * (fabsf(g.cx) + fabsf(W)), 1e-6f * (fabsf(g.cy) + fabsf(H)), g.cx - W, g.cy - H);
 }
 
 // v(x, g): t = R^T (mu - T) with each product and sum rounded separately, in the
 // order ((R0 dx + R3 dy) + R6 dz); visible iff near < t_z <= range and the
 // projection (fx t_x / t_z + cx, fy t_y / t_z + cy) lies in [0, W) x [0, H).
+// The two correctly rounded divisions (most of the test's instructions) are only made when
+// fx t_x + cx t_z is within 1e-6 of its terms from 0 or from W t_z: further away, the few
+// units of 2^-24 by which the separately rounded quotient and sum can be off do not matter.
 __device__ __forceinline__ bool visible(float mx, float my, float mz, const VisCam& c, float near_plane,
                                         float range) {
-  const float dx = __fsub_rn(mx, c.T[0]), dy = __fsub_rn(my, c.T[1]), dz = __fsub_rn(mz, c.T[2]);
-  const float tz = __fadd_rn(__fadd_rn(__fmul_rn(c.R[2], dx), __fmul_rn(c.R[5], dy)), __fmul_rn(c.R[8], dz));
+  const float4 ca = c.a, cb = c.b;
+  const float dx = __fsub_rn(mx, ca.x), dy = __fsub_rn(my, ca.y), dz = __fsub_rn(mz, ca.z);
+  const float tz = __fadd_rn(__fadd_rn(__fmul_rn(ca.w, dx), __fmul_rn(cb.x, dy)), __fmul_rn(cb.y, dz));
   if (!(tz > near_plane) || !(tz <= range)) return false;
-  const float tx = __fadd_rn(__fadd_rn(__fmul_rn(c.R[0], dx), __fmul_rn(c.R[3], dy)), __fmul_rn(c.R[6], dz));
-  const float ty = __fadd_rn(__fadd_rn(__fmul_rn(c.R[1], dx), __fmul_rn(c.R[4], dy)), __fmul_rn(c.R[7], dz));
-  const float u = __fadd_rn(__fdiv_rn(__fmul_rn(c.fx, tx), tz), c.cx);
-  const float v = __fadd_rn(__fdiv_rn(__fmul_rn(c.fy, ty), tz), c.cy);
-  return u >= 0.f && u < c.W && v >= 0.f && v < c.H;
+  const float4 cc = c.c, k = c.k, e = c.e;
+  const float tx = __fadd_rn(__fadd_rn(__fmul_rn(cb.z, dx), __fmul_rn(cb.w, dy)), __fmul_rn(cc.x, dz));
+  const float ty = __fadd_rn(__fadd_rn(__fmul_rn(cc.y, dx), __fmul_rn(cc.z, dy)), __fmul_rn(cc.w, dz));
+  const float ax = __fmul_rn(k.x, tx), ay = __fmul_rn(k.y, ty);
+  const float ex = fmaf(e.x, tz, 1e-6f * fabsf(ax)), ey = fmaf(e.y, tz, 1e-6f * fabsf(ay));
+  const float x0 = fmaf(k.z, tz, ax), x1 = fmaf(e.z, tz, ax);   // t_z u, t_z (u - W)
+  const float y0 = fmaf(k.w, tz, ay), y1 = fmaf(e.w, tz, ay);
+  if (tz > 1e-20f) {   // (the relative bound holds while nothing is subnormal)
+    if (x0 < -ex || x1 > ex || y0 < -ey || y1 > ey) return false;
+    if (x0 > ex && x1 < -ex && y0 > ey && y1 < -ey) return true;
+  }
+  const float u = __fadd_rn(__fdiv_rn(ax, tz), k.z);
+  const float v = __fadd_rn(__fdiv_rn(ay, tz), k.w);
+  return u >= 0.f && u < c.w.x && v >= 0.f && v < c.w.y;
+}
+
+// Group cull: false only if no mean within `rad` of (gx, gy, gz) can be visible.  t_z and the
+// four functions fx t_x + cx t_z >= 0, fx t_x + (cx - W) t_z < 0 (and the same in y) are
+// linear in the mean, so over the sphere each differs from its value at the centre by at most
+// rad times the norm of its gradient; the margin (1e-4 of the terms' magnitudes, against a few
+// units of 2^-24 that the separately rounded test can be off) covers both evaluations.
+// Comparisons with a NaN keep the view.
+__device__ __forceinline__ bool group_may_see(float gx, float gy, float gz, float rad, const VisCam& c,
+                                              float near_plane, float range) {
+  const float4 ca = c.a, cb = c.b, cc = c.c, k = c.k, w = c.w, g = c.g;
+  const float dx = gx - ca.x, dy = gy - ca.y, dz = gz - ca.z;
+  const float tx = cb.z * dx + cb.w * dy + cc.x * dz;
+  const float ty = cc.y * dx + cc.z * dy + cc.w * dz;
+  const float tz = ca.w * dx + cb.x * dy + cb.y * dz;
+  const float ext = fabsf(dx) + fabsf(dy) + fabsf(dz) + rad;
+  const float mz = w.z * (rad * 1.0001f + 1e-4f * ext) + 1e-6f;
+  if (tz + mz <= near_plane || tz - mz > range * 1.0001f) return false;
+  const float m = w.w * ext + 1e-6f, r = rad * 1.0001f;
+  if (k.x * tx + k.z * tz < -(g.x * r + m)) return false;
+  if (k.x * tx + (k.z - w.x) * tz > g.y * r + m) return false;
+  if (k.y * ty + k.w * tz < -(g.z * r + m)) return false;
+  if (k.y * ty + (k.w - w.y) * tz > g.w * r + m) return false;
+  return true;
 }
 
 // u_i = |mu_cur - mu_prev| (or its square); unchanged means keep their u.
@@ -65,69 +111,118 @@ __global__ void k_uncertainty_update(const float4* __restrict__ mo_prev, const f
   }
 }
 
-// Fixed-order block sum of doubles; valid in thread 0.
-__device__ double block_sum_d(double v, double* s) {
+constexpr int kMomThreads = 512;   // threads of the threshold kernels
+constexpr int kMomBlocks = 340;    // at most: sums, counts and squares of every block fill 1,020 of 1,024 slots
+
+__device__ __forceinline__ double warp_sum_d(double v) {
+#pragma unroll
   for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+  return v;   // valid in lane 0
+}
+
+// Fixed-order block sum of doubles; valid in thread 0.  (A warp's FP64 addition holds the
+// SM's FP64 unit for many cycles whatever the number of active lanes: only one warp adds the
+// warps' sums.)
+__device__ double block_sum_d(double v, double* s) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v = warp_sum_d(v);
+  __syncthreads();
   if (lane == 0) s[warp] = v;
   __syncthreads();
   double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s[w];
-  __syncthreads();
+  if (warp == 0) t = warp_sum_d(lane < (int)(blockDim.x >> 5) ? s[lane] : 0.0);
   return t;
 }
 
-// Per block: sum of u over the block's Gaussians (pass 0), or of (u - mean)^2
-// (pass 1), in a fixed order, into part[block].  Gaussians with mu_z < ground_z
-// are left out.
-__global__ void __launch_bounds__(kBlock) k_u_moments(const float4* __restrict__ mo, const float4* __restrict__ su,
-                                                      int64_t n, float ground_z, const double* __restrict__ stats,
-                                                      int pass, double* __restrict__ part) {
-  __shared__ double s[kWarps];
-  const double mean = pass ? stats[0] : 0.0;
+// Sum of g per-block partials in a fixed order by one warp; valid in lane 0.
+__device__ double sum_partials(const double* __restrict__ part, int g) {
+  double v = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x & 31; b < g; b += 32) v += part[b];
+  return warp_sum_d(v);
+}
+
+// Mean and spread of u over the Gaussians with mu_z >= ground_z, two passes over contiguous
+// block ranges.  Pass 0: part[b] = sum of u, part[g + b] = number of Gaussians (exact in FP64).
+// Pass 1: every block first forms the mean from pass 0's partials (a few hundred values from
+// L2, in the same order everywhere) and stores its sum of squared deviations in
+// part[2 g + b].  The last kernel forms the statistics.  Three launches; at first the count
+// and the two sums were finished in kernels of their own, by a single thread adding 304 values
+// one after the other (1M Gaussians: 80 us in six launches, now 34 us).
+template <int kPass>
+__global__ void __launch_bounds__(kMomThreads) k_u_moments(const float4* __restrict__ mo,
+                                                           const float4* __restrict__ su, int64_t n, float ground_z,
+                                                           double* __restrict__ part) {
+  __shared__ double s[kMomThreads / 32];
+  const int g = gridDim.x, warp = threadIdx.x >> 5;
+  double mean = 0.0;
+  if (kPass) {
+    if (warp < 2) {   // warp 0 the sum, warp 1 the count
+      const double t = sum_partials(part + warp * g, g);
+      if ((threadIdx.x & 31) == 0) s[warp] = t;
+    }
+    __syncthreads();
+    mean = s[1] > 0.0 ? s[0] / s[1] : 0.0;
+  }
   double acc = 0.0;
-  const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+  uint32_t cnt = 0;
+  const int64_t per = (n + g - 1) / g;
   const int64_t i0 = (int64_t)blockIdx.x * per;
   int64_t i1 = i0 + per;
   if (i1 > n) i1 = n;
-  for (int64_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-    if (!(mo[i].z >= ground_z)) continue;
-    const double u = (double)su[i].w;
-    acc += pass ? (u - mean) * (u - mean) : u;
+#pragma unroll 4
+  for (int64_t i = i0 + threadIdx.x; i < i1; i += kMomThreads) {
+    const float z = mo[i].z, uf = su[i].w;
+    if (!(z >= ground_z)) continue;
+    const double u = (double)uf;
+    acc += kPass ? (u - mean) * (u - mean) : u;
+    ++cnt;
   }
   const double t = block_sum_d(acc, s);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
+  if (kPass == 0) {
+    const uint32_t w = __reduce_add_sync(0xffffffffu, cnt);
+    __shared__ unsigned long long s_cnt;
+    if (threadIdx.x == 0) s_cnt = 0ull;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) atomicAdd(&s_cnt, (unsigned long long)w);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      part[blockIdx.x] = t;
+      part[g + blockIdx.x] = (double)s_cnt;
+    }
+  } else if (threadIdx.x == 0) {
+    part[2 * g + blockIdx.x] = t;
+  }
 }
 
-__global__ void k_u_count(const float4* __restrict__ mo, int64_t n, float ground_z, unsigned long long* cnt) {
-  unsigned long long c = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    c += (mo[i].z >= ground_z) ? 1ull : 0ull;
-  for (int d = 16; d > 0; d >>= 1) c += __shfl_down_sync(0xffffffffu, c, d);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(cnt, c);
-}
-
-// stats = (mean, sigma, t_high = mean + sigma/2, t_low = mean - sigma/2, count)
-__global__ void k_u_finish(const double* __restrict__ part, int g, const unsigned long long* cnt, int pass,
-                           double* __restrict__ stats) {
-  double t = 0.0;
-  for (int b = 0; b < g; ++b) t += part[b];
-  const double m = (double)*cnt;
-  if (pass == 0) {
-    stats[0] = m > 0 ? t / m : 0.0;
-    stats[4] = m;
-  } else {
-    const double sigma = m > 0 ? sqrt(t / m) : 0.0;
+// stats = (mean, sigma, t_high = mean + sigma/2, t_low = mean - sigma/2, count); 96 threads
+__global__ void __launch_bounds__(96) k_u_finish(const double* __restrict__ part, int g, double* __restrict__ stats) {
+  __shared__ double s[3];
+  const int warp = threadIdx.x >> 5;
+  const double t = sum_partials(part + warp * g, g);
+  if ((threadIdx.x & 31) == 0) s[warp] = t;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double m = s[1], mean = m > 0.0 ? s[0] / m : 0.0, sigma = m > 0.0 ? sqrt(s[2] / m) : 0.0;
+    stats[0] = mean;
     stats[1] = sigma;
-    stats[2] = stats[0] + 0.5 * sigma;
-    stats[3] = stats[0] - 0.5 * sigma;
+    stats[2] = mean + 0.5 * sigma;
+    stats[3] = mean - 0.5 * sigma;
+    stats[4] = m;
   }
 }
 
 // Per block and view: xi mode: count of visible high-uncertainty Gaussians minus
 // lambda * count of visible low ones (both counted exactly as integers, combined in
 // the final pass); sum mode: sum of u over the visible Gaussians.
+//
+// Bound: FP32 issue on the visibility tests.  A warp holds 32 consecutive Gaussians, which a
+// map built keyframe by keyframe has close together: 32 views at a time, one per lane, are
+// first tested against a sphere around the warp's Gaussians that count (group_may_see), and
+// only the views that pass are tested lane by lane.  A map in random order pays one group
+// test per 32 lane tests.  1M room Gaussians, 256 views: 672 us with every pair tested, 206 us
+// with the group cull, 146 us with the test's divisions left out where they cannot matter and
+// the warps' groups strided over the map.
 template <bool kSum>
 __global__ void __launch_bounds__(kBlock) k_view_utility(const float4* __restrict__ mo, const float4* __restrict__ su,
                                                          int64_t n, const gs_camera* __restrict__ cams, int v0, int nv,
@@ -135,49 +230,69 @@ __global__ void __launch_bounds__(kBlock) k_view_utility(const float4* __restric
                                                          uint32_t* __restrict__ cnt_part, float* __restrict__ sum_part,
                                                          int n_views) {
   __shared__ VisCam s_cam[kViewChunk];
-  __shared__ uint32_t s_hi[kWarps][kViewChunk];
-  __shared__ uint32_t s_lo[kWarps][kViewChunk];
-  __shared__ float s_sum[kWarps][kViewChunk];
+  __shared__ uint32_t s_acc[kSum ? 1 : 2][kWarps][kViewChunk];   // visible high, low; or the sum of u (float)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int i = threadIdx.x; i < nv; i += blockDim.x) load_vis_cam(cams[v0 + i], s_cam[i]);
-  for (int i = threadIdx.x; i < kWarps * kViewChunk; i += blockDim.x) {
-    (&s_hi[0][0])[i] = 0u;
-    (&s_lo[0][0])[i] = 0u;
-    (&s_sum[0][0])[i] = 0.f;
-  }
+  for (int i = threadIdx.x; i < (kSum ? 1 : 2) * kWarps * kViewChunk; i += blockDim.x) (&s_acc[0][0][0])[i] = 0u;
   __syncthreads();
+  uint32_t* a_hi = s_acc[0][warp];
+  uint32_t* a_lo = s_acc[kSum ? 0 : 1][warp];
+  float* a_sum = reinterpret_cast<float*>(a_hi);
   const double t_hi = kSum ? 0.0 : stats[2], t_lo = kSum ? 0.0 : stats[3];
-  // this block's Gaussians, 32 per warp at a time
-  const int64_t per = ((n + gridDim.x - 1) / gridDim.x + 31) / 32 * 32;
-  const int64_t i0 = (int64_t)blockIdx.x * per;
-  int64_t i1 = i0 + per;
-  if (i1 > n) i1 = n;
-  for (int64_t base = i0 + warp * 32; base < i1; base += kBlock) {
+  // 32 Gaussians per warp at a time, strided over the map: what a stretch of it costs depends
+  // on how many views see that part of the room
+  for (int64_t base = (int64_t)blockIdx.x * kBlock + warp * 32; base < n; base += (int64_t)gridDim.x * kBlock) {
     const int64_t i = base + lane;
     float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
     float u = 0.f;
     bool use = false;
-    if (i < i1) {
+    if (i < n) {
       m = mo[i];
       u = su[i].w;
       use = m.z >= prm.ground_z;
     }
     const bool hi = use && !kSum && (double)u > t_hi;
     const bool lo = use && !kSum && (double)u < t_lo;
-    const bool any = __any_sync(0xffffffffu, kSum ? use : (hi || lo));
-    if (!any) continue;
-    for (int v = 0; v < nv; ++v) {
-      const bool vis = (kSum ? use : (hi || lo)) && visible(m.x, m.y, m.z, s_cam[v], prm.near_plane, prm.range);
-      if (kSum) {
-        float s = vis ? u : 0.f;
+    const bool in = kSum ? use : (hi || lo);
+    const uint32_t mask = __ballot_sync(0xffffffffu, in);
+    if (!mask) continue;
+    // sphere around the group's counted means
+    float gx = in ? m.x : 0.f, gy = in ? m.y : 0.f, gz = in ? m.z : 0.f;
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
-        if (lane == 0) s_sum[warp][v] += s;
-      } else {
-        const uint32_t bh = __ballot_sync(0xffffffffu, vis && hi), bl = __ballot_sync(0xffffffffu, vis && lo);
-        if (lane == 0) {
-          s_hi[warp][v] += __popc(bh);
-          s_lo[warp][v] += __popc(bl);
+    for (int d = 16; d > 0; d >>= 1) {
+      gx += __shfl_xor_sync(0xffffffffu, gx, d);
+      gy += __shfl_xor_sync(0xffffffffu, gy, d);
+      gz += __shfl_xor_sync(0xffffffffu, gz, d);
+    }
+    const float inv = 1.f / (float)__popc(mask);
+    gx *= inv;
+    gy *= inv;
+    gz *= inv;
+    const float ex = m.x - gx, ey = m.y - gy, ez = m.z - gz;
+    // (a NaN or infinite mean makes the radius infinite: nothing is culled)
+    const float r2 = in ? ex * ex + ey * ey + ez * ez : 0.f;
+    const bool odd = __any_sync(0xffffffffu, !(r2 < INFINITY));
+    const float rad = odd ? INFINITY : sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(r2)))) * 1.0001f;
+    for (int vb = 0; vb < nv; vb += 32) {
+      const int iv = vb + lane;
+      const bool may = iv < nv && (odd || group_may_see(gx, gy, gz, rad, s_cam[iv], prm.near_plane, prm.range));
+      uint32_t cand = __ballot_sync(0xffffffffu, may);
+      while (cand) {
+        const int v = vb + __ffs(cand) - 1;
+        cand &= cand - 1u;
+        const bool vis = in && visible(m.x, m.y, m.z, s_cam[v], prm.near_plane, prm.range);
+        if (kSum) {
+          float s = vis ? u : 0.f;
+          if (!__any_sync(0xffffffffu, vis)) continue;
+#pragma unroll
+          for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
+          if (lane == 0) a_sum[v] += s;
+        } else {
+          const uint32_t bh = __ballot_sync(0xffffffffu, vis && hi), bl = __ballot_sync(0xffffffffu, vis && lo);
+          if (lane == 0 && (bh | bl)) {
+            a_hi[v] += __popc(bh);
+            a_lo[v] += __popc(bl);
+          }
         }
       }
     }
@@ -187,60 +302,140 @@ __global__ void __launch_bounds__(kBlock) k_view_utility(const float4* __restric
     const size_t o = (size_t)blockIdx.x * n_views + v0 + v;
     if (kSum) {
       float s = 0.f;
-      for (int w = 0; w < kWarps; ++w) s += s_sum[w][v];
+      for (int w = 0; w < kWarps; ++w) s += __uint_as_float(s_acc[0][w][v]);
       sum_part[o] = s;
     } else {
       uint32_t h = 0, l = 0;
       for (int w = 0; w < kWarps; ++w) {
-        h += s_hi[w][v];
-        l += s_lo[w][v];
+        h += s_acc[0][w][v];
+        l += s_acc[kSum ? 0 : 1][w][v];
       }
-      cnt_part[2 * o] = h;
-      cnt_part[2 * o + 1] = l;
+      *reinterpret_cast<uint2*>(cnt_part + 2 * o) = make_uint2(h, l);
     }
   }
 }
 
+// One warp per view adds the g blocks' partials (lanes take every 32nd, then a fixed tree).
+// One thread per view, walking all partials by itself, took 41 us for 256 views.
 template <bool kSum>
-__global__ void k_view_utility_finish(const uint32_t* __restrict__ cnt_part, const float* __restrict__ sum_part,
-                                      int g, int n_views, float lambda, float* __restrict__ xi,
-                                      uint32_t* __restrict__ counts) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(kBlock) k_view_utility_finish(const uint32_t* __restrict__ cnt_part,
+                                                                const float* __restrict__ sum_part, int g,
+                                                                int n_views, float lambda, float* __restrict__ xi,
+                                                                uint32_t* __restrict__ counts) {
+  const int v = blockIdx.x * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (v >= n_views) return;
   if (kSum) {
     float s = 0.f;
-    for (int b = 0; b < g; ++b) s += sum_part[(size_t)b * n_views + v];
-    xi[v] = s;
+    for (int b = lane; b < g; b += 32) s += sum_part[(size_t)b * n_views + v];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_down_sync(0xffffffffu, s, d);
+    if (lane == 0) xi[v] = s;
   } else {
     unsigned long long h = 0, l = 0;
-    for (int b = 0; b < g; ++b) {
-      h += cnt_part[2 * ((size_t)b * n_views + v)];
-      l += cnt_part[2 * ((size_t)b * n_views + v) + 1];
+    for (int b = lane; b < g; b += 32) {
+      const uint2 c = *reinterpret_cast<const uint2*>(cnt_part + 2 * ((size_t)b * n_views + v));
+      h += c.x;
+      l += c.y;
     }
-    xi[v] = (float)((double)h - (double)lambda * (double)l);
-    if (counts) {
-      counts[2 * v] = (uint32_t)h;
-      counts[2 * v + 1] = (uint32_t)l;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      h += __shfl_down_sync(0xffffffffu, h, d);
+      l += __shfl_down_sync(0xffffffffu, l, d);
+    }
+    if (lane == 0) {
+      xi[v] = (float)((double)h - (double)lambda * (double)l);
+      if (counts) {
+        counts[2 * v] = (uint32_t)h;
+        counts[2 * v + 1] = (uint32_t)l;
+      }
     }
   }
 }
 
 // Mean uncertainty of cuboid regions: region (ix, iy, iz) with i = floor((mu - origin) / size)
 // holds the Gaussians inside the grid; sums in FP64, counts exact.
-__global__ void k_regions(const float4* __restrict__ mo, const float4* __restrict__ su, int64_t n,
-                          gs_region_grid grid, double* __restrict__ sum, uint32_t* __restrict__ count) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float4 m = mo[i];
-    const float fx = floorf(__fdiv_rn(__fsub_rn(m.x, grid.origin[0]), grid.size));
-    const float fy = floorf(__fdiv_rn(__fsub_rn(m.y, grid.origin[1]), grid.size));
-    const float fz = floorf(__fdiv_rn(__fsub_rn(m.z, grid.origin[2]), grid.size));
-    if (!(fx >= 0.f && fy >= 0.f && fz >= 0.f && fx < (float)grid.dims[0] && fy < (float)grid.dims[1] &&
-          fz < (float)grid.dims[2]))
-      continue;
-    const int64_t r = ((int64_t)fz * grid.dims[1] + (int64_t)fy) * grid.dims[0] + (int64_t)fx;
-    atomicAdd(&sum[r], (double)su[i].w);
-    atomicAdd(&count[r], 1u);
+//
+// Bound at first: FP64 atomics on few addresses (regions are metres wide, so neighbouring
+// Gaussians share one), then FP64 additions themselves (a warp's addition holds the SM's FP64
+// unit for 16 cycles: a shuffle reduction per region and warp step took 42 us).  So every
+// warp keeps a table of the first kRegSlots regions it meets in its stretch of the map, with
+// one FP64 sum per slot and lane in shared memory: one addition per 32 Gaussians, and one
+// reduction and one global atomic per slot at the end.  Lanes whose region finds no slot (a
+// map in random order) add for themselves, and then meet few others on an address.
+// 1M Gaussians, 32 regions: 702 us with one atomic per Gaussian, now 25 us.
+constexpr int kRegSlots = 8;
+
+__global__ void __launch_bounds__(kBlock) k_regions(const float4* __restrict__ mo, const float4* __restrict__ su,
+                                                    int64_t n, gs_region_grid grid, double* __restrict__ sum,
+                                                    uint32_t* __restrict__ count) {
+  __shared__ double s_acc[kWarps][kRegSlots][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k = 0; k < kRegSlots; ++k) s_acc[warp][k][lane] = 0.0;
+  __syncwarp();
+  int tab = -1;        // lane k < n_tab: region of slot k
+  uint32_t cnt = 0;    // ... and its number of Gaussians
+  int n_tab = 0;       // slots in use (warp-uniform)
+  const int64_t n_warps = (int64_t)gridDim.x * kWarps;
+  const int64_t per = ((n + n_warps - 1) / n_warps + 31) / 32 * 32;
+  const int64_t i0 = ((int64_t)blockIdx.x * kWarps + warp) * per;
+  const int64_t i1 = i0 + per < n ? i0 + per : n;
+  float4 m_next = make_float4(0.f, 0.f, 0.f, 0.f);
+  float u_next = 0.f;
+  if (i0 + lane < i1) {
+    m_next = mo[i0 + lane];
+    u_next = su[i0 + lane].w;
   }
+  for (int64_t b = i0; b < i1; b += 32) {
+    const float4 m = m_next;
+    const float uf = u_next;
+    const bool have = b + lane < i1;
+    if (b + 32 + lane < i1) {
+      m_next = mo[b + 32 + lane];
+      u_next = su[b + 32 + lane].w;
+    }
+    int r = -1;
+    if (have) {
+      const float fx = floorf(__fdiv_rn(__fsub_rn(m.x, grid.origin[0]), grid.size));
+      const float fy = floorf(__fdiv_rn(__fsub_rn(m.y, grid.origin[1]), grid.size));
+      const float fz = floorf(__fdiv_rn(__fsub_rn(m.z, grid.origin[2]), grid.size));
+      if (fx >= 0.f && fy >= 0.f && fz >= 0.f && fx < (float)grid.dims[0] && fy < (float)grid.dims[1] &&
+          fz < (float)grid.dims[2])
+        r = (int)(((int64_t)fz * grid.dims[1] + (int64_t)fy) * grid.dims[0] + (int64_t)fx);   // at most 2^30 regions
+    }
+    uint32_t left = __ballot_sync(0xffffffffu, r >= 0);
+    int slot = -1;
+    while (left) {
+      const int rr = __shfl_sync(0xffffffffu, r, __ffs(left) - 1);
+      const uint32_t same = __ballot_sync(0xffffffffu, r == rr);
+      int k = __ffs(__ballot_sync(0xffffffffu, tab == rr)) - 1;
+      if (k < 0) {
+        if (n_tab == kRegSlots) {   // the table is full: its lanes add for themselves
+          left &= ~same;
+          continue;
+        }
+        k = n_tab++;
+        if (lane == k) tab = rr;
+      }
+      if (lane == k) cnt += __popc(same);
+      if (r == rr) slot = k;
+      left &= ~same;
+    }
+    if (slot >= 0) {
+      s_acc[warp][slot][lane] += (double)uf;
+    } else if (r >= 0) {
+      atomicAdd(&sum[r], (double)uf);
+      atomicAdd(&count[r], 1u);
+    }
+  }
+  __syncwarp();
+  for (int k = 0; k < n_tab; ++k) {
+    const int rr = __shfl_sync(0xffffffffu, tab, k);
+    double v = s_acc[warp][k][lane];
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+    if (lane == 0) atomicAdd(&sum[rr], v);
+  }
+  if (lane < n_tab) atomicAdd(&count[tab], cnt);
 }
 
 __global__ void k_region_mean(const double* __restrict__ sum, const uint32_t* __restrict__ count, int64_t n_reg,
@@ -358,7 +553,12 @@ __global__ void k_zero_bytes(uint8_t* p, size_t n) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) p[i] = 0;
 }
 
-int utility_grid() { return 2 * device_sm_count(); }
+// Blocks of the view-utility kernel: four of 256 threads fit an SM (45 KB of shared memory
+// each), within the 1,024 partial slots of the workspace.
+int utility_grid() {
+  const int g = 4 * device_sm_count();
+  return g > 1024 ? 1024 : g;
+}
 
 }  // namespace
 
@@ -382,20 +582,16 @@ cudaError_t launch_uncertainty_thresholds(const float* mo, const float* su, int6
                                           void* ws, cudaStream_t st) {
   Carver c(ws);
   double* part = c.take<double>(1024);
-  unsigned long long* cnt = c.take<unsigned long long>(2);
-  int g = utility_grid();
-  if (g > 1024) g = 1024;
-  k_zero_bytes<<<1, 32, 0, st>>>(reinterpret_cast<uint8_t*>(cnt), sizeof(unsigned long long) * 2);
+  int g = 2 * device_sm_count();
+  if (g > kMomBlocks) g = kMomBlocks;
+  const float4* m = reinterpret_cast<const float4*>(mo);
+  const float4* s = reinterpret_cast<const float4*>(su);
+  k_u_moments<0><<<g, kMomThreads, 0, st>>>(m, s, n, ground_z, part);
   note_launch();
-  k_u_count<<<g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo), n, ground_z, cnt);
+  k_u_moments<1><<<g, kMomThreads, 0, st>>>(m, s, n, ground_z, part);
   note_launch();
-  for (int pass = 0; pass < 2; ++pass) {
-    k_u_moments<<<g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su), n,
-                                      ground_z, stats, pass, part);
-    note_launch();
-    k_u_finish<<<1, 1, 0, st>>>(part, g, cnt, pass, stats);
-    note_launch();
-  }
+  k_u_finish<<<1, 96, 0, st>>>(part, g, stats);
+  note_launch();
   return cudaGetLastError();
 }
 
@@ -410,8 +606,7 @@ cudaError_t launch_view_utility(const float* mo, const float* su, int64_t n, con
   Carver c(ws);
   uint32_t* cnt_part = c.take<uint32_t>(2 * (size_t)1024 * n_views);
   float* sum_part = c.take<float>((size_t)1024 * n_views);
-  int g = utility_grid();
-  if (g > 1024) g = 1024;
+  const int g = utility_grid();
   const bool sum = mode == GS_XI_SUM;
   for (int v0 = 0; v0 < n_views; v0 += kViewChunk) {
     const int nv = n_views - v0 < kViewChunk ? n_views - v0 : kViewChunk;
@@ -425,9 +620,9 @@ cudaError_t launch_view_utility(const float* mo, const float* su, int64_t n, con
                                                   cnt_part, sum_part, n_views);
     note_launch();
   }
-  const int fb = (n_views + 255) / 256;
-  if (sum) k_view_utility_finish<true><<<fb, 256, 0, st>>>(cnt_part, sum_part, g, n_views, prm.lambda, xi, counts);
-  else k_view_utility_finish<false><<<fb, 256, 0, st>>>(cnt_part, sum_part, g, n_views, prm.lambda, xi, counts);
+  const int fb = (n_views + kWarps - 1) / kWarps;
+  if (sum) k_view_utility_finish<true><<<fb, kBlock, 0, st>>>(cnt_part, sum_part, g, n_views, prm.lambda, xi, counts);
+  else k_view_utility_finish<false><<<fb, kBlock, 0, st>>>(cnt_part, sum_part, g, n_views, prm.lambda, xi, counts);
   note_launch();
   return cudaGetLastError();
 }
@@ -450,10 +645,11 @@ cudaError_t launch_regions(const float* mo, const float* su, int64_t n, const gs
   k_zero_bytes<<<(unsigned)(zb < 1 ? 1 : zb), 256, 0, st>>>(reinterpret_cast<uint8_t*>(cnt), sizeof(uint32_t) * nr);
   note_launch();
   if (n > 0) {
-    int64_t g = (n + 255) / 256;
-    if (g > 4096) g = 4096;
-    k_regions<<<(unsigned)g, 256, 0, st>>>(reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su),
-                                            n, grid, sum, cnt);
+    int64_t g = (n + kBlock - 1) / kBlock;
+    const int64_t most = 8 * (int64_t)device_sm_count();
+    if (g > most) g = most;
+    k_regions<<<(unsigned)g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo),
+                                              reinterpret_cast<const float4*>(su), n, grid, sum, cnt);
     note_launch();
   }
   int64_t g2 = (nr + 255) / 256;

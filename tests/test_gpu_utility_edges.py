@@ -1,0 +1,68 @@
+"""Edges of the planner kernels' groups, chunks and windows against the oracle: groups of 32
+Gaussians with a bounding sphere (view utility, collision), chunks of 2,048 Gaussians and
+groups of 8 warps of points (collision), block sums in shared memory up to 2,048 regions,
+maps whose neighbours lie together and maps in random order."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2409_18122_gb300 import gs, scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def _map(n, order, seed=3):
+    g = scenes.config3(seed=seed, n=max(n, 64), n_side=1).gmap
+    if order == "random":
+        g = g.subset(np.random.default_rng(seed).permutation(g.n))
+    return g.subset(np.arange(n))
+
+
+@pytest.mark.parametrize("order", ["patches", "random"])
+@pytest.mark.parametrize("n,dims", [(1, (1, 1, 1)), (33, (4, 4, 2)), (5000, (16, 16, 8)), (5000, (683, 3, 1)),
+                                    (70001, (4, 4, 2))])
+def test_region_sums(n, dims, order):
+    g = _map(n, order)
+    size = 10.0 / dims[0]
+    omega, count = gs.region_uncertainty(gs.GaussianMapTensors.from_numpy(g), (0.0, 0.0, 0.0), size, dims)
+    ref, ref_cnt = O.region_uncertainty(g.mo, g.su[:, 3], (0.0, 0.0, 0.0), size, dims)
+    np.testing.assert_array_equal(count.cpu().numpy(), ref_cnt)
+    # FP64 sums rounded once to FP32
+    np.testing.assert_allclose(omega.cpu().numpy(), ref, rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("n", [1, 31, 33, 4097])
+def test_thresholds_edges(n):
+    g = _map(n, "random")
+    vu = gs.ViewUtility([scenes.yaw_camera(5, 5, 1.5, 0.3, 80, 60, 65.6)])
+    st = vu.thresholds(gs.GaussianMapTensors.from_numpy(g)).cpu().numpy()
+    ref = O.uncertainty_thresholds(g.mo, g.su[:, 3])
+    assert st[4] == ref[4]
+    np.testing.assert_allclose(st[:4], ref[:4], rtol=1e-13, atol=1e-15)
+
+
+@pytest.mark.parametrize("order", ["patches", "random"])
+@pytest.mark.parametrize("n,views", [(1, 1), (33, 31), (3000, 33), (20011, 257)])
+def test_view_counts(n, views, order):
+    g = _map(n, order)
+    if n > 100:   # a mean that is not a number keeps its group from being culled and is never visible
+        g.mo[n // 2, 0] = np.nan
+        g.mo[n // 3, 1] = np.inf
+    rng = np.random.default_rng(views)
+    cams = []
+    for i in range(views):
+        c = scenes.yaw_camera(*rng.uniform([0, 0, 0.5], [10, 10, 2.5]), rng.uniform(0, 6.28), 80 + i % 3, 60, 65.6)
+        if i % 5 == 1:
+            c.R = (c.R * np.float32(1.5)).astype(np.float32)   # not a rotation: the test is defined by its arithmetic
+        if i % 5 == 2:
+            c.cx, c.cy = -20.0, 200.0                          # principal point outside the image
+        cams.append(c)
+    gm = gs.GaussianMapTensors.from_numpy(g)
+    vu = gs.ViewUtility(cams)
+    st = vu.thresholds(gm).cpu().numpy()
+    xi = vu(gm).cpu().numpy()
+    with np.errstate(invalid="ignore"):
+        ref_xi, ref_cnt = O.view_utility(g.mo, g.su[:, 3], cams, thresholds=tuple(float(x) for x in st))
+    np.testing.assert_array_equal(vu.counts.cpu().numpy().astype(np.int64), ref_cnt)
+    np.testing.assert_array_equal(xi, ref_xi.astype(np.float32))
