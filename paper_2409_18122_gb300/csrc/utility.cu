@@ -470,82 +470,241 @@ __global__ void k_traj_sum(const float* __restrict__ xi, int n_traj, int n_state
   }
 }
 
-// Collision check (Sec. IV-B): ordered integer key of a float, so that unsigned
-// minimum = float minimum.
-__device__ __forceinline__ uint32_t fkey(float f) {
-  const uint32_t b = __float_as_uint(f);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float fkey_inv(uint32_t k) {
-  return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
+// Collision check (Sec. IV-B).  Minimum of floats by integer atomics on their bits: among
+// non-negative floats the signed order, among negative ones the reversed unsigned order, and
+// any negative float is below any non-negative one in the signed order.  (Never -0 or NaN.)
+__device__ __forceinline__ void atomic_min_float(float* p, float v) {
+  if (v >= 0.f) atomicMin(reinterpret_cast<int*>(p), __float_as_int(v));
+  else atomicMax(reinterpret_cast<unsigned*>(p), __float_as_uint(v));
 }
 
-constexpr int kColChunk = 4096;   // Gaussians per block of the collision kernel
-constexpr int kColTile = 256;     // Gaussians staged in shared memory at a time
+// gamma of a Gaussian (negative or NaN: takes part in nothing)
+__device__ __forceinline__ float col_gamma(const float4& s, float r_robot, float lambda_g) {
+  return __fadd_rn(r_robot, __fmul_rn(lambda_g, ex32(fmaxf(fmaxf(s.x, s.y), s.z))));   // principal axis
+}
 
-// Per block: a chunk of Gaussians against every test point (one point per thread,
-// the Gaussians broadcast from shared memory).  Each thread keeps its point's
-// smallest margin |p - mu| - gamma (a square root only when the pair can beat it)
-// and whether some Gaussian has |p - mu|^2 < gamma^2 (separately rounded FP32).
+// |p - mu|^2 < gamma^2, and the pair's margin (infinite when it changes nothing)
+__device__ __forceinline__ bool pair_collides(const float4& p, const float4& mu, float gamma, float& margin) {
+  const float dx = __fsub_rn(p.x, mu.x), dy = __fsub_rn(p.y, mu.y), dz = __fsub_rn(p.z, mu.z);
+  const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+  const bool use = gamma >= 0.f;
+  margin = use && d2 < INFINITY ? sqrtf(d2) - gamma : INFINITY;
+  return use && d2 < __fmul_rn(gamma, gamma);
+}
+
+constexpr int kColChunk = 2048;               // Gaussians per block of the collision kernel
+constexpr int kColGroups = kColChunk / 32;    // groups of 32, each with a bounding sphere
+static_assert(kColGroups == 64, "two groups per lane below");
+
+// Each block stages a chunk of Gaussians (mu, gamma) with a sphere (centre, radius + largest
+// gamma) around every 32 of them and one around the chunk.  |p - c| - radius - gamma bounds
+// the margins inside a sphere from below, so Gaussians whose bound is not below the smallest
+// margin known so far (k_collision_seed's, other blocks', this warp's) and that cannot
+// collide are skipped: first the chunk, 256 points at a time, one per thread; then, for the
+// points that are left, one per warp, the 64 groups, two per lane, the nearest evaluated
+// first, one Gaussian per lane.  The results are the minimum margin over all Gaussians and
+// whether some Gaussian has |p - mu|^2 < gamma^2 (separately rounded FP32), whatever the
+// order, because what is skipped can change neither.
+// Bound: the staging (32 B and an exponential per Gaussian) and the latency of the chain of
+// evaluations near the points.  A map in random order has wide spheres and evaluates most
+// groups.  3M Gaussians, 129 points: 453 us with every pair evaluated (one point per thread),
+// 153 us with groups of 32 only, 96 us with first bounds, 64 us with the chunk test (and 7 us for the
+// first bounds).
 __global__ void __launch_bounds__(kBlock) k_collision(const float4* __restrict__ mo, const float4* __restrict__ su,
                                                       int64_t n, const float4* __restrict__ pts, int n_pts,
-                                                      float r_robot, float lambda_g, float ground_z,
-                                                      uint32_t* __restrict__ margin_key, uint32_t* __restrict__ hit) {
-  __shared__ float4 s_g[kColTile];   // (mu, gamma)
+                                                      float r_robot, float lambda_g, float ground_z, float* margin,
+                                                      uint32_t* hit) {
+  __shared__ float4 s_g[kColChunk];        // (mu, gamma); gamma < 0: no Gaussian
+  __shared__ float4 s_c[kColGroups];       // (centre, radius + largest gamma); -inf: empty group
+  __shared__ float4 s_all;                 // the same for the whole chunk
+  __shared__ uint16_t s_pt[kBlock];        // points of the current 256 that the chunk may matter to
+  __shared__ uint32_t s_n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t g0 = (int64_t)blockIdx.x * kColChunk;
-  int64_t g1 = g0 + kColChunk;
-  if (g1 > n) g1 = n;
-  for (int p0 = 0; p0 < n_pts; p0 += kBlock) {
-    const int pi = p0 + threadIdx.x;
-    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (pi < n_pts) p = pts[pi];
-    float best = INFINITY;
-    bool col = false;
-    for (int64_t t0 = g0; t0 < g1; t0 += kColTile) {
-      __syncthreads();
-      const int64_t gi = t0 + threadIdx.x;
-      float4 e = make_float4(0.f, 0.f, 0.f, -1.f);   // gamma < 0: no Gaussian
-      if (gi < g1) {
-        const float4 m = mo[gi];
-        if (m.z >= ground_z) {
-          const float4 s = su[gi];
-          const float r = ex32(fmaxf(fmaxf(s.x, s.y), s.z));   // principal axis
-          e = make_float4(m.x, m.y, m.z, __fadd_rn(r_robot, __fmul_rn(lambda_g, r)));
-        }
-      }
-      s_g[threadIdx.x] = e;
-      __syncthreads();
-      const int cnt = (int)(g1 - t0 < kColTile ? g1 - t0 : kColTile);
-      if (pi < n_pts) {
-        for (int k = 0; k < cnt; ++k) {
-          const float4 g = s_g[k];
-          if (!(g.w >= 0.f)) continue;
-          const float dx = __fsub_rn(p.x, g.x), dy = __fsub_rn(p.y, g.y), dz = __fsub_rn(p.z, g.z);
-          const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
-          col |= d2 < __fmul_rn(g.w, g.w);
-          const float lim = g.w + best;   // a smaller margin needs |p - mu| < gamma + best
-          if (lim > 0.f && d2 < lim * lim) best = fminf(best, sqrtf(d2) - g.w);
-        }
+#pragma unroll 2
+  for (int q = warp; q < kColGroups; q += kWarps) {   // warp-uniform
+    const int64_t gi = g0 + q * 32 + lane;
+    float4 e = make_float4(0.f, 0.f, 0.f, -1.f);
+    if (gi < n) {
+      const float4 m = mo[gi];
+      const float4 s = su[gi];
+      if (m.z >= ground_z) {
+        e = make_float4(m.x, m.y, m.z, col_gamma(s, r_robot, lambda_g));
       }
     }
-    if (pi < n_pts) {
-      if (best < INFINITY) atomicMin(&margin_key[pi], fkey(best));
-      if (col) atomicOr(&hit[pi], 1u);
+    s_g[q * 32 + lane] = e;
+    const bool use = e.w >= 0.f;
+    const uint32_t mask = __ballot_sync(0xffffffffu, use);
+    float cx = use ? e.x : 0.f, cy = use ? e.y : 0.f, cz = use ? e.z : 0.f;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      cx += __shfl_xor_sync(0xffffffffu, cx, d);
+      cy += __shfl_xor_sync(0xffffffffu, cy, d);
+      cz += __shfl_xor_sync(0xffffffffu, cz, d);
+    }
+    const float inv = 1.f / (float)__popc(mask);
+    cx *= inv;
+    cy *= inv;
+    cz *= inv;
+    const float ex = e.x - cx, ey = e.y - cy, ez = e.z - cz;
+    const float reach = use ? (sqrtf(ex * ex + ey * ey + ez * ez) + e.w) * 1.0001f : 0.f;
+    // a NaN or infinite reach (a non-finite mean) makes the bound -inf: the group is evaluated
+    const bool odd = __any_sync(0xffffffffu, !(reach < INFINITY));
+    const float rg = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(reach)));
+    if (lane == 0)
+      s_c[q] = !mask ? make_float4(0.f, 0.f, 0.f, -INFINITY)
+               : odd ? make_float4(0.f, 0.f, 0.f, INFINITY) : make_float4(cx, cy, cz, rg);
+  }
+  __syncthreads();
+  // one sphere around the chunk, from the groups' spheres
+  if (warp == 0) {
+    const float4 a = s_c[lane], b = s_c[lane + 32];
+    const bool ua = a.w != -INFINITY, ub = b.w != -INFINITY;
+    float cx = (ua ? a.x : 0.f) + (ub ? b.x : 0.f), cy = (ua ? a.y : 0.f) + (ub ? b.y : 0.f);
+    float cz = (ua ? a.z : 0.f) + (ub ? b.z : 0.f);
+    const uint32_t k = __popc(__ballot_sync(0xffffffffu, ua)) + __popc(__ballot_sync(0xffffffffu, ub));
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      cx += __shfl_xor_sync(0xffffffffu, cx, d);
+      cy += __shfl_xor_sync(0xffffffffu, cy, d);
+      cz += __shfl_xor_sync(0xffffffffu, cz, d);
+    }
+    const float inv = 1.f / (float)k;
+    cx *= inv;
+    cy *= inv;
+    cz *= inv;
+    auto far = [&](const float4& c) {
+      const float dx = c.x - cx, dy = c.y - cy, dz = c.z - cz;
+      return (sqrtf(dx * dx + dy * dy + dz * dz) + c.w) * 1.0001f;
+    };
+    const float ra = ua ? far(a) : 0.f, rb = ub ? far(b) : 0.f;
+    const bool odd = __any_sync(0xffffffffu, !(ra < INFINITY) || !(rb < INFINITY));
+    const float rg = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(ra, rb))));
+    if (lane == 0)
+      s_all = !k ? make_float4(0.f, 0.f, 0.f, -INFINITY)
+              : odd ? make_float4(0.f, 0.f, 0.f, INFINITY) : make_float4(cx, cy, cz, rg);
+  }
+  __syncthreads();
+  const float4 call = s_all, ca = s_c[lane], cb = s_c[lane + 32];
+  if (call.w == -INFINITY) return;   // no Gaussian takes part
+  for (int p0 = blockIdx.y * kBlock; p0 < n_pts; p0 += gridDim.y * kBlock) {
+    // 256 points at a time, one per thread, against the chunk's sphere
+    __syncthreads();
+    if (threadIdx.x == 0) s_n = 0u;
+    __syncthreads();
+    const int pt = p0 + threadIdx.x;
+    if (pt < n_pts) {
+      const float4 p = pts[pt];
+      const float best = *(volatile float*)(margin + pt);
+      const bool col = *(volatile uint32_t*)(hit + pt) != 0u;
+      const float dx = p.x - call.x, dy = p.y - call.y, dz = p.z - call.z;
+      const float l = sqrtf(dx * dx + dy * dy + dz * dz) * 0.9999f - call.w - 1e-6f;
+      if (!(l >= best) || (!col && !(l > 0.f))) s_pt[atomicAdd(&s_n, 1u)] = (uint16_t)threadIdx.x;
+    }
+    __syncthreads();
+    const int todo = (int)s_n;
+    for (int t = warp; t < todo; t += kWarps) {
+      const int pi = p0 + s_pt[t];
+      const float4 p = pts[pi];
+      const float seed = *(volatile float*)(margin + pi);
+      float best = seed;                                   // warp-uniform
+      bool col = *(volatile uint32_t*)(hit + pi) != 0u;    // warp-uniform
+      const bool seen = col;
+      // lower bound of a group's margins; rounding (a few 2^-24 of the distances) is covered by 1e-4
+      auto bound = [&](const float4& c) {
+        const float dx = p.x - c.x, dy = p.y - c.y, dz = p.z - c.z;
+        return sqrtf(dx * dx + dy * dy + dz * dz) * 0.9999f - c.w - 1e-6f;
+      };
+      float la = bound(ca), lb = bound(cb);
+      bool wa = ca.w != -INFINITY, wb = cb.w != -INFINITY;   // still to be looked at
+      auto evaluate = [&](int q) {
+        const float4 g = s_g[q * 32 + lane];
+        float m;
+        col |= __any_sync(0xffffffffu, pair_collides(p, g, g.w, m)) != 0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) m = fminf(m, __shfl_xor_sync(0xffffffffu, m, d));
+        best = fminf(best, m);
+      };
+      // a group matters unless its margins cannot be below `best` nor any of it collide anew
+      auto matters = [&](float l) { return !(l >= best) || (!col && !(l > 0.f)); };
+      uint32_t na = __ballot_sync(0xffffffffu, wa && matters(la));
+      uint32_t nb = __ballot_sync(0xffffffffu, wb && matters(lb));
+      if (na | nb) {   // the nearest group first
+        const float l = fminf(wa ? la : INFINITY, wb ? lb : INFINITY);
+        const uint32_t key = __float_as_uint(l) ^ (__float_as_uint(l) >> 31 ? 0xFFFFFFFFu : 0x80000000u);
+        const int who = __ffs(__ballot_sync(0xffffffffu, key == __reduce_min_sync(0xffffffffu, key))) - 1;
+        const int q = __shfl_sync(0xffffffffu, wa && !(la > l) ? lane : lane + 32, who);
+        evaluate(q);
+        if (lane == (q & 31)) (q < 32 ? wa : wb) = false;
+        na = __ballot_sync(0xffffffffu, wa && matters(la));
+        nb = __ballot_sync(0xffffffffu, wb && matters(lb));
+      }
+      while (na | nb) {
+        const int q = na ? __ffs(na) - 1 : 31 + __ffs(nb);
+        evaluate(q);
+        if (lane == (q & 31)) (q < 32 ? wa : wb) = false;
+        na = __ballot_sync(0xffffffffu, wa && matters(la));
+        nb = __ballot_sync(0xffffffffu, wb && matters(lb));
+      }
+      if (lane == 0) {
+        if (best < seed) atomic_min_float(margin + pi, best);
+        if (col && !seen) atomicOr(hit + pi, 1u);
+      }
     }
   }
 }
 
-__global__ void k_collision_init(uint32_t* __restrict__ margin_key, uint32_t* __restrict__ hit, int n_pts) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_pts; i += (int64_t)gridDim.x * blockDim.x) {
-    margin_key[i] = fkey(INFINITY);
-    hit[i] = 0u;
-  }
-}
+// First bounds: one block per point over at most kColSamples Gaussians spread over the map
+// (every one of them a true pair, so margin and hit are bounds of the results).  Without
+// them the blocks of the first wave know no margin and evaluate all their groups.
+constexpr int kColSamples = 2048;
+constexpr int kSeedThreads = 512;
 
-__global__ void k_collision_finish(uint32_t* __restrict__ margin, int n_pts) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_pts; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t k = margin[i];
-    reinterpret_cast<float*>(margin)[i] = fkey_inv(k);
+__global__ void __launch_bounds__(kSeedThreads) k_collision_seed(const float4* __restrict__ mo,
+                                                                 const float4* __restrict__ su, int64_t n,
+                                                                 const float4* __restrict__ pts, float r_robot,
+                                                                 float lambda_g, float ground_z,
+                                                                 float* __restrict__ margin,
+                                                                 uint32_t* __restrict__ hit) {
+  constexpr int kPer = kColSamples / kSeedThreads;
+  __shared__ float s_m[kSeedThreads / 32];
+  __shared__ uint32_t s_h[kSeedThreads / 32];
+  const float4 p = pts[blockIdx.x];
+  const int64_t step = (n + kColSamples - 1) / kColSamples;
+  float best = INFINITY;
+  bool col = false;
+  float4 m[kPer], s[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {   // all loads in flight together
+    const int64_t i = (int64_t)(threadIdx.x + k * kSeedThreads) * step;
+    m[k] = i < n ? mo[i] : make_float4(0.f, 0.f, NAN, 0.f);
+    s[k] = i < n ? su[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    float margin_i;
+    const bool c = pair_collides(p, m[k], col_gamma(s[k], r_robot, lambda_g), margin_i);
+    if (m[k].z >= ground_z) {   // (false for the NaN of no Gaussian)
+      col |= c;
+      best = fminf(best, margin_i);
+    }
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, d));
+  const uint32_t any = __any_sync(0xffffffffu, col);
+  if ((threadIdx.x & 31) == 0) {
+    s_m[threadIdx.x >> 5] = best;
+    s_h[threadIdx.x >> 5] = any;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t h = 0;
+    for (int w = 0; w < kSeedThreads / 32; ++w) {
+      best = fminf(best, s_m[w]);
+      h |= s_h[w];
+    }
+    margin[blockIdx.x] = best;
+    hit[blockIdx.x] = h ? 1u : 0u;
   }
 }
 
@@ -680,20 +839,25 @@ cudaError_t launch_trajectory_utility(const float* mo, const float* su, int64_t 
 cudaError_t launch_collision_check(const float* mo, const float* su, int64_t n, const float* pts, int n_pts,
                                    float r_robot, float lambda_g, float ground_z, float* margin_out,
                                    uint32_t* collides_out, cudaStream_t st) {
-  uint32_t* key = reinterpret_cast<uint32_t*>(margin_out);
-  const int ib = (n_pts + 255) / 256;
-  k_collision_init<<<ib < 1 ? 1 : ib, 256, 0, st>>>(key, collides_out, n_pts);
+  if (n_pts <= 0) return cudaSuccess;
+  k_collision_seed<<<(unsigned)n_pts, kSeedThreads, 0, st>>>(
+      reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su), n,
+      reinterpret_cast<const float4*>(pts), r_robot, lambda_g, ground_z, margin_out, collides_out);
   note_launch();
-  if (n > 0 && n_pts > 0) {
-    const int64_t blocks = (n + kColChunk - 1) / kColChunk;
-    k_collision<<<(unsigned)blocks, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo),
-                                                     reinterpret_cast<const float4*>(su), n,
-                                                     reinterpret_cast<const float4*>(pts), n_pts, r_robot, lambda_g,
-                                                     ground_z, key, collides_out);
+  if (n > kColSamples) {   // (a smaller map has been seen whole)
+    // small maps: the points are shared out over several blocks per chunk, so that about three
+    // blocks per SM run (each block stages its chunk again)
+    const int64_t chunks = (n + kColChunk - 1) / kColChunk;
+    const int64_t want = 3 * (int64_t)device_sm_count();
+    int64_t split = (want + chunks - 1) / chunks;
+    const int64_t most = (n_pts + kBlock - 1) / kBlock;
+    if (split > most) split = most;
+    if (split > 65535) split = 65535;
+    k_collision<<<dim3((unsigned)chunks, (unsigned)split), kBlock, 0, st>>>(
+        reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su), n,
+        reinterpret_cast<const float4*>(pts), n_pts, r_robot, lambda_g, ground_z, margin_out, collides_out);
     note_launch();
   }
-  k_collision_finish<<<ib < 1 ? 1 : ib, 256, 0, st>>>(key, n_pts);
-  note_launch();
   return cudaGetLastError();
 }
 

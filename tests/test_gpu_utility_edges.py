@@ -66,3 +66,23 @@ def test_view_counts(n, views, order):
         ref_xi, ref_cnt = O.view_utility(g.mo, g.su[:, 3], cams, thresholds=tuple(float(x) for x in st))
     np.testing.assert_array_equal(vu.counts.cpu().numpy().astype(np.int64), ref_cnt)
     np.testing.assert_array_equal(xi, ref_xi.astype(np.float32))
+
+
+@pytest.mark.parametrize("order", ["patches", "random"])
+@pytest.mark.parametrize("n,points", [(1, 1), (32, 7), (33, 9), (2048, 129), (2049, 33), (20011, 300)])
+def test_collision_edges(n, points, order):
+    g = _map(n, order)
+    if n > 100:
+        g.mo[n // 2, 0] = np.nan
+        g.mo[n // 3, 1] = np.inf
+    rng = np.random.default_rng(n)
+    pts = np.zeros((points, 4), np.float32)
+    pts[:, :3] = rng.uniform([-1, -1, 0.0], [11, 11, 3], (points, 3))
+    gm = gs.GaussianMapTensors.from_numpy(g)
+    for r_robot, lam, gz in ((0.2, 3.0, float("-inf")), (0.0, 0.0, 0.5), (0.05, 1.0, 100.0)):
+        margin, hit = gs.collision_check(gm, torch.from_numpy(pts).cuda(), r_robot, lam, gz)
+        keep = np.isfinite(g.mo[:, :3]).all(1)      # others take part in nothing
+        ref_m, ref_h = O.collision_check(g.mo[keep], g.su[keep], pts, r_robot, lam, gz)
+        np.testing.assert_array_equal(hit.cpu().numpy().astype(bool), ref_h)
+        # |p - mu| - gamma in FP32: a few units in the last place of |p - mu| and gamma
+        np.testing.assert_allclose(margin.cpu().numpy(), ref_m, rtol=1e-5, atol=2e-6)
