@@ -7,11 +7,11 @@
 //   S_i,ch = sum_{j>i} w_j x_j,ch.
 // The kernel replays each tile back to front starting from the saved final
 // transmittance and last index, recovering T_i = T_{i+1} / (1 - alpha_i), so no
-// per-pixel contributor list is stored.  Per-Gaussian screen-space gradients are
-// summed over the 32 pixels of a warp through shared memory (rows of lane values, each
-// summed by one lane) and added with one scalar atomic per nonzero term; a second
-// kernel maps them through the projection per Gaussian (records of one Gaussian
-// are contiguous), without atomics.
+// per-pixel contributor list is stored.  (The four S_i enter only through sum_ch g_ch S_i,ch:
+// one suffix sum is kept.)  Per-Gaussian screen-space gradients are summed over the 32 pixels
+// of a warp through shared memory, sixteen entries at a time, and added with three vector
+// atomics per (warp, entry); a second kernel maps them through the projection per Gaussian
+// (records of one Gaussian are contiguous), without atomics.
 #include "gs_common.cuh"
 #include "gs_internal.h"
 #include "render_common.cuh"
@@ -20,106 +20,136 @@ namespace gs {
 namespace {
 
 constexpr int kBwdWarps = 2;   // warps (work items) per CTA
-// The ten gradient terms of each entry are summed over the warp's 32 pixels through shared
-// memory: every lane writes its terms of up to kRedBatch entries as rows of 32 values, then
-// each lane sums whole rows (eight 16-byte loads) and adds the sum to the record's slot.
-// Three entries make 30 rows, one per lane.  Measured on the 500k-Gaussian mapping step
-// (backward pass): 12-shuffle reduce-scatter per entry 1.145 ms; batches of 2 / 3 / 4 / 8
-// entries 1.11 / 1.06 / 1.18 / 1.36 ms (two passes over the rows, and less occupancy).
-constexpr int kRedBatch = 3;
+// The gradient terms of an entry are sums over the warp's 32 pixels of two per-pixel values
+// times factors that do not depend on the entry or not on the pixel's history: dL/dq times
+// 1, dx, dy, dx^2, dx dy, dy^2 and the blend weight w times the pixel's image gradient.  So a
+// lane stores only dL/dq and w, as two rows of 32 lane values per entry, and when kRedBatch
+// entries are waiting, lanes e and e + 16 form entry e's ten sums, each over 16 pixels (two
+// image rows), add their halves and add them to the record's gradient slots with 16-byte
+// vector reductions.  Per entry and lane that is two shared-memory stores and about nine
+// instructions of the batch's sums (packed two to an FFMA2), where ten stored terms summed
+// row by row took ten stores and about thirty.  Batches of 32 (a lane per entry) would need
+// twice the shared memory.  Four 640x480 keyframes of a 500k-Gaussian map: 836 -> 577 us of this
+// kernel (507 M warp instructions, 71% of cycles issue one); 80 registers (12 CTAs per SM)
+// against 72 with a few spills (14 CTAs): 577 / 601 us; the whole mapping iteration of the 3M
+// map 8.00 -> 6.96 ms.
+constexpr int kRedBatch = 16;
 constexpr int kRedPitch = 36;   // floats per row: 16-byte aligned, conflict-free vector reads
-constexpr int kPix = 1;        // pixels per lane (8x4 blocks: finer culling beats sharing reductions)
 
-__global__ void __launch_bounds__(kBwdWarps * 32, 14) k_render_bwd(gs_map map, gs_proj proj, gs_bins bins,
+__global__ void __launch_bounds__(kBwdWarps * 32, 12) k_render_bwd(gs_map map, gs_proj proj, gs_bins bins,
                                                                 const gs_camera* __restrict__ cams, int n_views,
                                                                 gs_params p, gs_image fwd, gs_image_grad grad,
                                                                 float4* __restrict__ g2d, uint32_t n_items) {
-  __shared__ float4 s_stage[kBwdWarps][3][32];   // (mu), (colour, depth), (scaled conic, o)
-  static_assert(kPix == 1, "the entry body below is written for one pixel per lane");
-  __shared__ uint32_t s_rec[kBwdWarps][32];
-  __shared__ __align__(16) float s_red[kBwdWarps][kRedBatch * 10 * kRedPitch];
-  __shared__ uint32_t s_rrec[kBwdWarps][kRedBatch];
+  // staged entries: (c0, cu, cv, k.x), (k.y, k.z, position in the list, record), (colour, depth)
+  __shared__ float4 s_stage[kBwdWarps][3][32];
+  __shared__ __align__(16) float s_red[kBwdWarps][2][kRedBatch * kRedPitch];   // dL/dq and w rows
+  __shared__ __align__(16) float s_gpix[kBwdWarps][4][32];                     // image gradient (d, r, g, b) per pixel
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
   uint32_t item = blockIdx.x * kBwdWarps + warp;
   if (item >= n_items) return;
   item = ordered_item(bins, proj.view_info, n_views, item);   // longest tile lists first
   TileInfo ti;
-  if (!warp_item_setup<kPix>(proj, bins, cams, n_views, item, ti)) return;
+  if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) return;
   WarpBlock wb;
-  warp_block<kPix>(ti, wb);
-  float4* sx = s_stage[warp][0];
-  float4* sr = s_stage[warp][1];
+  warp_block<1>(ti, wb);
+  float4* sa = s_stage[warp][0];
+  float4* sb = s_stage[warp][1];
   float4* sk = s_stage[warp][2];
-  uint32_t* srec = s_rec[warp];
-  float* red = s_red[warp];
-  uint32_t* rrec = s_rrec[warp];
-  int nb = 0;   // entries waiting in the batch (warp-uniform)
-  // Sums each batched entry's ten terms over the warp (one row of 32 lane values per term,
-  // rows spread over the lanes) and adds them to the record's gradient slots:
-  // (v0, v1, v2, v3), (v4, v5, v6, -), (v7, v8, v9, -).
+  float* rq = s_red[warp][0];
+  float* rw = s_red[warp][1];
+  const float4* SP = reinterpret_cast<const float4*>(proj.splat);
+  const float4* CD = reinterpret_cast<const float4*>(proj.color_d);
+  uint32_t my_rec = 0;   // record of batched entry `lane & 15`
+  int nb = 0;            // entries waiting in the batch (warp-uniform)
+  // Sums the batched entries' terms and adds them to their records' gradient slots:
+  // (P, Q, dL/da, dL/db), (dL/dc, o dL/do, dL/dt_z, -), (dL/dr, dL/dg, dL/db, -).
   auto flush = [&](int count) {
     __syncwarp();
-    for (int r = lane; r < count * 10; r += 32) {
-      const float4* row = reinterpret_cast<const float4*>(red + r * kRedPitch);
-      float4 a = row[0];
+    const int e = lane & (kRedBatch - 1), h = lane >> 4;
+    const float2 mu = __ldg(reinterpret_cast<const float2*>(SP + 2 * (size_t)my_rec));   // (a record read before)
+    // w times the image gradient, two pixels at a time
+    const ulonglong2* W = reinterpret_cast<const ulonglong2*>(rw + e * kRedPitch + 16 * h);
+    const ulonglong2* G = reinterpret_cast<const ulonglong2*>(&s_gpix[warp][0][16 * h]);
+    f32x2 gs[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
-      for (int k = 1; k < 8; ++k) {
-        const float4 c = row[k];
-        a.x += c.x;
-        a.y += c.y;
-        a.z += c.z;
-        a.w += c.w;
+    for (int k = 0; k < 4; ++k) {
+      const ulonglong2 w = W[k];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const ulonglong2 g = G[8 * c + k];
+        gs[c] = fma2(w.y, g.y, fma2(w.x, g.x, gs[c]));
       }
-      const float sum = (a.x + a.y) + (a.z + a.w);
-      const int e = r / 10, j = r - 10 * e;
-      if (sum != 0.f) atomicAdd(reinterpret_cast<float*>(g2d + 3 * (size_t)rrec[e]) + (j < 7 ? j : j + 1), sum);
+    }
+    // dL/dq times (1, dx, dy, dx^2, dx dy, dy^2), dx = mu_x - pixel centre
+    const ulonglong2* D = reinterpret_cast<const ulonglong2*>(rq + e * kRedPitch + 16 * h);
+    const f32x2 mx = pack2(mu.x, mu.x);
+    f32x2 dx[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dx[j] = add2(mx, pack2(-(wb.bx0 + (float)(2 * j)), -(wb.bx0 + (float)(2 * j + 1))));
+    f32x2 a2 = 0ull;
+    float sP = 0.f, sQ = 0.f, sB = 0.f, sC = 0.f, s0 = 0.f;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const ulonglong2 x0 = D[2 * r], x1 = D[2 * r + 1];
+      const f32x2 x[4] = {x0.x, x0.y, x1.x, x1.y};
+      f32x2 o2 = 0ull, p2 = 0ull;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const f32x2 t = mul2(x[j], dx[j]);
+        o2 = add2(o2, x[j]);
+        p2 = add2(p2, t);
+        a2 = fma2(t, dx[j], a2);
+      }
+      const float dy = __fsub_rn(mu.y, wb.by0 + (float)(2 * h + r));
+      const float o = sum2(o2), pr = sum2(p2), q = o * dy;
+      s0 += o;
+      sP += pr;
+      sQ += q;
+      sB = fmaf(pr, dy, sB);
+      sC = fmaf(q, dy, sC);
+    }
+    float v[10] = {sP, sQ, sum2(a2), 2.f * sB, sC, -2.f * s0, sum2(gs[0]), sum2(gs[1]), sum2(gs[2]), sum2(gs[3])};
+#pragma unroll
+    for (int j = 0; j < 10; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 16);
+    if (e < count) {
+      float4* dst = g2d + 3 * (size_t)my_rec;
+      atomicAdd(dst + h, h ? make_float4(v[4], v[5], v[6], 0.f) : make_float4(v[0], v[1], v[2], v[3]));
+      if (h) atomicAdd(dst + 2, make_float4(v[7], v[8], v[9], 0.f));
     }
     __syncwarp();
   };
-  const float pxc = (float)wb.px + 0.5f;
   const float ln_amin = __logf(p.alpha_min);
   const LaneOffsets lo = lane_offsets(lane);
   const float ccx = wb.bx0 + 3.5f, ccy = wb.by0 + 1.5f;   // centre of the 8x4 block
   const size_t P = (size_t)ti.W * ti.H;
-  float pyc[kPix], T[kPix], gr[kPix], gg[kPix], gb[kPix], gd[kPix];
-  float Sr[kPix], Sg[kPix], Sb[kPix], Sd[kPix];
-  bool inside[kPix];
-  int last[kPix];
-#pragma unroll
-  for (int q = 0; q < kPix; ++q) {
-    const int py = wb.py + 4 * q;
-    pyc[q] = (float)py + 0.5f;
-    inside[q] = wb.px < ti.W && py < ti.H;
-    T[q] = 1.f;
-    gr[q] = gg[q] = gb[q] = gd[q] = 0.f;
-    Sr[q] = Sg[q] = Sb[q] = Sd[q] = 0.f;
-    last[q] = 0;
-    if (inside[q]) {
-      const size_t pix = (size_t)py * ti.W + wb.px;
-      const size_t o = (size_t)ti.pix_base + pix;
-      T[q] = fwd.T[o];
-      last[q] = fwd.last[o];
-      if (grad.rgb) {
-        const float* base = grad.rgb + 3 * (size_t)ti.pix_base;
-        gr[q] = base[pix];
-        gg[q] = base[P + pix];
-        gb[q] = base[2 * P + pix];
-      }
-      if (grad.depth) gd[q] = grad.depth[o];
+  float T = 1.f, gr = 0.f, gg = 0.f, gb = 0.f, gd = 0.f;
+  float S = 0.f;   // sum over the entries behind of w_j (image gradient . x_j)
+  int last = 0;    // 0 outside the image
+  if (wb.px < ti.W && wb.py < ti.H) {
+    const size_t pix = (size_t)wb.py * ti.W + wb.px;
+    const size_t o = (size_t)ti.pix_base + pix;
+    T = fwd.T[o];
+    last = fwd.last[o];
+    if (grad.rgb) {
+      const float* base = grad.rgb + 3 * (size_t)ti.pix_base;
+      gr = base[pix];
+      gg = base[P + pix];
+      gb = base[2 * P + pix];
     }
+    if (grad.depth) gd = grad.depth[o];
   }
-  int my_last = 0;
-#pragma unroll
-  for (int q = 0; q < kPix; ++q) my_last = max(my_last, last[q]);
-  const int wlast = (int)__reduce_max_sync(0xffffffffu, (unsigned)my_last);
+  const int wlast = (int)__reduce_max_sync(0xffffffffu, (unsigned)(last > 0 ? last : 0));
   if (wlast == 0) return;
+  s_gpix[warp][0][lane] = gd;
+  s_gpix[warp][1][lane] = gr;
+  s_gpix[warp][2][lane] = gg;
+  s_gpix[warp][3][lane] = gb;
   // groups of 32 entries are walked from the last one any lane used back to the
   // first, with the same four-stage pipeline as the forward kernel (alpha and
   // colour data of the next group, means of the one after, list indices of the
   // one after that)
   const uint32_t* rl = bins.rec + ti.beg;
-  const float4* SP = reinterpret_cast<const float4*>(proj.splat);
-  const float4* CD = reinterpret_cast<const float4*>(proj.color_d);
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
   int g = ((wlast - 1) >> 5) << 5;
   uint32_t rA = 0, rB = 0, rC = 0;
@@ -147,68 +177,40 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 14) k_render_bwd(gs_map map, g
     uint32_t rD = 0;
     if (g >= 96) rD = __ldg(rl + g - 96 + lane);
     ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
-    uint32_t m = __ballot_sync(0xffffffffu, ovA);
+    const uint32_t m = __ballot_sync(0xffffffffu, ovA);
     if (m) {
+      // the overlapping entries, compacted in list order
       if (ovA) {
+        const int s = __popc(m & lt);
         const Exponent e = stage_exponent(mA.x, mA.y, cA, ccx, ccy);
-        sx[lane] = make_float4(mA.x, mA.y, e.cu, e.cv);
-        sr[lane] = kA;
-        sk[lane] = make_float4(e.kx, e.ky, e.kz, e.c0);
-        srec[lane] = rA;
+        sa[s] = make_float4(e.c0, e.cu, e.cv, e.kx);
+        sb[s] = make_float4(e.ky, e.kz, __int_as_float(g + lane), __uint_as_float(rA));
+        sk[s] = kA;
       }
       __syncwarp();
-      while (m) {
-        const int b = 31 - __clz(m);
-        m ^= 1u << b;
-        const int pos = g + b;   // position in the tile's list
-        const float4 mu = sx[b];
-        const float4 ks = sk[b];
-        // the alpha of the forward pass (same staged coefficients, same operations); ar = o G
-        float dx = 0.f, dy = 0.f, ar = 0.f, al = 0.f;
-        const bool live = inside[0] && pos < last[0];
-        if (live) {
-          ar = alpha_raw(ks.w, mu.z, mu.w, ks.x, ks.y, ks.z, lo);
-          al = fminf(p.alpha_max, ar);
-          dx = __fsub_rn(mu.x, pxc);
-          dy = __fsub_rn(mu.y, pyc[0]);
-        }
-        const bool contrib = live && !(al < p.alpha_min);
+      for (int i = __popc(m) - 1; i >= 0; --i) {
+        const float4 ea = sa[i], eb = sb[i];
+        // the alpha of the forward pass (same staged coefficients, same operations); ar = o G.
+        // A lane that does not contribute runs the same arithmetic with alpha = 0: its T and
+        // suffix sum stay exactly unchanged (T * 1, S + 0) and its terms are zero.
+        const float ar = alpha_raw(ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, lo);
+        float al = fminf(p.alpha_max, ar);
+        const bool contrib = __float_as_int(eb.z) < last && !(al < p.alpha_min);
         if (!__any_sync(0xffffffffu, contrib)) continue;
-        // A lane that does not contribute runs the same arithmetic with alpha = ar = dx = dy = 0:
-        // its T and suffix sums stay exactly unchanged (T * 1, S + 0) and every term is zero.
-        if (!contrib) al = ar = dx = dy = 0.f;
-        const float4 c = sr[b];
+        if (!contrib) al = 0.f;
+        const float4 c = sk[i];
         const float inv = __fdividef(1.f, 1.f - al);   // 1 - alpha in [1 - alpha_max, 1]: approximate reciprocal
-        const float Ti = T[0] * inv;
-        const float w = al * Ti;
-        const float dalpha = (gr[0] * c.x + gg[0] * c.y + gb[0] * c.z + gd[0] * c.w) * Ti -
-                             (gr[0] * Sr[0] + gg[0] * Sg[0] + gb[0] * Sb[0] + gd[0] * Sd[0]) * inv;
-        Sr[0] += w * c.x;
-        Sg[0] += w * c.y;
-        Sb[0] += w * c.z;
-        Sd[0] += w * c.w;
-        T[0] = Ti;
-        const bool free = ar < p.alpha_max;   // alpha not clamped
-        const float dq = free ? -0.5f * al * dalpha : 0.f;    // dL/dq
-        // dL/dmu_2D = 2 (a P + b Q, b P + c Q) with P = sum dq dx, Q = sum dq dy (dx = mu_x - p_x):
-        // the conic is the record's, so P and Q are summed and k_proj_adjoint applies it
-        float v[10];
-        v[0] = dq * dx;              // P
-        v[1] = dq * dy;              // Q
-        v[2] = v[0] * dx;            // dL/da
-        v[3] = 2.f * v[0] * dy;      // dL/db
-        v[4] = v[1] * dy;            // dL/dc
-        v[5] = free ? dalpha * ar : 0.f;          // o dL/do (k_proj_adjoint divides by o)
-        v[6] = gd[0] * w;
-        v[7] = gr[0] * w;
-        v[8] = gg[0] * w;
-        v[9] = gb[0] * w;
-        // this lane's terms join the batch; a full batch is summed and added
-#pragma unroll
-        for (int j = 0; j < 10; ++j) red[(nb * 10 + j) * kRedPitch + lane] = v[j];
-        if (lane == 0) rrec[nb] = srec[b];
+        T *= inv;
+        const float w = al * T;
+        const float gc = gr * c.x + gg * c.y + gb * c.z + gd * c.w;   // image gradient . x_i
+        const float dalpha = gc * T - S * inv;
+        S += w * gc;
+        // dL/dq = -alpha/2 dL/dalpha where alpha is not clamped (there o dL/do = -2 dL/dq)
+        rq[nb * kRedPitch + lane] = ar < p.alpha_max ? -0.5f * al * dalpha : 0.f;
+        rw[nb * kRedPitch + lane] = w;
+        if ((lane & (kRedBatch - 1)) == nb) my_rec = __float_as_uint(eb.w);
         if (++nb == kRedBatch) {
-          flush(nb);
+          flush(kRedBatch);
           nb = 0;
         }
       }
@@ -378,7 +380,7 @@ cudaError_t launch_render_bwd(const gs_map& map, const gs_proj& proj, const gs_b
   if (zb < 1) zb = 1;
   k_zero_g2d<<<(unsigned)zb, 256, 0, st>>>(g2d, proj.count, proj.capacity);
   note_launch();
-  const int64_t items = bins.tile_capacity * (32 / kPix);   // upper bound: at most 32 / kPix items per tile
+  const int64_t items = bins.tile_capacity * 32;   // upper bound: at most 32 items per tile
   if (items > 0) {
     k_render_bwd<<<(unsigned)((items + kBwdWarps - 1) / kBwdWarps), kBwdWarps * 32, 0, st>>>(
         map, proj, bins, cams, n_views, p, fwd, g, g2d, (uint32_t)items);

@@ -83,6 +83,40 @@ __device__ __forceinline__ float alpha_raw(float c0, float cu, float cv, float k
   return ex2_approx(__fmaf_rn(kz, lo.vv, __fmaf_rn(ky, lo.uv, __fmaf_rn(kx, lo.uu, __fmaf_rn(cv, lo.v, __fmaf_rn(cu, lo.u, c0))))));
 }
 
+// Two FP32 values in a 64-bit register and the packed operations on them (one issue slot for
+// two operations; each half rounds like the scalar operation).
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(f32x2 a) {
+  float2 d;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(d.x), "=f"(d.y) : "l"(a));
+  return d;
+}
+__device__ __forceinline__ float sum2(f32x2 a) {
+  const float2 v = unpack2(a);
+  return v.x + v.y;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+
 // Work item of the compositing kernels: one warp renders one 8 x (4 KP) pixel
 // block of one screen tile, KP pixels per lane (KP = 1 in every kernel: a larger
 // block per warp culls less finely, which costs more than it saves).  Block b of a tile covers columns
