@@ -113,7 +113,7 @@ typedef struct {
  *   ig_batch        chunk depth of the information-gain compositing: how many of a warp's
  *                   staged list entries have their alphas evaluated together before the
  *                   transmittance updates run through them in list order; 4, 8 or 16 (0: 8)
- *   fwd_batch       the same for gs_render_fwd: 1, 2 or 4 (0: 2)
+ *   fwd_batch       the same for gs_render_fwd: 1, 2 or 4 (0: 4; 1 runs as 2)
  * The outputs are bit for bit the same for every ig_batch and fwd_batch.
  * Defaults: 16, 16, 0.3, 0.2, 1.3, 1/255, 0.99, 1e-4, 0, 0. */
 typedef struct {

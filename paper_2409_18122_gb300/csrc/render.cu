@@ -6,11 +6,10 @@
 // same way gives the rendered information channel, whose per-view mean scores a
 // candidate view (Eq. (nbv) with the Jacobian replaced by the blend weights).
 //
-// One thread block per screen tile (tile_w x tile_h threads, one pixel each).
-// The tile's depth-sorted list is walked in chunks of blockDim entries staged
-// in shared memory; each thread leaves the inner loop as soon as its pixel is
-// saturated, so a warp stops issuing once all its lanes are done, and the
-// block stops loading chunks once every pixel is done (__syncthreads_count).
+// One warp per 8x4-pixel block of a screen tile, one pixel per lane.  The tile's depth-sorted
+// list is walked in groups of 32 entries; those that reach a live pixel of the block are staged
+// in a shared-memory ring and composited in whole chunks, so no warp waits for another and each
+// leaves its list as soon as all of its pixels are saturated.
 #include "gs_common.cuh"
 #include "gs_internal.h"
 #include "render_common.cuh"
@@ -19,56 +18,82 @@ namespace gs {
 namespace {
 
 constexpr int kFwdWarps = 2;   // warps (work items) per CTA: small CTAs free their slot as soon as both finish
-constexpr int kIgWarps = 8;    // warps per CTA of the persistent information-gain kernel
-constexpr int kIgRing = 64;    // staged entries per warp of the information-gain kernel (a ring)
+constexpr int kIgWarps = 2;    // the same for the persistent information-gain kernel
+constexpr int kRing = 64;      // staged entries per warp (a ring): a group of 32 and a partial chunk
 constexpr int kPix = 1;        // pixels per lane of the forward and information-gain kernels
-// Chunk depth: overlapping entries whose alphas are computed together, a template argument
-// of both compositing kernels chosen per launch by gs_params (forward 1, 2 or 4, default 2;
-// information gain 4, 8 or 16, default 8)
-constexpr int kFwdBatchDefault = 2;
+// Chunk depth: staged entries whose alphas are computed together, a template argument of both
+// compositing kernels chosen per launch by gs_params (forward 1, 2 or 4, default 4; 1 runs as 2,
+// the pair of one packed evaluation; information gain 4, 8 or 16, default 8)
+constexpr int kFwdBatchDefault = 4;
 constexpr int kIgBatchDefault = 8;
 
 // The list walk of all compositing kernels is a four-stage software pipeline
 // over groups of 32 entries (one per lane).  While group g is composited, the
 // alpha/colour data of group g+32 is fetched -- only for entries whose support
-// box touches the warp's pixel block, decided from their means fetched one
+// box touches the live pixels of the warp's block, decided from their means fetched one
 // iteration earlier -- the means of group g+64 are fetched, and the list
 // indices of group g+96.  Every fetch is issued one iteration before it is
 // used and none depends on a value loaded in the same iteration.
+//
+// Both kernels are bound by instruction issue where a batch fills the chip (about 0.75 of the
+// cycles issue one) and by the chain of transmittance updates of one long list where it does
+// not, so both are short per entry:
+//  - the exponents of two entries are evaluated by one packed fused multiply-add each
+//    (alpha_raw2), from a layout staged for it;
+//  - whole chunks leave the ring and a partial one waits for the next group, so only a list's
+//    last chunk is padded;
+//  - T runs through a chunk as if nothing stopped in it (one multiply and one subtraction per
+//    entry); the stop rule is a predicate beside that chain, and the sums follow it;
+//  - entries are culled against the bounding box of the pixels still live.
+// Measured against one entry per evaluation, a stop test inside the chain and (forward) a chunk
+// of 2 without the ring: forward 354 -> 307 us (500k Gaussians, four 640x480 views), 1551 ->
+// 1338 us (3M, eight 1280x720), 45 -> 28 us (20k, two 321x243: bound by its longest list);
+// information gain 3.07 -> 2.63 ms (1M, 256 views), 517 -> 428 us (200k, 27 views), 6.83 -> 6.22
+// ms (3M, 384 views).  Registers are held to 24 warps per SM in both: without the bound the
+// information gain takes 105 registers, 16 warps, and 3.10 ms.
 
-template <int kFwdBatch>
+// Narrows the block's cull box to the bounding box of its live pixels (lane l holds pixel
+// (l mod 8, l div 8); lm = ballot of the live lanes, not zero; (x0, y0) = the centre of the
+// block's first pixel): an entry that reaches only saturated pixels adds nothing.
+__device__ __forceinline__ void live_box(uint32_t lm, float x0, float y0, WarpBlock& wb) {
+  const uint32_t cols = (lm | (lm >> 8) | (lm >> 16) | (lm >> 24)) & 0xFFu;
+  const uint32_t rows = ((lm & 0xFFu) ? 1u : 0u) | ((lm & 0xFF00u) ? 2u : 0u) | ((lm & 0xFF0000u) ? 4u : 0u) |
+                        ((lm & 0xFF000000u) ? 8u : 0u);
+  wb.bx0 = x0 + (float)(__ffs(cols) - 1);
+  wb.bx1 = x0 + (float)(31 - __clz(cols));
+  wb.by0 = y0 + (float)(__ffs(rows) - 1);
+  wb.by1 = y0 + (float)(31 - __clz(rows));
+}
+
+// kPairs: packed pairs per chunk.  kCount: the per-pixel counts are asked for (n_contrib).
+template <int kPairs, bool kCount>
 __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, gs_proj proj, gs_bins bins,
                                                                 const gs_camera* __restrict__ cams, int n_views,
                                                                 gs_params p, gs_image img, uint32_t n_items) {
-  // staged entries: (c0, cu, cv, u), (k.x, k.y, k.z, lane), (r, g, b, depth) (stage_exponent)
-  __shared__ float4 s_stage[kFwdWarps][3][32];
+  constexpr int kChunk = 2 * kPairs;
+  __shared__ __align__(16) float s_exp[kFwdWarps][kRing / 2 * kPairFloats];   // staged exponents (stage_pair)
+  __shared__ float4 s_col[kFwdWarps][kRing];                                  // (r, g, b, depth)
+  __shared__ float2 s_up[kFwdWarps][kRing];                                   // (u, position in the list + 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
   uint32_t item = blockIdx.x * kFwdWarps + warp;
   if (item >= n_items) return;
-  static_assert(kPix == 1, "the binning's item order numbers 32-pixel blocks");
   item = ordered_item(bins, proj.view_info, n_views, item);
   TileInfo ti;
-  if (!warp_item_setup<kPix>(proj, bins, cams, n_views, item, ti)) return;
+  if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) return;
   WarpBlock wb;
-  warp_block<kPix>(ti, wb);
-  float4* sm = s_stage[warp][0];
-  float4* sc = s_stage[warp][1];
-  float4* sk = s_stage[warp][2];
+  warp_block<1>(ti, wb);
+  float* sx = s_exp[warp];
+  float4* sk = s_col[warp];
+  float2* su = s_up[warp];
   const float ln_amin = __logf(p.alpha_min);
-  const LaneOffsets lo = lane_offsets(lane);
+  const LaneOffsets2 lo = lane_offsets2(lane);
   const float ccx = wb.bx0 + 3.5f, ccy = wb.by0 + 1.5f;   // centre of the 8x4 block
-  bool inside[kPix], done[kPix];
-  float T[kPix], cr[kPix], cg[kPix], cb[kPix], cd[kPix], cu[kPix];
-  int32_t last[kPix], n_contrib[kPix];
-#pragma unroll
-  for (int q = 0; q < kPix; ++q) {
-    inside[q] = wb.px < ti.W && wb.py + 4 * q < ti.H;
-    done[q] = !inside[q];
-    T[q] = 1.f;
-    cr[q] = cg[q] = cb[q] = cd[q] = cu[q] = 0.f;
-    last[q] = n_contrib[q] = 0;
-  }
+  const bool inside = wb.px < ti.W && wb.py < ti.H;
+  bool alive = inside;
+  float T = 1.f, cu = 0.f;
+  f32x2 rg = 0ull, bd = 0ull;
+  int32_t last = 0, n_contrib = 0;
   const uint32_t n = ti.end - ti.beg;
   const uint32_t* rl = bins.rec + ti.beg;
   const float4* SP = reinterpret_cast<const float4*>(proj.splat);
@@ -87,8 +112,49 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
     cA = __ldg(SP + 2 * (size_t)rA + 1);
     kA = __ldg(CD + rA);
   }
+  // Composites the chunk at ring position i0, of which the first `valid` entries exist: the alphas
+  // are independent and computed together, the transmittance updates run in list order.
+  auto chunk = [&](int i0, int valid) {
+    float al[kChunk];
+#pragma unroll
+    for (int k = 0; k < kPairs; ++k) {
+      const float2 a = alpha_raw2(sx, (i0 >> 1) + k, lo);
+      al[2 * k] = fminf(p.alpha_max, a.x);
+      al[2 * k + 1] = fminf(p.alpha_max, a.y);
+    }
+    float w[kChunk];
+    bool add[kChunk];
+    float Tc = T;   // transmittance as if no entry of the chunk stopped the pixel
+#pragma unroll
+    for (int k = 0; k < kChunk; ++k) {
+      const bool hit = !(al[k] < p.alpha_min);
+      w[k] = (hit ? al[k] : 0.f) * Tc;
+      Tc = Tc - w[k];              // T (1 - alpha)
+      alive = alive && !(Tc < p.T_min);
+      add[k] = hit && alive && k < valid;
+      if (alive) T = Tc;
+    }
+#pragma unroll
+    for (int k = 0; k < kChunk; ++k) {
+      const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(sk + i0 + k);
+      const float2 e = su[i0 + k];
+      if (add[k]) {
+        const f32x2 w2 = pack2(w[k], w[k]);
+        rg = fma2(w2, c.x, rg);
+        bd = fma2(w2, c.y, bd);
+        cu += w[k] * e.x;
+        last = __float_as_int(e.y);
+        if (kCount) ++n_contrib;
+      }
+    }
+  };
+  uint32_t head = 0, tail = 0;   // ring entries [head, tail) are staged and not yet composited
+  uint32_t lm_prev = 0;
   for (uint32_t g = 0; g < n; g += 32) {
-    if (!__any_sync(0xffffffffu, !all_done<kPix>(done))) break;
+    const uint32_t lm = __ballot_sync(0xffffffffu, alive);
+    if (!lm) break;
+    if (lm != lm_prev) live_box(lm, ccx - 3.5f, ccy - 1.5f, wb);
+    lm_prev = lm;
     const bool ovB = g + 32 + lane < n && box_overlaps(mB, wb);
     float4 cB = z4, kB = z4;
     if (ovB) {
@@ -102,121 +168,88 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
     ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
     const uint32_t m = __ballot_sync(0xffffffffu, ovA);
     if (m) {
-      // the overlapping entries, compacted in list order: (c0, cu, cv, u), (k, position in
-      // the group), colour; padded to whole batches with entries of c0 = -inf (alpha = 0:
-      // always skipped)
-      const int n_ov = __popc(m);
-      const int n_pad = (n_ov + kFwdBatch - 1) / kFwdBatch * kFwdBatch;
+      // the overlapping entries join the ring in list order; whole chunks are composited at once
+      // and a partial chunk waits for the next group's entries
       if (ovA) {
-        const int s = __popc(m & lt);
-        const Exponent e = stage_exponent(mA.x, mA.y, cA, ccx, ccy);
-        sm[s] = make_float4(e.c0, e.cu, e.cv, mA.w);
-        sc[s] = make_float4(e.kx, e.ky, e.kz, __int_as_float(lane));
+        const uint32_t s = (tail + __popc(m & lt)) & (kRing - 1);
+        stage_pair(sx, s, stage_exponent(mA.x, mA.y, cA, ccx, ccy));
         sk[s] = kA;
+        su[s] = make_float2(mA.w, __int_as_float((int)(g + lane + 1)));
       }
-      if (lane >= n_ov && lane < n_pad) {   // slots [n_ov, n_pad): disjoint from the staged ones
-        sm[lane] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-        sc[lane] = z4;
-      }
+      tail += __popc(m);
       __syncwarp();
-      // kFwdBatch entries at a time: their alphas are independent and computed
-      // together; the transmittance updates then run in list order
-      for (int i0 = 0; i0 < n_ov && !all_done<kPix>(done); i0 += kFwdBatch) {
-        float al[kFwdBatch][kPix];
-#pragma unroll
-        for (int k = 0; k < kFwdBatch; ++k) {
-          const int i = i0 + k;
-          const float4 e0 = sm[i];
-          const float4 e1 = sc[i];
-#pragma unroll
-          for (int q = 0; q < kPix; ++q)
-            al[k][q] = fminf(p.alpha_max, alpha_raw(e0.x, e0.y, e0.z, e1.x, e1.y, e1.z, lo));
-        }
-#pragma unroll
-        for (int k = 0; k < kFwdBatch; ++k) {
-          const int i = i0 + k;
-#pragma unroll
-          for (int q = 0; q < kPix; ++q) {
-            if (done[q]) continue;
-            const float alpha = al[k][q];
-            if (alpha < p.alpha_min) continue;
-            const float w = alpha * T[q];
-            const float Tn = T[q] - w;      // T (1 - alpha)
-            if (Tn < p.T_min) { done[q] = true; continue; }
-            const float4 c = sk[i];
-            cr[q] += w * c.x;
-            cg[q] += w * c.y;
-            cb[q] += w * c.z;
-            cd[q] += w * c.w;
-            cu[q] += w * sm[i].w;
-            T[q] = Tn;
-            last[q] = (int32_t)(g + __float_as_int(sc[i].w) + 1);
-            ++n_contrib[q];
-          }
-        }
+      const uint32_t end = head + (tail - head) / kChunk * kChunk;
+      for (uint32_t h = head; h != end && alive; h += kChunk) {
+        chunk((int)(h & (kRing - 1)), kChunk);
       }
+      head = end;
       __syncwarp();
     }
     mA = mB; ovA = ovB; cA = cB; kA = kB;
     rB = rC; mB = mC;
     rC = rD;
   }
-  const size_t P = (size_t)ti.W * ti.H;
-#pragma unroll
-  for (int q = 0; q < kPix; ++q) {
-    if (!inside[q]) continue;
-    const size_t pix = (size_t)(wb.py + 4 * q) * ti.W + wb.px;
-    const size_t o = (size_t)ti.pix_base + pix;
-    if (img.rgb) {
-      float* base = img.rgb + 3 * (size_t)ti.pix_base;
-      base[pix] = cr[q];
-      base[P + pix] = cg[q];
-      base[2 * P + pix] = cb[q];
-    }
-    if (img.depth) img.depth[o] = cd[q];
-    if (img.unc) img.unc[o] = cu[q];
-    if (img.T) img.T[o] = T[q];
-    if (img.last) img.last[o] = last[q];
-    if (img.n_contrib) img.n_contrib[o] = n_contrib[q];
+  // the last partial chunk, padded with entries of c0 = -inf (alpha = 0)
+  if (tail != head && __any_sync(0xffffffffu, alive)) {
+    const int i0 = (int)(head & (kRing - 1));
+    if ((uint32_t)lane >= tail - head && lane < kChunk)
+      stage_pair(sx, i0 + lane, Exponent{-INFINITY, 0.f, 0.f, 0.f, 0.f, 0.f});
+    __syncwarp();
+    if (alive) chunk(i0, (int)(tail - head));
   }
-}
-
-// Staged form of an entry for the information-gain kernel: s0 = (c0, cu, cv, u),
-// s1 = (k.x, k.y, k.z, 0) (stage_exponent).
-__device__ __forceinline__ void ig_stage(const float4& m, const float4& co, float ccx, float ccy, float4& s0,
-                                         float4& s1) {
-  const Exponent e = stage_exponent(m.x, m.y, co, ccx, ccy);
-  s0 = make_float4(e.c0, e.cu, e.cv, m.w);
-  s1 = make_float4(e.kx, e.ky, e.kz, 0.f);
+  if (!inside) return;
+  const float2 vrg = unpack2(rg), vbd = unpack2(bd);
+  const size_t P = (size_t)ti.W * ti.H;
+  const size_t pix = (size_t)wb.py * ti.W + wb.px;
+  const size_t o = (size_t)ti.pix_base + pix;
+  if (img.rgb) {
+    float* base = img.rgb + 3 * (size_t)ti.pix_base;
+    base[pix] = vrg.x;
+    base[P + pix] = vrg.y;
+    base[2 * P + pix] = vbd.x;
+  }
+  if (img.depth) img.depth[o] = vbd.y;
+  if (img.unc) img.unc[o] = cu;
+  if (img.T) img.T[o] = T;
+  if (img.last) img.last[o] = last;
+  if (kCount) img.n_contrib[o] = n_contrib;
 }
 
 // Composites `chunks` whole chunks of kIgBatch staged entries, starting at ring position
 // `head` (a multiple of kIgBatch, so no chunk wraps): the alphas of a chunk are independent
-// and computed together, the transmittance updates then run in list order.  A lane leaves
-// as soon as its pixel is saturated.
+// and computed together, two to an instruction; the transmittance updates then run in list
+// order.  A lane leaves as soon as its pixel is saturated.
 template <int kIgBatch>
-__device__ __forceinline__ void composite_chunks(const float4* sm, const float4* sc, uint32_t head, uint32_t chunks,
-                                                 const LaneOffsets& lo, const gs_params& p, float& T, float& cu) {
+__device__ __forceinline__ void composite_chunks(const float* sx, const float* su, uint32_t head, uint32_t chunks,
+                                                 const LaneOffsets2& lo, const gs_params& p, float& T, float& cu) {
   for (uint32_t c = 0; c < chunks && T != 0.f; ++c) {
-    const uint32_t b0 = (head + c * kIgBatch) & (kIgRing - 1);
+    const uint32_t b0 = (head + c * kIgBatch) & (kRing - 1);
     float al[kIgBatch], uu[kIgBatch];
 #pragma unroll
-    for (int k = 0; k < kIgBatch; ++k) {
-      const float4 e0 = sm[b0 + k];
-      const float4 e1 = sc[b0 + k];
-      uu[k] = e0.w;
-      al[k] = fminf(p.alpha_max, alpha_raw(e0.x, e0.y, e0.z, e1.x, e1.y, e1.z, lo));
+    for (int k = 0; k < kIgBatch; k += 2) {
+      const float2 a = alpha_raw2(sx, (b0 + k) >> 1, lo);
+      al[k] = fminf(p.alpha_max, a.x);
+      al[k + 1] = fminf(p.alpha_max, a.y);
     }
 #pragma unroll
-    for (int k = 0; k < kIgBatch; ++k) {
-      const float alpha = al[k];
-      if (alpha < p.alpha_min) continue;
-      const float w = T * alpha;   // T (1 - alpha) taken as T - w: one instruction less
-      const float Tn = T - w;
-      if (Tn < p.T_min) { T = 0.f; continue; }
-      cu += w * uu[k];
-      T = Tn;
+    for (int k = 0; k < kIgBatch; k += 4) {
+      const float4 u = *reinterpret_cast<const float4*>(su + b0 + k);
+      uu[k] = u.x;
+      uu[k + 1] = u.y;
+      uu[k + 2] = u.z;
+      uu[k + 3] = u.w;
     }
+    bool alive = true;
+    float Tc = T;   // transmittance as if no entry of the chunk stopped the pixel
+#pragma unroll
+    for (int k = 0; k < kIgBatch; ++k) {
+      const bool hit = !(al[k] < p.alpha_min);
+      const float w = Tc * (hit ? al[k] : 0.f);
+      Tc = Tc - w;   // T (1 - alpha) taken as T - w: one instruction less
+      alive = alive && !(Tc < p.T_min);
+      if (hit && alive) cu += w * uu[k];
+    }
+    T = alive ? Tc : 0.f;
   }
 }
 
@@ -225,18 +258,19 @@ __device__ __forceinline__ void composite_chunks(const float4* sm, const float4*
 // and writes the sum of U over its pixels to the item's own slot (fixed shuffle
 // tree), never accumulating, so the result does not depend on scheduling.
 template <int kIgBatch>
-__global__ void __launch_bounds__(kIgWarps * 32) k_ig_items(gs_proj proj, gs_bins bins,
+__global__ void __launch_bounds__(kIgWarps * 32, 12) k_ig_items(gs_proj proj, gs_bins bins,
                                                              const gs_camera* __restrict__ cams, int n_views,
                                                              gs_params p, const uint32_t* __restrict__ order,
                                                              float* __restrict__ item_sum, int64_t item_cap,
                                                              uint32_t* __restrict__ work) {
-  // staged entries of each warp, a ring of kIgRing: (C0, Cu, Cv, u), (k.x, k.y, k.z, 0) (ig_stage)
-  __shared__ float4 s_stage[kIgWarps][2][kIgRing];
-  static_assert(kIgRing % kIgBatch == 0 && kIgRing >= 32 + kIgBatch, "ring holds a group plus a partial chunk");
+  // staged entries of each warp, a ring of kRing: exponents (stage_pair) and u
+  __shared__ __align__(16) float s_exp[kIgWarps][kRing / 2 * kPairFloats];
+  __shared__ __align__(16) float s_u[kIgWarps][kRing];
+  static_assert(kRing % kIgBatch == 0 && kRing >= 32 + kIgBatch, "ring holds a group plus a partial chunk");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  float4* sm = s_stage[warp][0];
-  float4* sc = s_stage[warp][1];
+  float* sx = s_exp[warp];
+  float* su = s_u[warp];
   uint32_t n_items = proj.view_info[kVI * n_views + 2] / kPix;
   if ((int64_t)n_items > item_cap) n_items = (uint32_t)item_cap;
   const float4* SP = reinterpret_cast<const float4*>(proj.splat);
@@ -259,7 +293,7 @@ __global__ void __launch_bounds__(kIgWarps * 32) k_ig_items(gs_proj proj, gs_bin
     const float ln_amin = __logf(p.alpha_min);
     const float bx_full = wb.bx0, by_full = wb.by0;   // centre of the block's first pixel
     const float ccx = bx_full + 3.5f, ccy = by_full + 1.5f;   // centre of the 8x4 block
-    const LaneOffsets lo = lane_offsets(lane);
+    const LaneOffsets2 lo = lane_offsets2(lane);
     // T = 0 marks a saturated pixel (and one outside the image): the stop rule sets it,
     // and a zero T adds nothing and stays zero, so no separate flag is kept
     float T = (wb.px < ti.W && wb.py < ti.H) ? 1.f : 0.f, cu = 0.f;
@@ -275,21 +309,13 @@ __global__ void __launch_bounds__(kIgWarps * 32) k_ig_items(gs_proj proj, gs_bin
     bool ovA = (uint32_t)lane < n && box_overlaps(mA, wb);
     float4 cA = z4;
     if (ovA) cA = __ldg(SP + 2 * (size_t)rA + 1);
+    uint32_t lm_prev = 0;
     uint32_t head = 0, tail = 0;   // ring entries [head, tail) are staged and not yet composited
     for (uint32_t g = 0; g < n; g += 32) {
       const uint32_t lm = __ballot_sync(0xffffffffu, T != 0.f);
       if (!lm) break;
-      // the culls below test the bounding box of the block's live pixels (lane l holds pixel
-      // (l mod 8, l div 8)): an entry that reaches only saturated pixels adds nothing
-      {
-        const uint32_t cols = (lm | (lm >> 8) | (lm >> 16) | (lm >> 24)) & 0xFFu;
-        const uint32_t rows = ((lm & 0xFFu) ? 1u : 0u) | ((lm & 0xFF00u) ? 2u : 0u) |
-                              ((lm & 0xFF0000u) ? 4u : 0u) | ((lm & 0xFF000000u) ? 8u : 0u);
-        wb.bx0 = bx_full + (float)(__ffs(cols) - 1);
-        wb.bx1 = bx_full + (float)(31 - __clz(cols));
-        wb.by0 = by_full + (float)(__ffs(rows) - 1);
-        wb.by1 = by_full + (float)(31 - __clz(rows));
-      }
+      if (lm != lm_prev) live_box(lm, bx_full, by_full, wb);
+      lm_prev = lm;
       const bool ovB = g + 32 + lane < n && box_overlaps(mB, wb);
       float4 cB = z4;
       if (ovB) cB = __ldg(SP + 2 * (size_t)rB + 1);
@@ -303,13 +329,14 @@ __global__ void __launch_bounds__(kIgWarps * 32) k_ig_items(gs_proj proj, gs_bin
         // the overlapping entries join the ring in list order; whole chunks of kIgBatch
         // are composited at once and a partial chunk waits for the next group's entries
         if (ovA) {
-          const uint32_t s = (tail + __popc(m & lt)) & (kIgRing - 1);
-          ig_stage(mA, cA, ccx, ccy, sm[s], sc[s]);
+          const uint32_t s = (tail + __popc(m & lt)) & (kRing - 1);
+          stage_pair(sx, s, stage_exponent(mA.x, mA.y, cA, ccx, ccy));
+          su[s] = mA.w;
         }
         tail += __popc(m);
         __syncwarp();
         const uint32_t chunks = (tail - head) / kIgBatch;
-        composite_chunks<kIgBatch>(sm, sc, head, chunks, lo, p, T, cu);
+        composite_chunks<kIgBatch>(sx, su, head, chunks, lo, p, T, cu);
         head += chunks * kIgBatch;
         __syncwarp();
       }
@@ -319,19 +346,19 @@ __global__ void __launch_bounds__(kIgWarps * 32) k_ig_items(gs_proj proj, gs_bin
     }
     // the last partial chunk, padded with entries of C0 = -inf (alpha = 0: adds nothing)
     if (tail != head && __any_sync(0xffffffffu, T != 0.f)) {
-      const uint32_t b0 = head & (kIgRing - 1);
+      const uint32_t b0 = head & (kRing - 1);
       if ((uint32_t)lane >= tail - head && (uint32_t)lane < kIgBatch) {
-        sm[b0 + lane] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-        sc[b0 + lane] = z4;
+        stage_pair(sx, b0 + lane, Exponent{-INFINITY, 0.f, 0.f, 0.f, 0.f, 0.f});
+        su[b0 + lane] = 0.f;
       }
       __syncwarp();
-      composite_chunks<kIgBatch>(sm, sc, head, 1u, lo, p, T, cu);
+      composite_chunks<kIgBatch>(sx, su, head, 1u, lo, p, T, cu);
       __syncwarp();
     }
-    float su = cu;
+    float sum = cu;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) su += __shfl_down_sync(0xffffffffu, su, d);
-    if (lane == 0) item_sum[slot] = su;
+    for (int d = 16; d > 0; d >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, d);
+    if (lane == 0) item_sum[slot] = sum;
   }
 }
 
@@ -405,12 +432,9 @@ cudaError_t launch_render_fwd(const gs_map& map, const gs_proj& proj, const gs_b
   if (items > 0) {
     const unsigned grid = (unsigned)((items + kFwdWarps - 1) / kFwdWarps);
     const int b = p.fwd_batch ? p.fwd_batch : kFwdBatchDefault;
-    if (b == 1)
-      k_render_fwd<1><<<grid, kFwdWarps * 32, 0, st>>>(map, proj, bins, cams, n_views, p, img, (uint32_t)items);
-    else if (b == 4)
-      k_render_fwd<4><<<grid, kFwdWarps * 32, 0, st>>>(map, proj, bins, cams, n_views, p, img, (uint32_t)items);
-    else
-      k_render_fwd<2><<<grid, kFwdWarps * 32, 0, st>>>(map, proj, bins, cams, n_views, p, img, (uint32_t)items);
+    auto kern = img.n_contrib ? (b == 4 ? k_render_fwd<2, true> : k_render_fwd<1, true>)
+                              : (b == 4 ? k_render_fwd<2, false> : k_render_fwd<1, false>);
+    kern<<<grid, kFwdWarps * 32, 0, st>>>(map, proj, bins, cams, n_views, p, img, (uint32_t)items);
     note_launch();
   }
   return cudaGetLastError();

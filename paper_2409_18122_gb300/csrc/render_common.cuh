@@ -117,6 +117,39 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   return d;
 }
 
+// Staged exponents of two consecutive entries of a list (positions 2 i and 2 i + 1), interleaved
+// so that each 16-byte load gives two packed operands:
+// (c0, c0', cu, cu'), (cv, cv', k.x, k.x'), (k.y, k.y', k.z, k.z').
+constexpr int kPairFloats = 12;
+
+// One entry's coefficients into position s of an array of such pairs.
+__device__ __forceinline__ void stage_pair(float* pairs, uint32_t s, const Exponent& e) {
+  float* d = pairs + kPairFloats * (s >> 1) + (s & 1u);
+  d[0] = e.c0;
+  d[2] = e.cu;
+  d[4] = e.cv;
+  d[6] = e.kx;
+  d[8] = e.ky;
+  d[10] = e.kz;
+}
+
+struct LaneOffsets2 {
+  f32x2 u, v, uu, uv, vv;
+};
+
+__device__ __forceinline__ LaneOffsets2 lane_offsets2(int lane) {
+  const LaneOffsets o = lane_offsets(lane);
+  return LaneOffsets2{pack2(o.u, o.u), pack2(o.v, o.v), pack2(o.uu, o.uu), pack2(o.uv, o.uv), pack2(o.vv, o.vv)};
+}
+
+// alpha_raw of both entries of pair i: the same operations in the same order, so the same bits.
+__device__ __forceinline__ float2 alpha_raw2(const float* pairs, uint32_t i, const LaneOffsets2& lo) {
+  const ulonglong2* d = reinterpret_cast<const ulonglong2*>(pairs + kPairFloats * i);
+  const ulonglong2 a = d[0], b = d[1], c = d[2];
+  const float2 e = unpack2(fma2(c.y, lo.vv, fma2(c.x, lo.uv, fma2(b.y, lo.uu, fma2(b.x, lo.v, fma2(a.y, lo.u, a.x))))));
+  return make_float2(ex2_approx(e.x), ex2_approx(e.y));
+}
+
 // Work item of the compositing kernels: one warp renders one 8 x (4 KP) pixel
 // block of one screen tile, KP pixels per lane (KP = 1 in every kernel: a larger
 // block per warp culls less finely, which costs more than it saves).  Block b of a tile covers columns

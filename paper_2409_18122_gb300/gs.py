@@ -34,7 +34,7 @@ class RenderParams:
     alpha_max: float = 0.99
     T_min: float = 1e-4
     ig_batch: int = 0      # chunk depth of the information-gain compositing: 4, 8 or 16 (0: 8)
-    fwd_batch: int = 0     # chunk depth of the forward compositing: 1, 2 or 4 (0: 2)
+    fwd_batch: int = 0     # chunk depth of the forward compositing: 1, 2 or 4 (0: 4; 1 runs as 2)
 
     def c(self) -> L.gs_params:
         return L.gs_params(self.tile_w, self.tile_h, self.eps2d, self.near, self.guard, self.alpha_min,
@@ -895,7 +895,7 @@ def autotune_mapping(gmap: GaussianMapTensors, cams: Sequence, params: RenderPar
         del fr, img, grads
         return ms
 
-    d_batch = params.fwd_batch or 2
+    d_batch = params.fwd_batch or 4
     for tw, th in tiles:
         if not valid_tile(tw, th):
             continue

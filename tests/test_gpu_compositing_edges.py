@@ -1,0 +1,74 @@
+"""Forward and information-gain compositing at the edges of its staging: lists whose length
+ends inside a chunk, a group of 32 or the 64-entry ring, pixels that saturate in the middle of
+a chunk or never, and alpha_min = 0 (no entry is skipped, the padding of a list's last chunk
+must still add nothing), against the oracle.  Tolerances are gpu_helpers'."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2409_18122_gb300 import gs
+from paper_2409_18122_gb300.scenes import Camera, GaussianMap
+
+from gpu_helpers import DEPTH_RTOL, IG_RTOL, IMG_ATOL, images_host
+
+pytestmark = pytest.mark.gpu
+
+
+def _stack(n, logit, seed=0):
+    """n Gaussians of about 2 to 6 pixels one behind another in front of an odd-sized 13 x 9 view."""
+    rng = np.random.default_rng(seed + n)
+    mo = np.zeros((n, 4), np.float32)
+    mo[:, :2] = rng.uniform(-0.5, 0.5, (n, 2))
+    mo[:, 2] = 2.0 + np.arange(n) * 0.01
+    mo[:, 3] = logit + 0.3 * rng.standard_normal(n)
+    su = np.concatenate([rng.uniform(-2.0, -1.0, (n, 3)), rng.uniform(0, 1, (n, 1))], 1).astype(np.float32)
+    q = rng.standard_normal((n, 4))
+    q = (q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32)
+    rgb = np.concatenate([rng.uniform(0, 1, (n, 3)), np.zeros((n, 1))], 1).astype(np.float32)
+    cam = Camera(30.0, 30.0, 6.5, 4.5, 13, 9, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
+    return GaussianMap(mo, su, q, rgb), [cam]
+
+
+@pytest.mark.parametrize("logit", [-4.0, 0.0])      # transparent: nothing saturates; opaque: all lanes do
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 8, 9, 31, 32, 33, 63, 64, 65, 97])
+def test_list_lengths(n, logit):
+    gmap, cams = _stack(n, logit)
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    ref = O.render_images(gmap, cams)[0]
+    outs = []
+    for b in gs.FWD_BATCH_CANDIDATES:
+        fr = gs.Frame(n, cams, gs.RenderParams(fwd_batch=b))
+        img = fr.forward(gm, fr.new_images(with_counts=True))
+        torch.cuda.synchronize()
+        fr.check_status()
+        h = images_host(fr, img)[0]
+        h["n_contrib"] = img["n_contrib"].cpu().numpy()
+        outs.append(h)
+        ok = ~ref["knife"]                    # pixels whose skip and stop decisions are clear of rounding
+        for k in ("rgb", "unc", "T"):
+            np.testing.assert_allclose(h[k][ok], ref[k][ok], rtol=0, atol=IMG_ATOL, err_msg=k)
+        np.testing.assert_allclose(h["depth"][ok], ref["depth"][ok], rtol=0, atol=DEPTH_RTOL * (2.0 + 0.01 * n))
+    for o in outs[1:]:
+        for k in ("rgb", "depth", "unc", "T", "last", "n_contrib"):
+            np.testing.assert_array_equal(o[k], outs[0][k])
+    if not ref["knife"].any():
+        for b in gs.IG_BATCH_CANDIDATES:
+            ig = float(gs.InfoGain(n, cams, gs.RenderParams(ig_batch=b))(gm)[0])
+            assert abs(ig - ref["unc"].mean()) <= IG_RTOL * abs(ref["unc"].mean()) + 1e-7
+
+
+@pytest.mark.parametrize("n", [1, 3, 5, 33])
+def test_padding_adds_nothing_without_an_opacity_floor(n):
+    """alpha_min = 0: the padded entries of the last chunk (alpha = 0) are not skipped by the
+    floor; colours that were staged by earlier work (here infinite ones) must not leak in."""
+    gmap, cams = _stack(n, -1.0)
+    hot = GaussianMap(gmap.mo, gmap.su, gmap.q, np.full_like(gmap.rgb, np.inf))
+    prm = gs.RenderParams(alpha_min=0.0)
+    gs.Frame(n, cams, prm).forward(gs.GaussianMapTensors.from_numpy(hot))
+    fr = gs.Frame(n, cams, prm)
+    img = fr.forward(gs.GaussianMapTensors.from_numpy(gmap), fr.new_images(with_counts=True))
+    torch.cuda.synchronize()
+    out = images_host(fr, img)[0]
+    assert np.isfinite(out["rgb"]).all() and np.isfinite(out["depth"]).all()
+    assert (out["last"] <= n).all() and (img["n_contrib"] <= n).all()
