@@ -274,7 +274,9 @@ __global__ void __launch_bounds__(kBinWarps * 32) k_bin_hist(const gs_proj proj,
 __global__ void k_bin_ranges(const uint32_t* __restrict__ off, const uint32_t* __restrict__ scan_n,
                              const uint32_t* __restrict__ total, int K, int64_t pair_cap, int64_t tile_cap,
                              const uint32_t* __restrict__ view_info, int n_views, uint32_t* __restrict__ ranges,
-                             uint32_t* __restrict__ bins_count, uint32_t* status) {
+                             uint32_t* __restrict__ bins_count, uint32_t* status,
+                             uint32_t* __restrict__ order_cnt) {
+  if (blockIdx.x == 0 && threadIdx.x < 2 * kOrderBuckets) order_cnt[threadIdx.x] = 0u;   // (kBlock threads)
   const int64_t lim = (int64_t)*scan_n / K;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const uint32_t t = *total;
@@ -311,7 +313,7 @@ __global__ void k_bin_ranges(const uint32_t* __restrict__ off, const uint32_t* _
 template <bool kTileIds>
 __global__ void __launch_bounds__(kBinWarps * 32, 5) k_bin_place(const gs_proj proj,
                                                                  const uint32_t* __restrict__ bounds,
-                                                                 const uint32_t* __restrict__ srec,
+                                                                 const SortedRecords sorted,
                                                                  const ushort4* __restrict__ srect, int n_views, int K,
                                                                  int64_t tile_cap, const uint32_t* __restrict__ off,
                                                                  gs_bins out) {
@@ -322,6 +324,7 @@ __global__ void __launch_bounds__(kBinWarps * 32, 5) k_bin_place(const gs_proj p
   __shared__ uint32_t s_magic[kWinCols + 1];
   for (int i = threadIdx.x; i <= kWinCols; i += blockDim.x) s_magic[i] = i > 1 ? 0xFFFFFFFFu / (uint32_t)i + 1u : 0u;
   __syncthreads();
+  const uint32_t* __restrict__ srec = sorted.get();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t lt = (1u << lane) - 1u;
   const uint32_t le = (2u << lane) - 1u;   // lanes 0 .. lane (all 32 for lane 31)
@@ -450,7 +453,6 @@ __global__ void __launch_bounds__(kBinWarps * 32, 5) k_bin_place(const gs_proj p
 // of view v) ordered longest tile list first, by a counting sort over kOrderBuckets buckets
 // of list length, four per doubling.  The compositing kernels take their items in this
 // order, so that the longest lists start first instead of wherever their tile falls.
-constexpr int kOrderBuckets = 64;
 
 // Bucket of a list of `len` pairs: 0 for the longest lists.
 __device__ inline uint32_t order_bucket(uint32_t len) {
@@ -476,22 +478,24 @@ __device__ inline uint32_t item_list_len(uint32_t i, const uint32_t* __restrict_
   return ranges[2 * (size_t)tile + 1] - ranges[2 * (size_t)tile];
 }
 
-__global__ void k_order_zero(uint32_t* __restrict__ cnt) {   // counts and cursors
-  for (int i = threadIdx.x; i < 2 * kOrderBuckets; i += blockDim.x) cnt[i] = 0u;
+// Items of the batch to order: all of them if the order array holds them, else none or
+// (clamp) the first item_cap.
+__device__ inline int64_t order_items(const uint32_t* __restrict__ view_info, int n_views, int64_t item_cap,
+                                      bool clamp) {
+  const int64_t n = view_info[kVI * n_views + 2];
+  return n <= item_cap ? n : (clamp ? item_cap : 0);
 }
 
-// Items per bucket (nothing when the batch has more than item_cap items).
+// Items per bucket.
 __global__ void __launch_bounds__(kBlock) k_order_count(const uint32_t* __restrict__ view_info, int n_views,
                                                         const uint32_t* __restrict__ ranges, int64_t tile_cap,
-                                                        int64_t item_cap, uint32_t* __restrict__ cnt) {
+                                                        int64_t item_cap, bool clamp, uint32_t* __restrict__ cnt) {
   __shared__ uint32_t s_cnt[kOrderBuckets];
   for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x) s_cnt[i] = 0u;
   __syncthreads();
-  const int64_t n = view_info[kVI * n_views + 2];
-  if (n <= item_cap) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-      atomicAdd(&s_cnt[order_bucket(item_list_len((uint32_t)i, view_info, n_views, ranges, tile_cap))], 1u);
-  }
+  const int64_t n = order_items(view_info, n_views, item_cap, clamp);
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(&s_cnt[order_bucket(item_list_len((uint32_t)i, view_info, n_views, ranges, tile_cap))], 1u);
   __syncthreads();
   for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x)
     if (s_cnt[i]) atomicAdd(&cnt[i], s_cnt[i]);
@@ -500,11 +504,11 @@ __global__ void __launch_bounds__(kBlock) k_order_count(const uint32_t* __restri
 // Every item to its bucket's next free position; one atomic per (warp, bucket).
 __global__ void __launch_bounds__(kBlock) k_order_place(const uint32_t* __restrict__ view_info, int n_views,
                                                         const uint32_t* __restrict__ ranges, int64_t tile_cap,
-                                                        int64_t item_cap, const uint32_t* __restrict__ cnt,
-                                                        uint32_t* __restrict__ cur, uint32_t* __restrict__ order) {
+                                                        int64_t item_cap, bool clamp,
+                                                        const uint32_t* __restrict__ cnt, uint32_t* __restrict__ cur,
+                                                        uint32_t* __restrict__ order) {
   __shared__ uint32_t s_base[kOrderBuckets];
-  const int64_t n = view_info[kVI * n_views + 2];
-  if (n > item_cap) return;
+  const int64_t n = order_items(view_info, n_views, item_cap, clamp);
   const int lane = threadIdx.x & 31;
   if (threadIdx.x < 32) {   // exclusive scan of the bucket counts, two per lane
     const uint32_t a = cnt[2 * lane], b = cnt[2 * lane + 1];
@@ -536,6 +540,16 @@ __global__ void __launch_bounds__(kBlock) k_order_place(const uint32_t* __restri
 
 }  // namespace
 
+void launch_item_order(const uint32_t* view_info, int n_views, const uint32_t* ranges, int64_t tile_cap,
+                       int64_t item_cap, bool clamp, uint32_t* cnt, uint32_t* order, cudaStream_t st) {
+  const unsigned og = grid_for(item_cap);
+  k_order_count<<<og, kBlock, 0, st>>>(view_info, n_views, ranges, tile_cap, item_cap, clamp, cnt);
+  note_launch();
+  k_order_place<<<og, kBlock, 0, st>>>(view_info, n_views, ranges, tile_cap, item_cap, clamp, cnt,
+                                       cnt + kOrderBuckets, order);
+  note_launch();
+}
+
 size_t bin_ws_bytes(int64_t rec_cap, int64_t pair_cap, int64_t tile_cap, int n_views) {
   const int K = chunks_per_view(n_views, tile_cap, pair_cap);
   const int64_t cnt_cap = (int64_t)K * tile_cap + 1;
@@ -553,7 +567,7 @@ size_t bin_ws_bytes(int64_t rec_cap, int64_t pair_cap, int64_t tile_cap, int n_v
   c.take<uint32_t>(cnt_cap);               // ... scanned
   c.take<uint32_t>((int64_t)n_views * (K + 1));   // first sorted record of every chunk
   c.take<uint32_t>(2 * kOrderBuckets);            // item order: bucket counts and cursors
-  size_t t = sort_temp_bytes(rec_cap, n_views);
+  size_t t = record_sort_temp_bytes(rec_cap, n_views);
   size_t s = scan_temp_bytes(cnt_cap > rec_cap ? cnt_cap : rec_cap);
   c.take<char>(t > s ? t : s);
   return align_up(c.off, 256);
@@ -568,7 +582,7 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
   const int64_t cnt_cap = (int64_t)K * tile_cap + 1;
   Carver c(ws);
   uint32_t* seg = c.take<uint32_t>(n_views + 1);
-  uint32_t* ctr = c.take<uint32_t>(4);      // [0] count entries to scan, [1] pair total
+  uint32_t* ctr = c.take<uint32_t>(4);      // [0] count entries to scan, [1] pair total, [2..3] key range
   uint32_t* rk_a = c.take<uint32_t>(rec_cap);
   uint32_t* rv_a = c.take<uint32_t>(rec_cap);
   uint32_t* rk_b = c.take<uint32_t>(rec_cap);
@@ -580,7 +594,7 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
   uint32_t* off = c.take<uint32_t>(cnt_cap);
   uint32_t* bounds = c.take<uint32_t>((int64_t)n_views * (K + 1));
   uint32_t* ocnt = c.take<uint32_t>(2 * kOrderBuckets);
-  size_t t = sort_temp_bytes(rec_cap, n_views);
+  size_t t = record_sort_temp_bytes(rec_cap, n_views);
   size_t s = scan_temp_bytes(cnt_cap > rec_cap ? cnt_cap : rec_cap);
   void* tmp = c.take<char>(t > s ? t : s);
 
@@ -594,14 +608,13 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
     k_segments<<<grid_for(rec_cap), kBlock, 0, st>>>(proj, n_views, tile_cap, K, seg, &ctr[0]);
     note_launch();
   }
-  // 2. record indices by depth bits within each view (4 passes: result back in the a buffers)
+  // 2. record indices by depth bits within each view
   // (the last pass also writes the rectangles in sorted order and their pair counts)
-  bool in_a = false;
   const SortRectEpilogue epi{reinterpret_cast<const ushort4*>(proj.rect), proj.view_info, srect, rcnt, proj.status};
-  cudaError_t e = radix_sort(proj.depth_key, nullptr, SortBufs{rk_a, rv_a, rk_b, rv_b}, proj.count, rec_cap, 0, 32,
-                             tmp, st, &in_a, seg, n_views, &epi);
+  SortedRecords srec;
+  cudaError_t e = record_sort(proj.depth_key, SortBufs{rk_a, rv_a, rk_b, rv_b}, proj.count, rec_cap, seg, n_views, epi,
+                              &ctr[2], tmp, st, &srec);
   if (e != cudaSuccess) return e;
-  const uint32_t* srec = in_a ? rv_a : rv_b;
   // 3. pair numbering
   e = scan_exclusive(rcnt, poff, proj.count, rec_cap, nullptr, tmp, st);
   if (e != cudaSuccess) return e;
@@ -616,7 +629,7 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
   e = scan_exclusive(cnt, off, &ctr[0], cnt_cap - 1, &ctr[1], tmp, st);
   if (e != cudaSuccess) return e;
   k_bin_ranges<<<grid_for(tile_cap), kBlock, 0, st>>>(off, &ctr[0], &ctr[1], K, out.pair_capacity, tile_cap,
-                                                      proj.view_info, n_views, out.ranges, out.count, proj.status);
+                                                      proj.view_info, n_views, out.ranges, out.count, proj.status, ocnt);
   note_launch();
   // 6. placement
   if (out.tile)
@@ -626,14 +639,7 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
   note_launch();
   // 7. warp items longest tile list first, for the compositing kernels (optional)
   if (out.item_order && out.item_capacity > 0) {
-    k_order_zero<<<1, 2 * kOrderBuckets, 0, st>>>(ocnt);
-    note_launch();
-    const unsigned og = grid_for(out.item_capacity);
-    k_order_count<<<og, kBlock, 0, st>>>(proj.view_info, n_views, out.ranges, tile_cap, out.item_capacity, ocnt);
-    note_launch();
-    k_order_place<<<og, kBlock, 0, st>>>(proj.view_info, n_views, out.ranges, tile_cap, out.item_capacity, ocnt,
-                                         ocnt + kOrderBuckets, out.item_order);
-    note_launch();
+    launch_item_order(proj.view_info, n_views, out.ranges, tile_cap, out.item_capacity, false, ocnt, out.item_order, st);
   }
   return cudaGetLastError();
 }

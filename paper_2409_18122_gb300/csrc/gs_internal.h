@@ -54,28 +54,20 @@ size_t scan_temp_bytes(int64_t n_cap);
 cudaError_t scan_exclusive(const uint32_t* in, uint32_t* out, const uint32_t* n_dev, int64_t n_cap,
                            uint32_t* total_out, void* temp, cudaStream_t st);
 
-// ------------------------------------------------------------------ radix sort
-// Stable LSD radix sort of (key, value) uint32 pairs on bits [bit_begin, bit_end).
-// Input: keys_in, vals_in (nullable: identity 0..n-1).  Buffers a/b are
-// ping-pong storage of n_cap entries each; the sorted result ends in a if the
-// number of 8-bit passes is even, else in b.  *result_in_a tells which.
-// n = min(*n_dev, n_cap).  With seg != NULL and n_seg > 1 (segmented mode) the
-// elements [seg[s], seg[s+1]) of every segment s < n_seg (seg non-decreasing,
-// seg[n_seg] = n) are sorted among themselves and stay in place.
-// sort_temp_bytes(n_cap, n_seg): scratch for either mode (n_seg 0 for plain).
+// ------------------------------------------------------------------ record sort
+// Stable sort of record indices by their keys within each segment (view): the elements
+// [seg[s], seg[s+1]) of every segment s < n_seg (seg non-decreasing, seg[n_seg] = n =
+// min(*n_dev, n_cap)) are sorted among themselves and stay in place.  Buffers a/b are ping-pong
+// storage of n_cap entries each; ctl: two words that stay valid as long as the result is used.
 struct SortBufs {
   uint32_t* keys_a;
   uint32_t* vals_a;
   uint32_t* keys_b;
   uint32_t* vals_b;
 };
-size_t sort_temp_bytes(int64_t n_cap, int n_seg = 0);
-// Optional work of the last pass of a sort whose segments are the views of a
-// binning batch and whose values are record indices: for the element r written
-// to position i, out_rect[i] = rect[r] and out_cnt[i] = its number of tiles (0,
-// with an empty out_rect[i], for an empty rectangle or one outside its view's
-// tile grid -- the latter also sets GS_FLAG_BAD_RECORDS).  The sorted keys are
-// then not written.
+// Work of the last pass: for the record r written to position i, out_rect[i] = rect[r] and
+// out_cnt[i] = its number of tiles (0, with an empty out_rect[i], for an empty rectangle or one
+// outside its view's tile grid -- the latter also sets GS_FLAG_BAD_RECORDS).
 struct SortRectEpilogue {
   const ushort4* rect;
   const uint32_t* view_info;
@@ -83,10 +75,20 @@ struct SortRectEpilogue {
   uint32_t* out_cnt;
   uint32_t* status;
 };
-int sort_passes(int bit_begin, int bit_end);
-cudaError_t radix_sort(const uint32_t* keys_in, const uint32_t* vals_in, SortBufs bufs, const uint32_t* n_dev,
-                       int64_t n_cap, int bit_begin, int bit_end, void* temp, cudaStream_t st, bool* result_in_a,
-                       const uint32_t* seg = nullptr, int n_seg = 0, const SortRectEpilogue* epi = nullptr);
+// Whether three 9-bit passes sort the keys (ctl = smallest and largest key): their top 14 bits
+// differ by less than 512.
+__host__ __device__ inline bool sorted_in_three(const uint32_t* ctl) { return (ctl[1] >> 18) - (ctl[0] >> 18) < 512u; }
+// The sorted record indices: which buffer holds them is known on the device.
+struct SortedRecords {
+  const uint32_t* three;   // after three passes
+  const uint32_t* four;    // after four
+  const uint32_t* ctl;
+  __device__ const uint32_t* get() const { return sorted_in_three(ctl) ? three : four; }
+};
+size_t record_sort_temp_bytes(int64_t n_cap, int n_seg);
+cudaError_t record_sort(const uint32_t* keys, SortBufs bufs, const uint32_t* n_dev, int64_t n_cap, const uint32_t* seg,
+                        int n_seg, const SortRectEpilogue& epi, uint32_t* ctl, void* temp, cudaStream_t st,
+                        SortedRecords* out);
 
 // ------------------------------------------------------------------ pipeline stages
 size_t project_ws_bytes(int64_t n, int n_views);
@@ -98,6 +100,13 @@ size_t bin_ws_bytes(int64_t rec_cap, int64_t pair_cap, int64_t tile_cap, int n_v
 // come from proj.grp_base and the group count in view_info[V][3].
 cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_views, const gs_params& p,
                             const gs_bins& out, void* ws, cudaStream_t st);
+
+// The warp items of the batch (n of them, view_info[V][2]) ordered longest tile list first.
+// cnt: 2 * kOrderBuckets words, zero.  n > item_cap: the first item_cap items if `clamp`, else
+// nothing is written.
+constexpr int kOrderBuckets = 64;
+void launch_item_order(const uint32_t* view_info, int n_views, const uint32_t* ranges, int64_t tile_cap,
+                       int64_t item_cap, bool clamp, uint32_t* cnt, uint32_t* order, cudaStream_t st);
 
 cudaError_t launch_render_fwd(const gs_map& map, const gs_proj& proj, const gs_bins& bins, const gs_camera* cams,
                               int n_views, const gs_params& p, const gs_image& img, cudaStream_t st);
