@@ -1,16 +1,23 @@
 // loss.cu -- the mapping loss of Eq. 3 (L1 depth + L1 colour + SSIM) and its gradient
 // with respect to the rendered images.
 //
-// Two tiled passes over 32x16-pixel output tiles of each (view, channel), one CTA each:
+// Two tiled passes over 32x54-pixel output tiles of each (view, channel), one CTA each:
 //   pass 1  loads the tile of x (render) and y (reference) with a 5-pixel halo into shared
-//           memory, blurs the five moments x, y, x^2, y^2, xy with the separable 11-tap
-//           window (rows, then columns), evaluates S(p) and the partial derivatives of S
-//           with respect to the three moments that depend on x (m1 = G*x, m2 = G*x^2,
-//           m12 = G*xy), stores those as three planes and reduces S and the L1 terms of the
-//           tile into one FP64 partial per CTA;
+//           memory, blurs the four moments x, y, (x - y)^2, xy with the separable 11-tap window
+//           (rows, then columns; S needs the two variances only as their sum, which is
+//           var(x - y) + 2 cov(x, y)), evaluates S(p)
+//           and the partial derivatives of S with respect to the three moments that depend on x
+//           (m1 = G*x, m2 = G*x^2, m12 = G*xy), stores those as three planes and reduces S and
+//           the L1 terms of the tile into one FP64 partial per CTA;
 //   pass 2  blurs the three derivative planes with the same window (the adjoint of the
 //           zero-padded correlation with a symmetric window is itself) and forms
 //           dS/dx = G*dm1 + 2 x G*dm2 + y G*dm12, then dL/dx with the L1 sign term.
+// Both are bound by the multiply-adds and shared-memory traffic of the blur (pass 1: about 100
+// fused multiply-adds and 30 shared wavefronts per 32 pixels), so the window slides in registers:
+// a thread blurs four neighbouring pixels of a row from five 16-byte loads per plane, then seven
+// pixels of a column from seventeen loads; the moments' products are formed on the way.  54 rows
+// and the halo are 64, two row quads per thread, 1.19 row blurs per output row.  Eight 1280x720
+// views: pass 1 478 -> 283 us, pass 2 276 -> 184 us, the sum of the partials 57 -> 17 us.
 // A one-CTA kernel sums the partials in FP64 in a fixed order.  Without the SSIM term
 // (w_ssim = 0) the loss is elementwise: one flat kernel over the colour and one over the
 // depth array (contiguous chunks per block, fixed partial slots) replaces both passes.
@@ -21,13 +28,18 @@
 namespace gs {
 namespace {
 
-constexpr int kLTW = 32, kLTH = 16;           // output tile
 constexpr int kR = 5, kWin = 2 * kR + 1;      // 11-tap window
-constexpr int kInW = kLTW + 2 * kR, kInH = kLTH + 2 * kR;
-constexpr int kLossThreads = 256;             // 8 warps: warp w owns output rows 2w, 2w+1
+constexpr int kLTW = 32, kLTH = 54;           // output tile
+constexpr int kInH = kLTH + 2 * kR;           // 64 rows of input
+constexpr int kPitch = 48;                    // input columns x0 - 8 .. x0 + 39: quads of columns are 16-byte aligned
+constexpr int kPad = 8;                       // columns before the output tile in a row of shared memory
+constexpr int kLossThreads = 256;             // 8 warps
+constexpr int kColRows = 7;                   // output rows of a thread in the column pass: warp w owns 7w .. 7w + 6
+constexpr int kRowsH = kColRows * kLossThreads / 32 + kWin - 1;   // ... whose inputs reach past the 64 rows (not used)
 constexpr int kLossViewsPerLaunch = 64;
 constexpr float kC1 = 0.01f * 0.01f, kC2 = 0.03f * 0.03f;
-static_assert(kLossThreads == kLTW * kLTH / 2, "two output pixels per thread");
+static_assert(kLTW == 32 && kInH * kLTW / 4 == 2 * kLossThreads, "two row quads per thread");
+static_assert(kColRows * (kLossThreads / 32) >= kLTH, "the warps cover the output rows");
 
 struct LossView {
   int64_t pix_base;  // first pixel of the view in the concatenated images
@@ -78,52 +90,91 @@ __device__ __forceinline__ TileGeo tile_geo(const LossArgs& a, int t, int ch) {
   return g;
 }
 
-// Loads NP planes (src[k] + base) of a halo tile into s[k], zero outside the image.
+// Copies NP planes (src[k] + base) of a halo tile into s[k], zero outside the image: a warp per row,
+// columns x0 - 5 .. x0 + 36.  The copies are asynchronous, so that all of a thread's are in flight
+// together (through registers, the few loads that are in flight at a time made the
+// tiles wait for memory: 421 and 386 us).
 template <int NP>
-__device__ __forceinline__ void load_halo(const float* const* src, const TileGeo& g, float (*s)[kInH][kInW]) {
-  for (int i = threadIdx.x; i < kInH * kInW; i += kLossThreads) {
-    const int r = i / kInW, c = i - r * kInW;
-    const int gx = g.x0 - kR + c, gy = g.y0 - kR + r;
-    const bool in = gx >= 0 && gx < g.W && gy >= 0 && gy < g.H;
-    const int64_t o = g.base + (int64_t)gy * g.W + gx;
+__device__ __forceinline__ void load_halo(const float* const* src, const TileGeo& g, float (*s)[kInH][kPitch]) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) s[k][r][c] = in ? src[k][o] : 0.f;
+  for (int i = 0; i < kInH / (kLossThreads / 32); ++i) {
+    const int r = (threadIdx.x >> 5) + i * (kLossThreads / 32);
+    const int gy = g.y0 - kR + r;
+    const bool row = gy >= 0 && gy < g.H;
+    const int64_t o = g.base + (int64_t)gy * g.W;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int c = h * 32 + lane, gx = g.x0 - kR + c;
+      const bool in = row && gx >= 0 && gx < g.W;
+      if (c < kLTW + 2 * kR) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+          const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s[k][r][kPad - kR + c]);
+          const float* from = src[k] + (in ? o + gx : g.base);   // (nothing is read outside the image)
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(from), "r"(in ? 4 : 0) : "memory");
+        }
+      }
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Row pass: plane k of the NP blurred ones at input column t is val(k, v) of the NI loaded values v
+// of that column; each thread blurs two quads of four columns.
+template <int NI, int NP, class F>
+__device__ __forceinline__ void blur_rows(const LossArgs& a, const float (*s_in)[kInH][kPitch],
+                                          float (*s_h)[kRowsH][kLTW], F val) {
+#pragma unroll 1
+  for (int i = threadIdx.x; i < kInH * kLTW / 4; i += kLossThreads) {
+    const int r = i >> 3, c = 4 * (i & 7);
+    float acc[NP][4];
+#pragma unroll
+    for (int k = 0; k < NP; ++k)
+#pragma unroll
+      for (int o = 0; o < 4; ++o) acc[k][o] = 0.f;
+    // output column c + o takes input columns c + o - 5 .. c + o + 5, which are at kPad further on
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      float v[NI][4];
+#pragma unroll
+      for (int n = 0; n < NI; ++n) {
+        const float4 w = *reinterpret_cast<const float4*>(&s_in[n][r][c + 4 * q]);
+        v[n][0] = w.x; v[n][1] = w.y; v[n][2] = w.z; v[n][3] = w.w;
+      }
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int j = 4 * q + t - (kPad - kR);   // tap of output column c
+        if (j < 0 || j > kWin + 2) continue;
+        float in[NI], m[NP];
+#pragma unroll
+        for (int n = 0; n < NI; ++n) in[n] = v[n][t];
+        val(in, m);
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+          if (j - o < 0 || j - o >= kWin) continue;
+#pragma unroll
+          for (int k = 0; k < NP; ++k) acc[k][o] = fmaf(a.g[j - o], m[k], acc[k][o]);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NP; ++k)
+      *reinterpret_cast<float4*>(&s_h[k][r][c]) = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
   }
 }
 
-// Row pass then column pass of the separable window over NP planes; out[k][q] is the
-// blurred value of plane k at output row 2 * warp + q, column lane.
-template <int NP>
-__device__ __forceinline__ void blur_tile(const LossArgs& a, float (*s_in)[kInH][kInW], float (*s_h)[kInH][kLTW],
-                                          float (&out)[NP][2]) {
-  for (int i = threadIdx.x; i < kInH * kLTW; i += kLossThreads) {
-    const int r = i / kLTW, c = i % kLTW;
-    float acc[NP];
+// Column pass of one plane: out[q] = blurred value at output row r0 + q, column c.
+__device__ __forceinline__ void blur_column(const LossArgs& a, const float (*s_h)[kLTW], int r0, int c,
+                                            float (&out)[kColRows]) {
 #pragma unroll
-    for (int k = 0; k < NP; ++k) acc[k] = 0.f;
+  for (int q = 0; q < kColRows; ++q) out[q] = 0.f;
 #pragma unroll
-    for (int j = 0; j < kWin; ++j) {
+  for (int j = 0; j < kColRows + kWin - 1; ++j) {
+    const float h = s_h[r0 + j][c];
 #pragma unroll
-      for (int k = 0; k < NP; ++k) acc[k] = fmaf(a.g[j], s_in[k][r][c + j], acc[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < NP; ++k) s_h[k][r][c] = acc[k];
-  }
-  __syncthreads();
-  const int c = threadIdx.x & 31, r0 = 2 * (threadIdx.x >> 5);
-#pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    float h[kWin + 1];
-#pragma unroll
-    for (int j = 0; j <= kWin; ++j) h[j] = s_h[k][r0 + j][c];
-    float a0 = 0.f, a1 = 0.f;
-#pragma unroll
-    for (int j = 0; j < kWin; ++j) {
-      a0 = fmaf(a.g[j], h[j], a0);
-      a1 = fmaf(a.g[j], h[j + 1], a1);
-    }
-    out[k][0] = a0;
-    out[k][1] = a1;
+    for (int q = 0; q < kColRows; ++q)
+      if (j - q >= 0 && j - q < kWin) out[q] = fmaf(a.g[j - q], h, out[q]);
   }
 }
 
@@ -155,38 +206,45 @@ __device__ __forceinline__ void block_partial(float v0, float v1, float v2, doub
   }
 }
 
+constexpr size_t kFwdSmem = sizeof(float) * (2 * kInH * kPitch + 4 * kRowsH * kLTW);
+constexpr size_t kBwdSmem = sizeof(float) * (3 * kInH * kPitch + 3 * kRowsH * kLTW);
+
 __global__ void __launch_bounds__(kLossThreads) k_loss_fwd(const __grid_constant__ LossArgs a) {
+  extern __shared__ __align__(16) float s_mem[];
+  float (*s_in)[kInH][kPitch] = reinterpret_cast<float (*)[kInH][kPitch]>(s_mem);   // x, y
+  float (*s_h)[kRowsH][kLTW] = reinterpret_cast<float (*)[kRowsH][kLTW]>(s_mem + 2 * kInH * kPitch);
   const int t = blockIdx.x, ch = blockIdx.y;
   const TileGeo g = tile_geo(a, t, ch);
-  const int c = threadIdx.x & 31, r0 = 2 * (threadIdx.x >> 5);
+  const int c = threadIdx.x & 31, r0 = kColRows * (threadIdx.x >> 5);
+  const int px = g.x0 + c;
   float s_sum = 0.f, l1c = 0.f, l1d = 0.f;
 
-  __shared__ float s_in[5][kInH][kInW];  // x, y, x^2, y^2, xy
-  __shared__ float s_h[5][kInH][kLTW];
-  for (int i = threadIdx.x; i < kInH * kInW; i += kLossThreads) {
-    const int r = i / kInW, cc = i - r * kInW;
-    const int gx = g.x0 - kR + cc, gy = g.y0 - kR + r;
-    const bool in = gx >= 0 && gx < g.W && gy >= 0 && gy < g.H;
-    const int64_t o = g.base + (int64_t)gy * g.W + gx;
-    const float xv = in ? a.rgb[o] : 0.f, yv = in ? a.rgb_ref[o] : 0.f;
-    s_in[0][r][cc] = xv;
-    s_in[1][r][cc] = yv;
-    s_in[2][r][cc] = xv * xv;
-    s_in[3][r][cc] = yv * yv;
-    s_in[4][r][cc] = xv * yv;
-  }
+  const float* src[2] = {a.rgb, a.rgb_ref};
+  load_halo<2>(src, g, s_in);
   __syncthreads();
-  float m[5][2];
-  blur_tile<5>(a, s_in, s_h, m);
+  blur_rows<2, 4>(a, s_in, s_h, [](const float* v, float* m) {
+    m[0] = v[0];
+    m[1] = v[1];
+    const float d = v[0] - v[1];
+    m[2] = d * d;
+    m[3] = v[0] * v[1];
+  });
+  __syncthreads();
+  float m1[kColRows], m2[kColRows], m3[kColRows], m4[kColRows];
+  blur_column(a, s_h[0], r0, c, m1);
+  blur_column(a, s_h[1], r0, c, m2);
+  blur_column(a, s_h[2], r0, c, m3);
+  blur_column(a, s_h[3], r0, c, m4);
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int px = g.x0 + c, py = g.y0 + r0 + q;
-    if (px >= g.W || py >= g.H) continue;
+  for (int q = 0; q < kColRows; ++q) {
+    const int py = g.y0 + r0 + q;
+    if (px >= g.W || py >= g.H || r0 + q >= kLTH) continue;
     const int64_t o = g.base + (int64_t)py * g.W + px;
-    const float mx = m[0][q], my = m[1][q];
-    const float sxx = m[2][q] - mx * mx, syy = m[3][q] - my * my, sxy = m[4][q] - mx * my;
+    const float mx = m1[q], my = m2[q];
+    // the variances' sum is 2 cov(x, y) + var(x - y): less cancellation than two variances
+    const float dm = mx - my, sxy = m4[q] - mx * my;
     const float A1 = 2.f * mx * my + kC1, A2 = 2.f * sxy + kC2;
-    const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
+    const float B1 = A1 + dm * dm, B2 = A2 + (m3[q] - dm * dm);
     const float iD = __frcp_rn(B1 * B2);
     const float S = A1 * A2 * iD;
     s_sum += S;
@@ -196,14 +254,14 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_fwd(const __grid_constant
       a.dm[3 * a.P + o] = -S * B1 * iD;
       a.dm[6 * a.P + o] = 2.f * A1 * iD;
     }
-    l1c += fabsf(s_in[0][r0 + q + kR][c + kR] - s_in[1][r0 + q + kR][c + kR]);
+    l1c += fabsf(s_in[0][r0 + q + kR][c + kPad] - s_in[1][r0 + q + kR][c + kPad]);
   }
 
   if (ch == 0 && (a.depth || a.d_depth)) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int px = g.x0 + c, py = g.y0 + r0 + q;
-      if (px >= g.W || py >= g.H) continue;
+    for (int q = 0; q < kColRows; ++q) {
+      const int py = g.y0 + r0 + q;
+      if (px >= g.W || py >= g.H || r0 + q >= kLTH) continue;
       const int64_t o = g.pix + (int64_t)py * g.W + px;
       const float dd = a.depth ? a.depth[o] - a.depth_ref[o] : 0.f;
       l1d += fabsf(dd);
@@ -214,24 +272,42 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_fwd(const __grid_constant
 }
 
 __global__ void __launch_bounds__(kLossThreads) k_loss_ssim_bwd(const __grid_constant__ LossArgs a) {
-  __shared__ float s_in[3][kInH][kInW];
-  __shared__ float s_h[3][kInH][kLTW];
+  extern __shared__ __align__(16) float s_mem[];
+  float (*s_in)[kInH][kPitch] = reinterpret_cast<float (*)[kInH][kPitch]>(s_mem);   // dS/dm1, dS/dm2, dS/dm12
+  float (*s_h)[kRowsH][kLTW] = reinterpret_cast<float (*)[kRowsH][kLTW]>(s_mem + 3 * kInH * kPitch);
   const int t = blockIdx.x, ch = blockIdx.y;
   const TileGeo g = tile_geo(a, t, ch);
   const float* src[3] = {a.dm, a.dm + 3 * a.P, a.dm + 6 * a.P};
+  const int c = threadIdx.x & 31, r0 = kColRows * (threadIdx.x >> 5);
+  const int px = g.x0 + c;
+  float x[kColRows], y[kColRows];
+#pragma unroll
+  for (int q = 0; q < kColRows; ++q) {
+    const int py = g.y0 + r0 + q;
+    const bool in = px < g.W && py < g.H && r0 + q < kLTH;
+    const int64_t o = g.base + (int64_t)py * g.W + px;
+    x[q] = in ? a.rgb[o] : 0.f;
+    y[q] = in ? a.rgb_ref[o] : 0.f;
+  }
   load_halo<3>(src, g, s_in);
   __syncthreads();
-  float b[3][2];
-  blur_tile<3>(a, s_in, s_h, b);
-  const int c = threadIdx.x & 31, r0 = 2 * (threadIdx.x >> 5);
+  blur_rows<3, 3>(a, s_in, s_h, [](const float* v, float* m) {
+    m[0] = v[0];
+    m[1] = v[1];
+    m[2] = v[2];
+  });
+  __syncthreads();
+  float b0[kColRows], b1[kColRows], b2[kColRows];
+  blur_column(a, s_h[0], r0, c, b0);
+  blur_column(a, s_h[1], r0, c, b1);
+  blur_column(a, s_h[2], r0, c, b2);
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int px = g.x0 + c, py = g.y0 + r0 + q;
-    if (px >= g.W || py >= g.H) continue;
+  for (int q = 0; q < kColRows; ++q) {
+    const int py = g.y0 + r0 + q;
+    if (px >= g.W || py >= g.H || r0 + q >= kLTH) continue;
     const int64_t o = g.base + (int64_t)py * g.W + px;
-    const float x = a.rgb[o], y = a.rgb_ref[o];
-    const float dS = fmaf(y, b[2][q], fmaf(2.f * x, b[1][q], b[0][q]));
-    a.d_rgb[o] = a.w_c * sgnf(x - y) * a.inv_n - a.w_s * a.inv_3n * dS;
+    const float dS = fmaf(y[q], b2[q], fmaf(2.f * x[q], b1[q], b0[q]));
+    a.d_rgb[o] = a.w_c * sgnf(x[q] - y[q]) * a.inv_n - a.w_s * a.inv_3n * dS;
   }
 }
 
@@ -255,16 +331,19 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_l1(const float* __restric
   block_partial(0.f, field == 1 ? acc : 0.f, field == 2 ? acc : 0.f, part + 3 * (slot0 + blockIdx.x));
 }
 
-__global__ void __launch_bounds__(kLossThreads)
+// Sums the partials in a fixed order: thread t takes slots t, t + 1024, ..., then a fixed tree.
+constexpr int kFinishThreads = 1024;
+__global__ void __launch_bounds__(kFinishThreads)
     k_loss_finish(const double* part, int64_t n_slots, float w_d, float w_c, float w_s, bool ssim, double n_pix,
                   float* out) {
-  __shared__ double s[3][kLossThreads];
+  __shared__ double s[3][kFinishThreads];
   double acc[3] = {0.0, 0.0, 0.0};
-  for (int64_t i = threadIdx.x; i < n_slots; i += kLossThreads)
+#pragma unroll 4
+  for (int64_t i = threadIdx.x; i < n_slots; i += kFinishThreads)
     for (int k = 0; k < 3; ++k) acc[k] += part[3 * i + k];
   for (int k = 0; k < 3; ++k) s[k][threadIdx.x] = acc[k];
   __syncthreads();
-  for (int h = kLossThreads / 2; h > 0; h >>= 1) {
+  for (int h = kFinishThreads / 2; h > 0; h >>= 1) {
     if (threadIdx.x < h)
       for (int k = 0; k < 3; ++k) s[k][threadIdx.x] += s[k][threadIdx.x + h];
     __syncthreads();
@@ -342,6 +421,14 @@ cudaError_t launch_image_loss(const int32_t* sizes, int n_views, const float* rg
     for (int j = 0; j < kWin; ++j) a.g[j] = (float)(gw[j] / sum);
   }
 
+  static bool attr_set = false;
+  if (ssim && !attr_set) {
+    cudaError_t e = cudaFuncSetAttribute(k_loss_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_loss_ssim_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem);
+    if (e != cudaSuccess) return e;
+    attr_set = true;
+  }
   int64_t pix = 0, slot = 0;
   if (!ssim) {
     // elementwise: contiguous chunks of at least 4096 elements (at most P / 1024 + 2 partial
@@ -374,15 +461,15 @@ cudaError_t launch_image_loss(const int32_t* sizes, int n_views, const float* rg
       tb += ((W + kLTW - 1) / kLTW) * ((H + kLTH - 1) / kLTH);
     }
     const dim3 grid((unsigned)tb, 3);
-    k_loss_fwd<<<grid, kLossThreads, 0, st>>>(a);
+    k_loss_fwd<<<grid, kLossThreads, kFwdSmem, st>>>(a);
     note_launch();
     if (d_rgb) {
-      k_loss_ssim_bwd<<<grid, kLossThreads, 0, st>>>(a);
+      k_loss_ssim_bwd<<<grid, kLossThreads, kBwdSmem, st>>>(a);
       note_launch();
     }
     slot += 3 * (int64_t)tb;
   }
-  k_loss_finish<<<1, kLossThreads, 0, st>>>(part, slot, w.w_depth, w.w_rgb, w.w_ssim, ssim, (double)lay.P,
+  k_loss_finish<<<1, kFinishThreads, 0, st>>>(part, slot, w.w_depth, w.w_rgb, w.w_ssim, ssim, (double)lay.P,
                                             loss_out);
   note_launch();
   return cudaGetLastError();
