@@ -30,6 +30,7 @@ __device__ __forceinline__ void adam1(float& p, float g, float& m, float& v, con
 }
 
 __global__ void __launch_bounds__(kAdamThreads) k_adam(const __grid_constant__ AdamArgs a) {
+  pdl_begin();
   const int ti = blockIdx.y;
   if (ti >= a.nt || !a.g[ti]) return;
   // bias corrections 1 - beta^t = -expm1(t ln beta), accurate also for beta close to 1
@@ -54,7 +55,8 @@ __global__ void __launch_bounds__(kAdamThreads) k_adam(const __grid_constant__ A
   }
 }
 
-__global__ void k_adam_count(uint32_t* step) { *step += 1u; }
+__global__ void k_adam_count(uint32_t* step) {
+  pdl_begin(); *step += 1u; }
 
 }  // namespace
 
@@ -85,11 +87,9 @@ cudaError_t launch_adam(float* const* params, const float* const* grads, float* 
     int64_t bx = (n4_max + kAdamThreads - 1) / kAdamThreads;
     const int64_t cap = (int64_t)device_sm_count() * 8;
     if (bx > cap) bx = cap;
-    k_adam<<<dim3((unsigned)bx, (unsigned)n_tensors), kAdamThreads, 0, st>>>(a);
-    note_launch();
+    launch(k_adam, dim3((unsigned)bx, (unsigned)n_tensors), kAdamThreads, 0, st, a);
   }
-  k_adam_count<<<1, 1, 0, st>>>(step);
-  note_launch();
+  launch(k_adam_count, 1, 1, 0, st, step);
   return cudaGetLastError();
 }
 

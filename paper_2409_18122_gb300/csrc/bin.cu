@@ -69,6 +69,7 @@ __device__ inline int64_t clamp_count(const uint32_t* n_dev, int64_t cap) {
 }
 
 __global__ void k_zero_u32(uint32_t* __restrict__ p, int64_t n) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = 0u;
 }
 
@@ -79,6 +80,7 @@ __global__ void k_zero_u32(uint32_t* __restrict__ p, int64_t n) {
 // that step 4 scans: K * min(total tiles, tile_cap).
 __global__ void k_segments(const gs_proj proj, int n_views, int64_t tile_cap, int K, uint32_t* __restrict__ seg,
                            uint32_t* __restrict__ scan_n) {
+  pdl_begin();
   const int64_t n = clamp_count(proj.count, proj.capacity);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     int64_t tiles = proj.view_info[kVI * n_views];
@@ -127,6 +129,7 @@ __global__ void k_segments(const gs_proj proj, int n_views, int64_t tile_cap, in
 // view_info[V][3]; seg[V] = the record count.
 __global__ void k_segments_from_groups(const gs_proj proj, int n_views, int64_t tile_cap, int K,
                                        uint32_t* __restrict__ seg, uint32_t* __restrict__ scan_n) {
+  pdl_begin();
   const int64_t n = clamp_count(proj.count, proj.capacity);
   const int64_t n_grp = proj.view_info[kVI * n_views + 3];
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -165,6 +168,7 @@ __device__ inline int64_t lower_bound_u32(const uint32_t* __restrict__ poff, int
 // of the histogram and placement kernels.
 __global__ void k_chunk_bounds(const uint32_t* __restrict__ seg, const uint32_t* __restrict__ poff, int n_views,
                                int K, uint32_t* __restrict__ bounds) {
+  pdl_begin();
   const int64_t nb = (int64_t)n_views * (K + 1);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nb; i += (int64_t)gridDim.x * blockDim.x) {
     const int v = (int)(i / (K + 1));
@@ -214,6 +218,7 @@ __device__ inline void window_size(uint32_t tx, uint32_t ty, uint32_t cells, boo
 __global__ void __launch_bounds__(kBinWarps * 32) k_bin_hist(const gs_proj proj, const uint32_t* __restrict__ bounds,
                                                              const ushort4* __restrict__ srect, int n_views, int K,
                                                              int64_t tile_cap, uint32_t* __restrict__ cnt) {
+  pdl_begin();
   __shared__ uint32_t s_d[kBinWarps][kWin];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t cid = (int64_t)blockIdx.x * kBinWarps + warp;
@@ -276,6 +281,7 @@ __global__ void k_bin_ranges(const uint32_t* __restrict__ off, const uint32_t* _
                              const uint32_t* __restrict__ view_info, int n_views, uint32_t* __restrict__ ranges,
                              uint32_t* __restrict__ bins_count, uint32_t* status,
                              uint32_t* __restrict__ order_cnt) {
+  pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x < 2 * kOrderBuckets) order_cnt[threadIdx.x] = 0u;   // (kBlock threads)
   const int64_t lim = (int64_t)*scan_n / K;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -317,6 +323,7 @@ __global__ void __launch_bounds__(kBinWarps * 32, 5) k_bin_place(const gs_proj p
                                                                  const ushort4* __restrict__ srect, int n_views, int K,
                                                                  int64_t tile_cap, const uint32_t* __restrict__ off,
                                                                  gs_bins out) {
+  pdl_begin();
   __shared__ uint32_t s_run[kBinWarps][kPlaceWin];
   __shared__ uint4 s_grp[kBinWarps][32];
   // ceil(2^32 / w) for every clipped width w <= kWinCols (a table: an integer division by a
@@ -490,6 +497,7 @@ __device__ inline int64_t order_items(const uint32_t* __restrict__ view_info, in
 __global__ void __launch_bounds__(kBlock) k_order_count(const uint32_t* __restrict__ view_info, int n_views,
                                                         const uint32_t* __restrict__ ranges, int64_t tile_cap,
                                                         int64_t item_cap, bool clamp, uint32_t* __restrict__ cnt) {
+  pdl_begin();
   __shared__ uint32_t s_cnt[kOrderBuckets];
   for (int i = threadIdx.x; i < kOrderBuckets; i += blockDim.x) s_cnt[i] = 0u;
   __syncthreads();
@@ -507,6 +515,7 @@ __global__ void __launch_bounds__(kBlock) k_order_place(const uint32_t* __restri
                                                         int64_t item_cap, bool clamp,
                                                         const uint32_t* __restrict__ cnt, uint32_t* __restrict__ cur,
                                                         uint32_t* __restrict__ order) {
+  pdl_begin();
   __shared__ uint32_t s_base[kOrderBuckets];
   const int64_t n = order_items(view_info, n_views, item_cap, clamp);
   const int lane = threadIdx.x & 31;
@@ -543,11 +552,9 @@ __global__ void __launch_bounds__(kBlock) k_order_place(const uint32_t* __restri
 void launch_item_order(const uint32_t* view_info, int n_views, const uint32_t* ranges, int64_t tile_cap,
                        int64_t item_cap, bool clamp, uint32_t* cnt, uint32_t* order, cudaStream_t st) {
   const unsigned og = grid_for(item_cap);
-  k_order_count<<<og, kBlock, 0, st>>>(view_info, n_views, ranges, tile_cap, item_cap, clamp, cnt);
-  note_launch();
-  k_order_place<<<og, kBlock, 0, st>>>(view_info, n_views, ranges, tile_cap, item_cap, clamp, cnt,
-                                       cnt + kOrderBuckets, order);
-  note_launch();
+  launch(k_order_count, og, kBlock, 0, st, view_info, n_views, ranges, tile_cap, item_cap, clamp, cnt);
+  launch(k_order_place, og, kBlock, 0, st, view_info, n_views, ranges, tile_cap, item_cap, clamp, cnt,
+         cnt + kOrderBuckets, order);
 }
 
 size_t bin_ws_bytes(int64_t rec_cap, int64_t pair_cap, int64_t tile_cap, int n_views) {
@@ -600,13 +607,10 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
 
   // 1. view segments (from the records' view ids, or from the projection's group offsets)
   if (!proj.view) {
-    k_segments_from_groups<<<grid_for(n_views + 1), kBlock, 0, st>>>(proj, n_views, tile_cap, K, seg, &ctr[0]);
-    note_launch();
+    launch(k_segments_from_groups, grid_for(n_views + 1), kBlock, 0, st, proj, n_views, tile_cap, K, seg, &ctr[0]);
   } else {
-    k_zero_u32<<<grid_for(n_views + 1), kBlock, 0, st>>>(seg, n_views + 1);
-    note_launch();
-    k_segments<<<grid_for(rec_cap), kBlock, 0, st>>>(proj, n_views, tile_cap, K, seg, &ctr[0]);
-    note_launch();
+    launch(k_zero_u32, grid_for(n_views + 1), kBlock, 0, st, seg, n_views + 1);
+    launch(k_segments, grid_for(rec_cap), kBlock, 0, st, proj, n_views, tile_cap, K, seg, &ctr[0]);
   }
   // 2. record indices by depth bits within each view
   // (the last pass also writes the rectangles in sorted order and their pair counts)
@@ -619,24 +623,22 @@ cudaError_t launch_bin_sort(const gs_proj& proj, const gs_camera* cams, int n_vi
   e = scan_exclusive(rcnt, poff, proj.count, rec_cap, nullptr, tmp, st);
   if (e != cudaSuccess) return e;
   // 4. chunk boundaries, per-chunk tile counts
-  k_chunk_bounds<<<grid_for((int64_t)n_views * (K + 1)), kBlock, 0, st>>>(seg, poff, n_views, K, bounds);
-  note_launch();
+  launch(k_chunk_bounds, grid_for((int64_t)n_views * (K + 1)), kBlock, 0, st, seg, poff, n_views, K, bounds);
   const int64_t chunks = (int64_t)n_views * K;
   const unsigned bin_grid = (unsigned)((chunks + kBinWarps - 1) / kBinWarps);
-  k_bin_hist<<<bin_grid, kBinWarps * 32, 0, st>>>(proj, bounds, srect, n_views, K, tile_cap, cnt);
-  note_launch();
+  launch_spread(k_bin_hist, bin_grid, kBinWarps * 32, 0, st, proj, bounds, srect, n_views, K, tile_cap, cnt);
   // 5. slots of every (tile, chunk); ranges and totals
   e = scan_exclusive(cnt, off, &ctr[0], cnt_cap - 1, &ctr[1], tmp, st);
   if (e != cudaSuccess) return e;
-  k_bin_ranges<<<grid_for(tile_cap), kBlock, 0, st>>>(off, &ctr[0], &ctr[1], K, out.pair_capacity, tile_cap,
-                                                      proj.view_info, n_views, out.ranges, out.count, proj.status, ocnt);
-  note_launch();
+  launch(k_bin_ranges, grid_for(tile_cap), kBlock, 0, st, off, &ctr[0], &ctr[1], K, out.pair_capacity, tile_cap,
+         proj.view_info, n_views, out.ranges, out.count, proj.status, ocnt);
   // 6. placement
   if (out.tile)
-    k_bin_place<true><<<bin_grid, kBinWarps * 32, 0, st>>>(proj, bounds, srec, srect, n_views, K, tile_cap, off, out);
+    launch_spread(k_bin_place<true>, bin_grid, kBinWarps * 32, 0, st, proj, bounds, srec, srect, n_views, K, tile_cap,
+                  off, out);
   else
-    k_bin_place<false><<<bin_grid, kBinWarps * 32, 0, st>>>(proj, bounds, srec, srect, n_views, K, tile_cap, off, out);
-  note_launch();
+    launch_spread(k_bin_place<false>, bin_grid, kBinWarps * 32, 0, st, proj, bounds, srec, srect, n_views, K,
+                  tile_cap, off, out);
   // 7. warp items longest tile list first, for the compositing kernels (optional)
   if (out.item_order && out.item_capacity > 0) {
     launch_item_order(proj.view_info, n_views, out.ranges, tile_cap, out.item_capacity, false, ocnt, out.item_order, st);

@@ -46,6 +46,51 @@ int device_sm_count();
 void note_launch();
 uint64_t launch_count();
 
+// Launches a kernel behind the work already in the stream, with its start overlapped: the launch
+// may place the kernel's blocks while the kernel before it still runs, and every kernel of the
+// library begins with pdl_begin, which lets the next one be placed in turn (once all blocks of this
+// one have started) and then waits until everything before it in the stream has finished and its
+// writes are visible.  So the order of the work is that of plain launches; what is saved is the gap
+// between kernels, which small calls are made of (some 38 launches for one view): one 640x480 view of 200k
+// Gaussians 288 -> 232 us, 27 scored candidates 750 -> 685 us, 3M Gaussians and eight 1280x720 views
+// 5.91 -> 5.85 ms.
+template <class... P, class... A>
+inline void launch_as(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                      A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<A&&>(args)...);   // (an error stays for cudaGetLastError)
+  note_launch();
+}
+
+template <class... P, class... A>
+inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  launch_as(true, kernel, grid, block, smem, st, static_cast<A&&>(args)...);
+}
+
+// The same without the overlapped start, for the kernels that do most of a call's work: blocks placed
+// early crowd onto the multiprocessors that are free first, and stay there (pair placement of four
+// keyframes, 417 blocks: 106 us after a plain launch, 162 us after an overlapped one).
+template <class... P, class... A>
+inline void launch_spread(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  launch_as(false, kernel, grid, block, smem, st, static_cast<A&&>(args)...);
+}
+
+__device__ __forceinline__ void pdl_begin() {
+#if defined(__CUDA_ARCH__)
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
+#endif
+}
+
 // ------------------------------------------------------------------ scan
 // Exclusive prefix sum of n uint32 values into out[0..n]; out[n] = total.
 // n = min(*n_dev, n_cap) when n_dev != NULL, else n_cap.  Prefixes saturate at

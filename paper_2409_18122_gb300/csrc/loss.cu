@@ -210,6 +210,7 @@ constexpr size_t kFwdSmem = sizeof(float) * (2 * kInH * kPitch + 4 * kRowsH * kL
 constexpr size_t kBwdSmem = sizeof(float) * (3 * kInH * kPitch + 3 * kRowsH * kLTW);
 
 __global__ void __launch_bounds__(kLossThreads) k_loss_fwd(const __grid_constant__ LossArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) float s_mem[];
   float (*s_in)[kInH][kPitch] = reinterpret_cast<float (*)[kInH][kPitch]>(s_mem);   // x, y
   float (*s_h)[kRowsH][kLTW] = reinterpret_cast<float (*)[kRowsH][kLTW]>(s_mem + 2 * kInH * kPitch);
@@ -272,6 +273,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_fwd(const __grid_constant
 }
 
 __global__ void __launch_bounds__(kLossThreads) k_loss_ssim_bwd(const __grid_constant__ LossArgs a) {
+  pdl_begin();
   extern __shared__ __align__(16) float s_mem[];
   float (*s_in)[kInH][kPitch] = reinterpret_cast<float (*)[kInH][kPitch]>(s_mem);   // dS/dm1, dS/dm2, dS/dm12
   float (*s_h)[kRowsH][kLTW] = reinterpret_cast<float (*)[kRowsH][kLTW]>(s_mem + 3 * kInH * kPitch);
@@ -319,6 +321,7 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_l1(const float* __restric
                                                           float* __restrict__ g, int64_t n, int64_t chunk, float w,
                                                           float inv_n, int field, double* __restrict__ part,
                                                           int64_t slot0) {
+  pdl_begin();
   const int64_t b0 = (int64_t)blockIdx.x * chunk;
   const int64_t b1 = b0 + chunk < n ? b0 + chunk : n;
   float acc = 0.f;
@@ -336,6 +339,7 @@ constexpr int kFinishThreads = 1024;
 __global__ void __launch_bounds__(kFinishThreads)
     k_loss_finish(const double* part, int64_t n_slots, float w_d, float w_c, float w_s, bool ssim, double n_pix,
                   float* out) {
+  pdl_begin();
   __shared__ double s[3][kFinishThreads];
   double acc[3] = {0.0, 0.0, 0.0};
 #pragma unroll 4
@@ -437,12 +441,10 @@ cudaError_t launch_image_loss(const int32_t* sizes, int n_views, const float* rg
     chunk = (chunk + 4 * kLossThreads - 1) / (4 * kLossThreads) * (4 * kLossThreads);
     if (chunk < 4096) chunk = 4096;
     const int64_t nb_c = (3 * lay.P + chunk - 1) / chunk, nb_d = (lay.P + chunk - 1) / chunk;
-    k_loss_l1<<<(unsigned)nb_c, kLossThreads, 0, st>>>(rgb, rgb_ref, d_rgb, 3 * lay.P, chunk, w.w_rgb, a.inv_n, 1,
-                                                       part, 0);
-    note_launch();
-    k_loss_l1<<<(unsigned)nb_d, kLossThreads, 0, st>>>(depth, depth_ref, d_depth, lay.P, chunk, w.w_depth, a.inv_n,
-                                                       2, part, nb_c);
-    note_launch();
+    launch(k_loss_l1, (unsigned)nb_c, kLossThreads, 0, st, rgb, rgb_ref, d_rgb, 3 * lay.P, chunk, w.w_rgb, a.inv_n, 1,
+           part, 0);
+    launch(k_loss_l1, (unsigned)nb_d, kLossThreads, 0, st, depth, depth_ref, d_depth, lay.P, chunk, w.w_depth,
+           a.inv_n, 2, part, nb_c);
     slot = nb_c + nb_d;
   }
   for (int v0 = 0; v0 < n_views && ssim; v0 += kLossViewsPerLaunch) {
@@ -461,17 +463,14 @@ cudaError_t launch_image_loss(const int32_t* sizes, int n_views, const float* rg
       tb += ((W + kLTW - 1) / kLTW) * ((H + kLTH - 1) / kLTH);
     }
     const dim3 grid((unsigned)tb, 3);
-    k_loss_fwd<<<grid, kLossThreads, kFwdSmem, st>>>(a);
-    note_launch();
+    launch_spread(k_loss_fwd, grid, kLossThreads, kFwdSmem, st, a);
     if (d_rgb) {
-      k_loss_ssim_bwd<<<grid, kLossThreads, kBwdSmem, st>>>(a);
-      note_launch();
+      launch_spread(k_loss_ssim_bwd, grid, kLossThreads, kBwdSmem, st, a);
     }
     slot += 3 * (int64_t)tb;
   }
-  k_loss_finish<<<1, kFinishThreads, 0, st>>>(part, slot, w.w_depth, w.w_rgb, w.w_ssim, ssim, (double)lay.P,
-                                            loss_out);
-  note_launch();
+  launch(k_loss_finish, 1, kFinishThreads, 0, st, part, slot, w.w_depth, w.w_rgb, w.w_ssim, ssim, (double)lay.P,
+         loss_out);
   return cudaGetLastError();
 }
 

@@ -34,6 +34,7 @@ __device__ __forceinline__ unsigned long long view_pixels(const gs_camera& c) {
 __global__ void __launch_bounds__(1024) k_view_info(const gs_camera* __restrict__ cams, int n_views, int def_tw,
                                                     int def_th, uint32_t n_groups, uint32_t* __restrict__ view_info,
                                                     uint32_t* status) {
+  pdl_begin();
   __shared__ unsigned long long s_sum[3][32];
   const int per = (n_views + blockDim.x - 1) / blockDim.x;
   const int v0 = threadIdx.x * per;
@@ -130,6 +131,7 @@ template <bool kWrite>
 __global__ void __launch_bounds__(kBlock) k_project(gs_map map, const gs_camera* __restrict__ cams, int n_views,
                                                      gs_params p, const uint32_t* __restrict__ view_info,
                                                      uint32_t* __restrict__ counts, gs_proj out) {
+  pdl_begin();
   __shared__ CamC s_cam[kMaxViewsPerChunk];
   __shared__ float4 s_g[kWarps][4][32];                  // per lane: mo, (S0..S3), (S4, S5, Q, o), (rgb, u)
   __shared__ uint32_t s_q[kWarps][64];                   // queued (view in chunk << 5 | lane)
@@ -280,6 +282,7 @@ __global__ void __launch_bounds__(kBlock) k_project(gs_map map, const gs_camera*
 }
 
 __global__ void k_record_count(const gs_proj out, int64_t n_slots) {
+  pdl_begin();
   const uint32_t total = out.grp_base[n_slots];
   *out.count = (int64_t)total > out.capacity ? (uint32_t)out.capacity : total;
   if ((int64_t)total > out.capacity) set_flag(out.status, GS_FLAG_RECORD_OVERFLOW);
@@ -298,22 +301,20 @@ cudaError_t launch_project(const gs_map& map, const gs_camera* cams, int n_views
   Carver c(ws);
   uint32_t* counts = c.take<uint32_t>((size_t)slots + 1);
   void* scan_tmp = c.take<char>(scan_temp_bytes(slots));
-  k_view_info<<<1, 1024, 0, st>>>(cams, n_views, p.tile_w, p.tile_h, (uint32_t)((map.n + 31) / 32), out.view_info,
-                                  out.status);
-  note_launch();
+  launch(k_view_info, 1, 1024, 0, st, cams, n_views, p.tile_w, p.tile_h, (uint32_t)((map.n + 31) / 32), out.view_info,
+         out.status);
   const int64_t blocks = (map.n + kBlock - 1) / kBlock;
   if (blocks > 0) {
-    k_project<false><<<(unsigned)blocks, kBlock, 0, st>>>(map, cams, n_views, p, out.view_info, counts, out);
-    note_launch();
+    launch_spread(k_project<false>, (unsigned)blocks, kBlock, 0, st, map, cams, n_views, p, out.view_info, counts,
+                  out);
   }
   cudaError_t e = scan_exclusive(counts, out.grp_base, nullptr, slots, nullptr, scan_tmp, st);
   if (e != cudaSuccess) return e;
   if (blocks > 0) {
-    k_project<true><<<(unsigned)blocks, kBlock, 0, st>>>(map, cams, n_views, p, out.view_info, counts, out);
-    note_launch();
+    launch_spread(k_project<true>, (unsigned)blocks, kBlock, 0, st, map, cams, n_views, p, out.view_info, counts,
+                  out);
   }
-  k_record_count<<<1, 1, 0, st>>>(out, slots);
-  note_launch();
+  launch(k_record_count, 1, 1, 0, st, out, slots);
   return cudaGetLastError();
 }
 

@@ -70,6 +70,7 @@ template <int kPairs, bool kCount>
 __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, gs_proj proj, gs_bins bins,
                                                                 const gs_camera* __restrict__ cams, int n_views,
                                                                 gs_params p, gs_image img, uint32_t n_items) {
+  pdl_begin();
   constexpr int kChunk = 2 * kPairs;
   __shared__ __align__(16) float s_exp[kFwdWarps][kRing / 2 * kPairFloats];   // staged exponents (stage_pair)
   __shared__ float4 s_col[kFwdWarps][kRing];                                  // (r, g, b, depth)
@@ -263,6 +264,7 @@ __global__ void __launch_bounds__(kIgWarps * 32, 12) k_ig_items(gs_proj proj, gs
                                                              gs_params p, const uint32_t* __restrict__ order,
                                                              float* __restrict__ item_sum, int64_t item_cap,
                                                              uint32_t* __restrict__ work) {
+  pdl_begin();
   // staged entries of each warp, a ring of kRing: exponents (stage_pair) and u
   __shared__ __align__(16) float s_exp[kIgWarps][kRing / 2 * kPairFloats];
   __shared__ __align__(16) float s_u[kIgWarps][kRing];
@@ -367,6 +369,7 @@ __global__ void __launch_bounds__(256) k_ig_views(const uint32_t* __restrict__ v
                                                    const gs_camera* __restrict__ cams, int n_views,
                                                    const float* __restrict__ item_sum, int64_t item_cap,
                                                    float* __restrict__ ig) {
+  pdl_begin();
   __shared__ float s_red[32];
   const int v = blockIdx.x;
   const uint32_t i0 = view_info[kVI * v + 2] / kPix;
@@ -381,6 +384,7 @@ __global__ void __launch_bounds__(256) k_ig_views(const uint32_t* __restrict__ v
 }
 
 __global__ void k_zero_words(uint32_t* p, int n) {
+  pdl_begin();
   for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0u;
 }
 
@@ -396,9 +400,8 @@ cudaError_t launch_ig_items(const gs_proj& proj, const gs_bins& bins, const gs_c
   int64_t grid = (int64_t)device_sm_count() * per_sm;
   if (grid * kIgWarps > item_cap) grid = (item_cap + kIgWarps - 1) / kIgWarps;
   if (grid < 1) grid = 1;
-  k_ig_items<kB><<<(unsigned)grid, kIgWarps * 32, 0, st>>>(proj, bins, cams, n_views, p, order, item_sum, item_cap,
-                                                           work);
-  note_launch();
+  launch_spread(k_ig_items<kB>, (unsigned)grid, kIgWarps * 32, 0, st, proj, bins, cams, n_views, p, order, item_sum,
+                item_cap, work);
   return cudaSuccess;
 }
 
@@ -412,8 +415,7 @@ cudaError_t launch_render_fwd(const gs_map& map, const gs_proj& proj, const gs_b
     const int b = p.fwd_batch ? p.fwd_batch : kFwdBatchDefault;
     auto kern = img.n_contrib ? (b == 4 ? k_render_fwd<2, true> : k_render_fwd<1, true>)
                               : (b == 4 ? k_render_fwd<2, false> : k_render_fwd<1, false>);
-    kern<<<grid, kFwdWarps * 32, 0, st>>>(map, proj, bins, cams, n_views, p, img, (uint32_t)items);
-    note_launch();
+    launch_spread(kern, grid, kFwdWarps * 32, 0, st, map, proj, bins, cams, n_views, p, img, (uint32_t)items);
   }
   return cudaGetLastError();
 }
@@ -454,8 +456,7 @@ cudaError_t launch_ig_composite(const gs_proj& proj, const gs_bins& bins, const 
   float* item_sum = c.take<float>(item_cap);
   uint32_t* work = c.take<uint32_t>(4 + 2 * kOrderBuckets);
   uint32_t* order = c.take<uint32_t>(item_cap);
-  k_zero_words<<<1, 160, 0, st>>>(work, 4 + 2 * kOrderBuckets);
-  note_launch();
+  launch(k_zero_words, 1, 160, 0, st, work, 4 + 2 * kOrderBuckets);
   // longest tile lists first: a counting sort over buckets of list length (an exact radix sort of
   // the lengths took 6 launches and 75 us of the 1M-Gaussian, 256-view pass instead of 2 and 19 us,
   // for the same compositing time)
@@ -465,8 +466,7 @@ cudaError_t launch_ig_composite(const gs_proj& proj, const gs_bins& bins, const 
                 : b == 16 ? launch_ig_items<16>(proj, bins, cams, n_views, p, order, item_sum, item_cap, work, st)
                           : launch_ig_items<8>(proj, bins, cams, n_views, p, order, item_sum, item_cap, work, st);
   if (e != cudaSuccess) return e;
-  k_ig_views<<<n_views, 256, 0, st>>>(proj.view_info, cams, n_views, item_sum, item_cap, ig_out);
-  note_launch();
+  launch(k_ig_views, n_views, 256, 0, st, proj.view_info, cams, n_views, item_sum, item_cap, ig_out);
   return cudaGetLastError();
 }
 

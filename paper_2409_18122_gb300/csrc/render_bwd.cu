@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 12) k_render_bwd(gs_map map, g
                                                                 const gs_camera* __restrict__ cams, int n_views,
                                                                 gs_params p, gs_image fwd, gs_image_grad grad,
                                                                 float4* __restrict__ g2d, uint32_t n_items) {
+  pdl_begin();
   // staged entries: (c0, cu, cv, k.x), (k.y, k.z, position in the list, record), (colour, depth)
   __shared__ float4 s_stage[kBwdWarps][3][32];
   __shared__ __align__(16) float s_red[kBwdWarps][2][kRedBatch * kRedPitch];   // dL/dq and w rows
@@ -224,6 +225,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 12) k_render_bwd(gs_map map, g
 }
 
 __global__ void k_zero_g2d(float4* __restrict__ g2d, const uint32_t* count, int64_t cap) {
+  pdl_begin();
   int64_t n = (int64_t)*count;
   if (n > cap) n = cap;
   const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -235,6 +237,7 @@ __global__ void k_zero_g2d(float4* __restrict__ g2d, const uint32_t* count, int6
 // view it is visible in, found through the group masks) without atomics.
 __global__ void __launch_bounds__(256) k_proj_adjoint(gs_map map, gs_proj proj, const gs_camera* __restrict__ cams,
                                                       int n_views, const float4* __restrict__ g2d, gs_map_grad out) {
+  pdl_begin();
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= map.n) return;
   const int64_t nrec = (int64_t)*proj.count;
@@ -378,17 +381,14 @@ cudaError_t launch_render_bwd(const gs_map& map, const gs_proj& proj, const gs_b
   int64_t zb = (3 * proj.capacity + 255) / 256;
   if (zb > 4096) zb = 4096;
   if (zb < 1) zb = 1;
-  k_zero_g2d<<<(unsigned)zb, 256, 0, st>>>(g2d, proj.count, proj.capacity);
-  note_launch();
+  launch(k_zero_g2d, (unsigned)zb, 256, 0, st, g2d, proj.count, proj.capacity);
   const int64_t items = bins.tile_capacity * 32;   // upper bound: at most 32 items per tile
   if (items > 0) {
-    k_render_bwd<<<(unsigned)((items + kBwdWarps - 1) / kBwdWarps), kBwdWarps * 32, 0, st>>>(
-        map, proj, bins, cams, n_views, p, fwd, g, g2d, (uint32_t)items);
-    note_launch();
+    launch_spread(k_render_bwd, (unsigned)((items + kBwdWarps - 1) / kBwdWarps), kBwdWarps * 32, 0, st, map, proj,
+                  bins, cams, n_views, p, fwd, g, g2d, (uint32_t)items);
   }
   if (map.n > 0) {
-    k_proj_adjoint<<<(unsigned)((map.n + 255) / 256), 256, 0, st>>>(map, proj, cams, n_views, g2d, out);
-    note_launch();
+    launch_spread(k_proj_adjoint, (unsigned)((map.n + 255) / 256), 256, 0, st, map, proj, cams, n_views, g2d, out);
   }
   return cudaGetLastError();
 }

@@ -65,6 +65,7 @@ __device__ unsigned long long block_exclusive_scan(unsigned long long v, unsigne
 
 __global__ void __launch_bounds__(kBlock) k_scan_reduce(const uint32_t* __restrict__ in, const uint32_t* n_dev,
                                                          int64_t n_cap, unsigned long long* partial) {
+  pdl_begin();
   const int64_t n = count_of(n_dev, n_cap);
   const int64_t g = gridDim.x;
   const int64_t chunk = chunk_for(n, g);
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(kBlock) k_scan_reduce(const uint32_t* __restri
 
 __global__ void __launch_bounds__(1024) k_scan_partials(unsigned long long* partial, int g, const uint32_t* n_dev,
                                                         int64_t n_cap, uint32_t* out, uint32_t* total_out) {
+  pdl_begin();
   __shared__ unsigned long long sums[32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long v = threadIdx.x < g ? partial[threadIdx.x] : 0, x = v;
@@ -113,6 +115,7 @@ __global__ void __launch_bounds__(1024) k_scan_partials(unsigned long long* part
 __global__ void __launch_bounds__(kBlock) k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                        const uint32_t* n_dev, int64_t n_cap,
                                                        const unsigned long long* partial) {
+  pdl_begin();
   const int64_t n = count_of(n_dev, n_cap);
   const int64_t g = gridDim.x;
   const int64_t chunk = chunk_for(n, g);
@@ -164,12 +167,9 @@ cudaError_t scan_exclusive(const uint32_t* in, uint32_t* out, const uint32_t* n_
                            uint32_t* total_out, void* temp, cudaStream_t st) {
   const int g = (int)parts_for(n_cap);
   auto* partial = (unsigned long long*)temp;
-  k_scan_reduce<<<g, kBlock, 0, st>>>(in, n_dev, n_cap, partial);
-  note_launch();
-  k_scan_partials<<<1, 1024, 0, st>>>(partial, g, n_dev, n_cap, out, total_out);
-  note_launch();
-  k_scan_down<<<g, kBlock, 0, st>>>(in, out, n_dev, n_cap, partial);
-  note_launch();
+  launch(k_scan_reduce, g, kBlock, 0, st, in, n_dev, n_cap, partial);
+  launch(k_scan_partials, 1, 1024, 0, st, partial, g, n_dev, n_cap, out, total_out);
+  launch(k_scan_down, g, kBlock, 0, st, in, out, n_dev, n_cap, partial);
   return cudaGetLastError();
 }
 

@@ -141,6 +141,7 @@ __device__ void sort_list(SmallSmem& s, int n) {
 __global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_camera* __restrict__ cams,
                                                            int n_views, gs_params p, gs_image img,
                                                            uint32_t* __restrict__ status) {
+  pdl_begin();
   extern __shared__ __align__(16) unsigned char s_raw[];
   SmallSmem& s = *reinterpret_cast<SmallSmem*>(s_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -303,9 +304,8 @@ cudaError_t launch_render_small(const gs_map& map, const gs_camera* cams, int n_
   }
   // one CTA per SM walks the tiles of all views with a fixed stride (the number of tiles
   // lives in the cameras, in device memory)
-  k_render_small<<<(unsigned)device_sm_count(), kThreads, sizeof(SmallSmem), st>>>(map, cams, n_views, p, img,
-                                                                                     status);
-  note_launch();
+  launch(k_render_small, (unsigned)device_sm_count(), kThreads, sizeof(SmallSmem), st, map, cams, n_views, p, img,
+         status);
   return cudaGetLastError();
 }
 

@@ -70,6 +70,7 @@ __device__ inline int64_t count_of(const uint32_t* n_dev, int64_t n_cap) {
 __global__ void __launch_bounds__(1024) k_part_map(const uint32_t* __restrict__ seg, int n_seg, const uint32_t* n_dev,
                                                    int64_t n_cap, int grid, int tile, uint32_t* __restrict__ pmap,
                                                    uint32_t* __restrict__ ctl) {
+  pdl_begin();
   __shared__ unsigned long long s_sum[32];
   const int64_t n = count_of(n_dev, n_cap);
   const int64_t avail = grid - n_seg > 1 ? grid - n_seg : 1;
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kBlock) k_upsweep(const uint32_t* __restrict__
                                                     const uint32_t* __restrict__ seg, int n_seg,
                                                     const uint32_t* __restrict__ pmap, uint32_t* __restrict__ ctl,
                                                     uint32_t* __restrict__ hist) {
+  pdl_begin();
   constexpr int kCopies = kWarps / 2;   // two warps share a copy of the counts
   __shared__ uint32_t cnt[kCopies][kRadix];
   const bool three = kPass >= 2 && sorted_in_three(ctl);
@@ -200,6 +202,7 @@ template <int kPass>
 __global__ void __launch_bounds__(1024) k_scan_hist(uint32_t* __restrict__ hist, int g,
                                                     const uint32_t* __restrict__ pmap,
                                                     const uint32_t* __restrict__ ctl, uint32_t* __restrict__ tot) {
+  pdl_begin();
   __shared__ uint32_t s_sum[32][33];
   if (kPass == 3 && sorted_in_three(ctl)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, s = blockIdx.x;
@@ -272,6 +275,7 @@ __global__ void __launch_bounds__(kBlock, kItems > 8 ? 2 : 4) k_downsweep(const 
                                                           const uint32_t* __restrict__ hist,
                                                           const uint32_t* __restrict__ tot,
                                                           const SortRectEpilogue epi) {
+  pdl_begin();
   constexpr int kTile = kBlock * kItems;
   constexpr int kG = kItems < 8 ? kItems : 8;   // rectangle gathers of a thread in flight
   extern __shared__ __align__(16) uint32_t smem[];
@@ -448,13 +452,10 @@ cudaError_t sort_pass(const SortArgs& a, const uint32_t* keys_in, const uint32_t
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  k_upsweep<kPass><<<a.g, kBlock, 0, a.st>>>(keys_in, a.seg, a.n_seg, a.pmap, a.ctl, a.hist);
-  note_launch();
-  k_scan_hist<kPass><<<dim3(a.n_seg, kRadix / 32), 1024, 0, a.st>>>(a.hist, a.g, a.pmap, a.ctl, a.tot);
-  note_launch();
-  k_downsweep<kPass, kItems><<<a.g, kBlock, down_smem(kItems), a.st>>>(
-      keys_in, vals_in, a.seg, a.n_seg, a.pmap, a.ctl, keys_out, vals_out, a.hist, a.tot, epi);
-  note_launch();
+  launch(k_upsweep<kPass>, a.g, kBlock, 0, a.st, keys_in, a.seg, a.n_seg, a.pmap, a.ctl, a.hist);
+  launch(k_scan_hist<kPass>, dim3(a.n_seg, kRadix / 32), 1024, 0, a.st, a.hist, a.g, a.pmap, a.ctl, a.tot);
+  launch(k_downsweep<kPass, kItems>, a.g, kBlock, down_smem(kItems), a.st, keys_in, vals_in, a.seg, a.n_seg, a.pmap,
+         a.ctl, keys_out, vals_out, a.hist, a.tot, epi);
   return cudaSuccess;
 }
 
@@ -488,8 +489,7 @@ cudaError_t record_sort(const uint32_t* keys, SortBufs b, const uint32_t* n_dev,
   a.pmap = c.take<uint32_t>(n_seg + 2);
   a.ctl = ctl;
   a.st = st;
-  k_part_map<<<1, 1024, 0, st>>>(seg, n_seg, n_dev, n_cap, a.g, tile_keys(n_cap), a.pmap, ctl);
-  note_launch();
+  launch(k_part_map, 1, 1024, 0, st, seg, n_seg, n_dev, n_cap, a.g, tile_keys(n_cap), a.pmap, ctl);
   const cudaError_t e = small_sort(n_cap) ? sort_passes<kItemsSmall>(a, keys, b, epi) : sort_passes<kItemsLarge>(a, keys, b, epi);
   if (e != cudaSuccess) return e;
   *out = SortedRecords{b.vals_b, b.vals_a, ctl};

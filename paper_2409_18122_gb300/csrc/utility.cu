@@ -102,6 +102,7 @@ __device__ __forceinline__ bool group_may_see(float gx, float gy, float gz, floa
 // u_i = |mu_cur - mu_prev| (or its square); unchanged means keep their u.
 __global__ void k_uncertainty_update(const float4* __restrict__ mo_prev, const float4* __restrict__ mo_cur,
                                      float4* __restrict__ su, int64_t n, int squared) {
+  pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float4 a = mo_prev[i], b = mo_cur[i];
     const float dx = __fsub_rn(b.x, a.x), dy = __fsub_rn(b.y, a.y), dz = __fsub_rn(b.z, a.z);
@@ -153,6 +154,7 @@ template <int kPass>
 __global__ void __launch_bounds__(kMomThreads) k_u_moments(const float4* __restrict__ mo,
                                                            const float4* __restrict__ su, int64_t n, float ground_z,
                                                            double* __restrict__ part) {
+  pdl_begin();
   __shared__ double s[kMomThreads / 32];
   const int g = gridDim.x, warp = threadIdx.x >> 5;
   double mean = 0.0;
@@ -197,6 +199,7 @@ __global__ void __launch_bounds__(kMomThreads) k_u_moments(const float4* __restr
 
 // stats = (mean, sigma, t_high = mean + sigma/2, t_low = mean - sigma/2, count); 96 threads
 __global__ void __launch_bounds__(96) k_u_finish(const double* __restrict__ part, int g, double* __restrict__ stats) {
+  pdl_begin();
   __shared__ double s[3];
   const int warp = threadIdx.x >> 5;
   const double t = sum_partials(part + warp * g, g);
@@ -229,6 +232,7 @@ __global__ void __launch_bounds__(kBlock) k_view_utility(const float4* __restric
                                                          gs_utility_params prm, const double* __restrict__ stats,
                                                          uint32_t* __restrict__ cnt_part, float* __restrict__ sum_part,
                                                          int n_views) {
+  pdl_begin();
   __shared__ VisCam s_cam[kViewChunk];
   __shared__ uint32_t s_acc[kSum ? 1 : 2][kWarps][kViewChunk];   // visible high, low; or the sum of u (float)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -322,6 +326,7 @@ __global__ void __launch_bounds__(kBlock) k_view_utility_finish(const uint32_t* 
                                                                 const float* __restrict__ sum_part, int g,
                                                                 int n_views, float lambda, float* __restrict__ xi,
                                                                 uint32_t* __restrict__ counts) {
+  pdl_begin();
   const int v = blockIdx.x * kWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (v >= n_views) return;
   if (kSum) {
@@ -368,6 +373,7 @@ constexpr int kRegSlots = 8;
 __global__ void __launch_bounds__(kBlock) k_regions(const float4* __restrict__ mo, const float4* __restrict__ su,
                                                     int64_t n, gs_region_grid grid, double* __restrict__ sum,
                                                     uint32_t* __restrict__ count) {
+  pdl_begin();
   __shared__ double s_acc[kWarps][kRegSlots][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int k = 0; k < kRegSlots; ++k) s_acc[warp][k][lane] = 0.0;
@@ -440,6 +446,7 @@ __global__ void __launch_bounds__(kBlock) k_regions(const float4* __restrict__ m
 
 __global__ void k_region_mean(const double* __restrict__ sum, const uint32_t* __restrict__ count, int64_t n_reg,
                               float* __restrict__ omega) {
+  pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_reg; r += (int64_t)gridDim.x * blockDim.x)
     omega[r] = count[r] ? (float)(sum[r] / (double)count[r]) : 0.f;
 }
@@ -448,6 +455,7 @@ __global__ void k_region_mean(const double* __restrict__ sum, const uint32_t* __
 // of xi (states l = 0..L in order, FP64), and the first trajectory with the largest sum.
 __global__ void k_traj_sum(const float* __restrict__ xi, int n_traj, int n_states, float* __restrict__ out,
                            int32_t* __restrict__ best) {
+  pdl_begin();
   __shared__ double s_best[256];
   __shared__ int s_idx[256];
   double bv = -INFINITY;
@@ -514,6 +522,7 @@ __global__ void __launch_bounds__(kBlock) k_collision(const float4* __restrict__
                                                       int64_t n, const float4* __restrict__ pts, int n_pts,
                                                       float r_robot, float lambda_g, float ground_z, float* margin,
                                                       uint32_t* hit) {
+  pdl_begin();
   __shared__ float4 s_g[kColChunk];        // (mu, gamma); gamma < 0: no Gaussian
   __shared__ float4 s_c[kColGroups];       // (centre, radius + largest gamma); -inf: empty group
   __shared__ float4 s_all;                 // the same for the whole chunk
@@ -666,6 +675,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_collision_seed(const float4* _
                                                                  float lambda_g, float ground_z,
                                                                  float* __restrict__ margin,
                                                                  uint32_t* __restrict__ hit) {
+  pdl_begin();
   constexpr int kPer = kColSamples / kSeedThreads;
   __shared__ float s_m[kSeedThreads / 32];
   __shared__ uint32_t s_h[kSeedThreads / 32];
@@ -709,6 +719,7 @@ __global__ void __launch_bounds__(kSeedThreads) k_collision_seed(const float4* _
 }
 
 __global__ void k_zero_bytes(uint8_t* p, size_t n) {
+  pdl_begin();
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) p[i] = 0;
 }
 
@@ -726,10 +737,8 @@ cudaError_t launch_uncertainty_update(const float* mo_prev, const float* mo_cur,
   if (n <= 0) return cudaSuccess;
   int64_t g = (n + kBlock - 1) / kBlock;
   if (g > 4096) g = 4096;
-  k_uncertainty_update<<<(unsigned)g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo_prev),
-                                                       reinterpret_cast<const float4*>(mo_cur),
-                                                       reinterpret_cast<float4*>(su), n, squared);
-  note_launch();
+  launch(k_uncertainty_update, (unsigned)g, kBlock, 0, st, reinterpret_cast<const float4*>(mo_prev),
+         reinterpret_cast<const float4*>(mo_cur), reinterpret_cast<float4*>(su), n, squared);
   return cudaGetLastError();
 }
 
@@ -745,12 +754,9 @@ cudaError_t launch_uncertainty_thresholds(const float* mo, const float* su, int6
   if (g > kMomBlocks) g = kMomBlocks;
   const float4* m = reinterpret_cast<const float4*>(mo);
   const float4* s = reinterpret_cast<const float4*>(su);
-  k_u_moments<0><<<g, kMomThreads, 0, st>>>(m, s, n, ground_z, part);
-  note_launch();
-  k_u_moments<1><<<g, kMomThreads, 0, st>>>(m, s, n, ground_z, part);
-  note_launch();
-  k_u_finish<<<1, 96, 0, st>>>(part, g, stats);
-  note_launch();
+  launch_spread(k_u_moments<0>, g, kMomThreads, 0, st, m, s, n, ground_z, part);
+  launch_spread(k_u_moments<1>, g, kMomThreads, 0, st, m, s, n, ground_z, part);
+  launch(k_u_finish, 1, 96, 0, st, part, g, stats);
   return cudaGetLastError();
 }
 
@@ -770,19 +776,17 @@ cudaError_t launch_view_utility(const float* mo, const float* su, int64_t n, con
   for (int v0 = 0; v0 < n_views; v0 += kViewChunk) {
     const int nv = n_views - v0 < kViewChunk ? n_views - v0 : kViewChunk;
     if (sum)
-      k_view_utility<true><<<g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo),
-                                                 reinterpret_cast<const float4*>(su), n, cams, v0, nv, prm, stats,
-                                                 cnt_part, sum_part, n_views);
+      launch_spread(k_view_utility<true>, g, kBlock, 0, st, reinterpret_cast<const float4*>(mo),
+                    reinterpret_cast<const float4*>(su), n, cams, v0, nv, prm, stats, cnt_part, sum_part, n_views);
     else
-      k_view_utility<false><<<g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo),
-                                                  reinterpret_cast<const float4*>(su), n, cams, v0, nv, prm, stats,
-                                                  cnt_part, sum_part, n_views);
-    note_launch();
+      launch_spread(k_view_utility<false>, g, kBlock, 0, st, reinterpret_cast<const float4*>(mo),
+                    reinterpret_cast<const float4*>(su), n, cams, v0, nv, prm, stats, cnt_part, sum_part, n_views);
   }
   const int fb = (n_views + kWarps - 1) / kWarps;
-  if (sum) k_view_utility_finish<true><<<fb, kBlock, 0, st>>>(cnt_part, sum_part, g, n_views, prm.lambda, xi, counts);
-  else k_view_utility_finish<false><<<fb, kBlock, 0, st>>>(cnt_part, sum_part, g, n_views, prm.lambda, xi, counts);
-  note_launch();
+  if (sum) launch(k_view_utility_finish<true>, fb, kBlock, 0, st, cnt_part, sum_part, g, n_views, prm.lambda, xi,
+                  counts);
+  else launch(k_view_utility_finish<false>, fb, kBlock, 0, st, cnt_part, sum_part, g, n_views, prm.lambda, xi,
+              counts);
   return cudaGetLastError();
 }
 
@@ -799,22 +803,19 @@ cudaError_t launch_regions(const float* mo, const float* su, int64_t n, const gs
   if (count_out) cnt = count_out;
   int64_t zb = ((int64_t)sizeof(double) * nr + 255) / 256;
   if (zb > 4096) zb = 4096;
-  k_zero_bytes<<<(unsigned)(zb < 1 ? 1 : zb), 256, 0, st>>>(reinterpret_cast<uint8_t*>(sum), sizeof(double) * nr);
-  note_launch();
-  k_zero_bytes<<<(unsigned)(zb < 1 ? 1 : zb), 256, 0, st>>>(reinterpret_cast<uint8_t*>(cnt), sizeof(uint32_t) * nr);
-  note_launch();
+  launch(k_zero_bytes, (unsigned)(zb < 1 ? 1 : zb), 256, 0, st, reinterpret_cast<uint8_t*>(sum), sizeof(double) * nr);
+  launch(k_zero_bytes, (unsigned)(zb < 1 ? 1 : zb), 256, 0, st, reinterpret_cast<uint8_t*>(cnt),
+         sizeof(uint32_t) * nr);
   if (n > 0) {
     int64_t g = (n + kBlock - 1) / kBlock;
     const int64_t most = 8 * (int64_t)device_sm_count();
     if (g > most) g = most;
-    k_regions<<<(unsigned)g, kBlock, 0, st>>>(reinterpret_cast<const float4*>(mo),
-                                              reinterpret_cast<const float4*>(su), n, grid, sum, cnt);
-    note_launch();
+    launch_spread(k_regions, (unsigned)g, kBlock, 0, st, reinterpret_cast<const float4*>(mo),
+                  reinterpret_cast<const float4*>(su), n, grid, sum, cnt);
   }
   int64_t g2 = (nr + 255) / 256;
   if (g2 > 4096) g2 = 4096;
-  k_region_mean<<<(unsigned)(g2 < 1 ? 1 : g2), 256, 0, st>>>(sum, cnt, nr, omega);
-  note_launch();
+  launch(k_region_mean, (unsigned)(g2 < 1 ? 1 : g2), 256, 0, st, sum, cnt, nr, omega);
   return cudaGetLastError();
 }
 
@@ -831,8 +832,7 @@ cudaError_t launch_trajectory_utility(const float* mo, const float* su, int64_t 
   float* xi = c.take<float>((size_t)total);
   cudaError_t e = launch_view_utility(mo, su, n, cams, total, prm, mode, stats, xi, nullptr, uws, st);
   if (e != cudaSuccess) return e;
-  k_traj_sum<<<1, 256, 0, st>>>(xi, n_traj, n_states, traj_out, best_out);
-  note_launch();
+  launch(k_traj_sum, 1, 256, 0, st, xi, n_traj, n_states, traj_out, best_out);
   return cudaGetLastError();
 }
 
@@ -840,10 +840,9 @@ cudaError_t launch_collision_check(const float* mo, const float* su, int64_t n, 
                                    float r_robot, float lambda_g, float ground_z, float* margin_out,
                                    uint32_t* collides_out, cudaStream_t st) {
   if (n_pts <= 0) return cudaSuccess;
-  k_collision_seed<<<(unsigned)n_pts, kSeedThreads, 0, st>>>(
-      reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su), n,
-      reinterpret_cast<const float4*>(pts), r_robot, lambda_g, ground_z, margin_out, collides_out);
-  note_launch();
+  launch(k_collision_seed, (unsigned)n_pts, kSeedThreads, 0, st, reinterpret_cast<const float4*>(mo),
+         reinterpret_cast<const float4*>(su), n, reinterpret_cast<const float4*>(pts), r_robot, lambda_g, ground_z,
+         margin_out, collides_out);
   if (n > kColSamples) {   // (a smaller map has been seen whole)
     // small maps: the points are shared out over several blocks per chunk, so that about three
     // blocks per SM run (each block stages its chunk again)
@@ -853,10 +852,9 @@ cudaError_t launch_collision_check(const float* mo, const float* su, int64_t n, 
     const int64_t most = (n_pts + kBlock - 1) / kBlock;
     if (split > most) split = most;
     if (split > 65535) split = 65535;
-    k_collision<<<dim3((unsigned)chunks, (unsigned)split), kBlock, 0, st>>>(
-        reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su), n,
-        reinterpret_cast<const float4*>(pts), n_pts, r_robot, lambda_g, ground_z, margin_out, collides_out);
-    note_launch();
+    launch_spread(k_collision, dim3((unsigned)chunks, (unsigned)split), kBlock, 0, st,
+                  reinterpret_cast<const float4*>(mo), reinterpret_cast<const float4*>(su), n,
+                  reinterpret_cast<const float4*>(pts), n_pts, r_robot, lambda_g, ground_z, margin_out, collides_out);
   }
   return cudaGetLastError();
 }
