@@ -77,143 +77,146 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
   __shared__ float2 s_up[kFwdWarps][kRing];                                   // (u, position in the list + 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  uint32_t item = blockIdx.x * kFwdWarps + warp;
-  if (item >= n_items) return;
-  item = ordered_item(bins, proj.view_info, n_views, item);
-  TileInfo ti;
-  if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) return;
-  WarpBlock wb;
-  warp_block<1>(ti, wb);
-  float* sx = s_exp[warp];
-  float4* sk = s_col[warp];
-  float2* su = s_up[warp];
-  const float ln_amin = __logf(p.alpha_min);
-  const LaneOffsets2 lo = lane_offsets2(lane);
-  const float ccx = wb.bx0 + 3.5f, ccy = wb.by0 + 1.5f;   // centre of the 8x4 block
-  const bool inside = wb.px < ti.W && wb.py < ti.H;
-  bool alive = inside;
-  float T = 1.f, cu = 0.f;
-  f32x2 rg = 0ull, bd = 0ull;
-  int32_t last = 0, n_contrib = 0;
-  const uint32_t n = ti.end - ti.beg;
-  const uint32_t* rl = bins.rec + ti.beg;
-  const float4* SP = reinterpret_cast<const float4*>(proj.splat);
-  const float4* CD = reinterpret_cast<const float4*>(proj.color_d);
-  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  uint32_t rA = 0, rB = 0, rC = 0;
-  if ((uint32_t)lane < n) rA = __ldg(rl + lane);
-  if (32u + lane < n) rB = __ldg(rl + 32 + lane);
-  if (64u + lane < n) rC = __ldg(rl + 64 + lane);
-  float4 mA = z4, mB = z4;
-  if ((uint32_t)lane < n) mA = __ldg(SP + 2 * (size_t)rA);
-  if (32u + lane < n) mB = __ldg(SP + 2 * (size_t)rB);
-  bool ovA = (uint32_t)lane < n && box_overlaps(mA, wb);
-  float4 cA = z4, kA = z4;
-  if (ovA) {
-    cA = __ldg(SP + 2 * (size_t)rA + 1);
-    kA = __ldg(CD + rA);
-  }
-  // Composites the chunk at ring position i0, of which the first `valid` entries exist: the alphas
-  // are independent and computed together, the transmittance updates run in list order.
-  auto chunk = [&](int i0, int valid) {
-    float al[kChunk];
-#pragma unroll
-    for (int k = 0; k < kPairs; ++k) {
-      const float2 a = alpha_raw2(sx, (i0 >> 1) + k, lo);
-      al[2 * k] = fminf(p.alpha_max, a.x);
-      al[2 * k + 1] = fminf(p.alpha_max, a.y);
+  const uint32_t total = item_total(proj, n_views, n_items);
+  // (usually one round: the grid covers the batch's items, see item_blocks)
+  for (uint64_t i = (uint64_t)blockIdx.x * kFwdWarps + warp; i < total; i += (uint64_t)gridDim.x * kFwdWarps) {
+    const uint32_t item = ordered_item(bins, proj.view_info, n_views, (uint32_t)i);
+    TileInfo ti;
+    if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) continue;
+    WarpBlock wb;
+    warp_block<1>(ti, wb);
+    float* sx = s_exp[warp];
+    float4* sk = s_col[warp];
+    float2* su = s_up[warp];
+    const float ln_amin = __logf(p.alpha_min);
+    const LaneOffsets2 lo = lane_offsets2(lane);
+    const float ccx = wb.bx0 + 3.5f, ccy = wb.by0 + 1.5f;   // centre of the 8x4 block
+    const bool inside = wb.px < ti.W && wb.py < ti.H;
+    bool alive = inside;
+    float T = 1.f, cu = 0.f;
+    f32x2 rg = 0ull, bd = 0ull;
+    int32_t last = 0, n_contrib = 0;
+    const uint32_t n = ti.end - ti.beg;
+    const uint32_t* rl = bins.rec + ti.beg;
+    const float4* SP = reinterpret_cast<const float4*>(proj.splat);
+    const float4* CD = reinterpret_cast<const float4*>(proj.color_d);
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t rA = 0, rB = 0, rC = 0;
+    if ((uint32_t)lane < n) rA = __ldg(rl + lane);
+    if (32u + lane < n) rB = __ldg(rl + 32 + lane);
+    if (64u + lane < n) rC = __ldg(rl + 64 + lane);
+    float4 mA = z4, mB = z4;
+    if ((uint32_t)lane < n) mA = __ldg(SP + 2 * (size_t)rA);
+    if (32u + lane < n) mB = __ldg(SP + 2 * (size_t)rB);
+    bool ovA = (uint32_t)lane < n && box_overlaps(mA, wb);
+    float4 cA = z4, kA = z4;
+    if (ovA) {
+      cA = __ldg(SP + 2 * (size_t)rA + 1);
+      kA = __ldg(CD + rA);
     }
-    float w[kChunk];
-    bool add[kChunk];
-    float Tc = T;   // transmittance as if no entry of the chunk stopped the pixel
+    // Composites the chunk at ring position i0, of which the first `valid` entries exist: the alphas
+    // are independent and computed together, the transmittance updates run in list order.
+    auto chunk = [&](int i0, int valid) {
+      float al[kChunk];
 #pragma unroll
-    for (int k = 0; k < kChunk; ++k) {
-      const bool hit = !(al[k] < p.alpha_min);
-      w[k] = (hit ? al[k] : 0.f) * Tc;
-      Tc = Tc - w[k];              // T (1 - alpha)
-      alive = alive && !(Tc < p.T_min);
-      add[k] = hit && alive && k < valid;
-      if (alive) T = Tc;
-    }
-#pragma unroll
-    for (int k = 0; k < kChunk; ++k) {
-      const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(sk + i0 + k);
-      const float2 e = su[i0 + k];
-      if (add[k]) {
-        const f32x2 w2 = pack2(w[k], w[k]);
-        rg = fma2(w2, c.x, rg);
-        bd = fma2(w2, c.y, bd);
-        cu += w[k] * e.x;
-        last = __float_as_int(e.y);
-        if (kCount) ++n_contrib;
+      for (int k = 0; k < kPairs; ++k) {
+        const float2 a = alpha_raw2(sx, (i0 >> 1) + k, lo);
+        al[2 * k] = fminf(p.alpha_max, a.x);
+        al[2 * k + 1] = fminf(p.alpha_max, a.y);
       }
-    }
-  };
-  uint32_t head = 0, tail = 0;   // ring entries [head, tail) are staged and not yet composited
-  uint32_t lm_prev = 0;
-  for (uint32_t g = 0; g < n; g += 32) {
-    const uint32_t lm = __ballot_sync(0xffffffffu, alive);
-    if (!lm) break;
-    if (lm != lm_prev) live_box(lm, ccx - 3.5f, ccy - 1.5f, wb);
-    lm_prev = lm;
-    const bool ovB = g + 32 + lane < n && box_overlaps(mB, wb);
-    float4 cB = z4, kB = z4;
-    if (ovB) {
-      cB = __ldg(SP + 2 * (size_t)rB + 1);
-      kB = __ldg(CD + rB);
-    }
-    float4 mC = z4;
-    if (g + 64 + lane < n) mC = __ldg(SP + 2 * (size_t)rC);
-    uint32_t rD = 0;
-    if (g + 96 + lane < n) rD = __ldg(rl + g + 96 + lane);
-    ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
-    const uint32_t m = __ballot_sync(0xffffffffu, ovA);
-    if (m) {
-      // the overlapping entries join the ring in list order; whole chunks are composited at once
-      // and a partial chunk waits for the next group's entries
-      if (ovA) {
-        const uint32_t s = (tail + __popc(m & lt)) & (kRing - 1);
-        stage_pair(sx, s, stage_exponent(mA.x, mA.y, cA, ccx, ccy));
-        sk[s] = kA;
-        su[s] = make_float2(mA.w, __int_as_float((int)(g + lane + 1)));
+      float w[kChunk];
+      bool add[kChunk];
+      float Tc = T;   // transmittance as if no entry of the chunk stopped the pixel
+#pragma unroll
+      for (int k = 0; k < kChunk; ++k) {
+        const bool hit = !(al[k] < p.alpha_min);
+        w[k] = (hit ? al[k] : 0.f) * Tc;
+        Tc = Tc - w[k];              // T (1 - alpha)
+        alive = alive && !(Tc < p.T_min);
+        add[k] = hit && alive && k < valid;
+        if (alive) T = Tc;
       }
-      tail += __popc(m);
+#pragma unroll
+      for (int k = 0; k < kChunk; ++k) {
+        const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(sk + i0 + k);
+        const float2 e = su[i0 + k];
+        if (add[k]) {
+          const f32x2 w2 = pack2(w[k], w[k]);
+          rg = fma2(w2, c.x, rg);
+          bd = fma2(w2, c.y, bd);
+          cu += w[k] * e.x;
+          last = __float_as_int(e.y);
+          if (kCount) ++n_contrib;
+        }
+      }
+    };
+    uint32_t head = 0, tail = 0;   // ring entries [head, tail) are staged and not yet composited
+    uint32_t lm_prev = 0;
+    for (uint32_t g = 0; g < n; g += 32) {
+      const uint32_t lm = __ballot_sync(0xffffffffu, alive);
+      if (!lm) break;
+      if (lm != lm_prev) live_box(lm, ccx - 3.5f, ccy - 1.5f, wb);
+      lm_prev = lm;
+      const bool ovB = g + 32 + lane < n && box_overlaps(mB, wb);
+      float4 cB = z4, kB = z4;
+      if (ovB) {
+        cB = __ldg(SP + 2 * (size_t)rB + 1);
+        kB = __ldg(CD + rB);
+      }
+      float4 mC = z4;
+      if (g + 64 + lane < n) mC = __ldg(SP + 2 * (size_t)rC);
+      uint32_t rD = 0;
+      if (g + 96 + lane < n) rD = __ldg(rl + g + 96 + lane);
+      ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
+      const uint32_t m = __ballot_sync(0xffffffffu, ovA);
+      if (m) {
+        // the overlapping entries join the ring in list order; whole chunks are composited at once
+        // and a partial chunk waits for the next group's entries
+        if (ovA) {
+          const uint32_t s = (tail + __popc(m & lt)) & (kRing - 1);
+          stage_pair(sx, s, stage_exponent(mA.x, mA.y, cA, ccx, ccy));
+          sk[s] = kA;
+          su[s] = make_float2(mA.w, __int_as_float((int)(g + lane + 1)));
+        }
+        tail += __popc(m);
+        __syncwarp();
+        const uint32_t end = head + (tail - head) / kChunk * kChunk;
+        for (uint32_t h = head; h != end && alive; h += kChunk) {
+          chunk((int)(h & (kRing - 1)), kChunk);
+        }
+        head = end;
+        __syncwarp();
+      }
+      mA = mB; ovA = ovB; cA = cB; kA = kB;
+      rB = rC; mB = mC;
+      rC = rD;
+    }
+    // the last partial chunk, padded with entries of c0 = -inf (alpha = 0)
+    if (tail != head && __any_sync(0xffffffffu, alive)) {
+      const int i0 = (int)(head & (kRing - 1));
+      if ((uint32_t)lane >= tail - head && lane < kChunk)
+        stage_pair(sx, i0 + lane, Exponent{-INFINITY, 0.f, 0.f, 0.f, 0.f, 0.f});
       __syncwarp();
-      const uint32_t end = head + (tail - head) / kChunk * kChunk;
-      for (uint32_t h = head; h != end && alive; h += kChunk) {
-        chunk((int)(h & (kRing - 1)), kChunk);
-      }
-      head = end;
-      __syncwarp();
+      if (alive) chunk(i0, (int)(tail - head));
     }
-    mA = mB; ovA = ovB; cA = cB; kA = kB;
-    rB = rC; mB = mC;
-    rC = rD;
+    __syncwarp();   // (the next round stages over this one's entries)
+    if (!inside) continue;
+    const float2 vrg = unpack2(rg), vbd = unpack2(bd);
+    const size_t P = (size_t)ti.W * ti.H;
+    const size_t pix = (size_t)wb.py * ti.W + wb.px;
+    const size_t o = (size_t)ti.pix_base + pix;
+    if (img.rgb) {
+      float* base = img.rgb + 3 * (size_t)ti.pix_base;
+      base[pix] = vrg.x;
+      base[P + pix] = vrg.y;
+      base[2 * P + pix] = vbd.x;
+    }
+    if (img.depth) img.depth[o] = vbd.y;
+    if (img.unc) img.unc[o] = cu;
+    if (img.T) img.T[o] = T;
+    if (img.last) img.last[o] = last;
+    if (kCount) img.n_contrib[o] = n_contrib;
   }
-  // the last partial chunk, padded with entries of c0 = -inf (alpha = 0)
-  if (tail != head && __any_sync(0xffffffffu, alive)) {
-    const int i0 = (int)(head & (kRing - 1));
-    if ((uint32_t)lane >= tail - head && lane < kChunk)
-      stage_pair(sx, i0 + lane, Exponent{-INFINITY, 0.f, 0.f, 0.f, 0.f, 0.f});
-    __syncwarp();
-    if (alive) chunk(i0, (int)(tail - head));
-  }
-  if (!inside) return;
-  const float2 vrg = unpack2(rg), vbd = unpack2(bd);
-  const size_t P = (size_t)ti.W * ti.H;
-  const size_t pix = (size_t)wb.py * ti.W + wb.px;
-  const size_t o = (size_t)ti.pix_base + pix;
-  if (img.rgb) {
-    float* base = img.rgb + 3 * (size_t)ti.pix_base;
-    base[pix] = vrg.x;
-    base[P + pix] = vrg.y;
-    base[2 * P + pix] = vbd.x;
-  }
-  if (img.depth) img.depth[o] = vbd.y;
-  if (img.unc) img.unc[o] = cu;
-  if (img.T) img.T[o] = T;
-  if (img.last) img.last[o] = last;
-  if (kCount) img.n_contrib[o] = n_contrib;
 }
 
 // Composites `chunks` whole chunks of kIgBatch staged entries, starting at ring position
@@ -411,7 +414,7 @@ cudaError_t launch_render_fwd(const gs_map& map, const gs_proj& proj, const gs_b
                               int n_views, const gs_params& p, const gs_image& img, cudaStream_t st) {
   const int64_t items = bins.tile_capacity * (32 / kPix);   // upper bound: at most 32 items per tile
   if (items > 0) {
-    const unsigned grid = (unsigned)((items + kFwdWarps - 1) / kFwdWarps);
+    const unsigned grid = item_blocks(bins, items, kFwdWarps);
     const int b = p.fwd_batch ? p.fwd_batch : kFwdBatchDefault;
     auto kern = img.n_contrib ? (b == 4 ? k_render_fwd<2, true> : k_render_fwd<1, true>)
                               : (b == 4 ? k_render_fwd<2, false> : k_render_fwd<1, false>);

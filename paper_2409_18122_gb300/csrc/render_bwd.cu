@@ -47,181 +47,184 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 12) k_render_bwd(gs_map map, g
   __shared__ __align__(16) float s_gpix[kBwdWarps][4][32];                     // image gradient (d, r, g, b) per pixel
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  uint32_t item = blockIdx.x * kBwdWarps + warp;
-  if (item >= n_items) return;
-  item = ordered_item(bins, proj.view_info, n_views, item);   // longest tile lists first
-  TileInfo ti;
-  if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) return;
-  WarpBlock wb;
-  warp_block<1>(ti, wb);
-  float4* sa = s_stage[warp][0];
-  float4* sb = s_stage[warp][1];
-  float4* sk = s_stage[warp][2];
-  float* rq = s_red[warp][0];
-  float* rw = s_red[warp][1];
-  const float4* SP = reinterpret_cast<const float4*>(proj.splat);
-  const float4* CD = reinterpret_cast<const float4*>(proj.color_d);
-  uint32_t my_rec = 0;   // record of batched entry `lane & 15`
-  int nb = 0;            // entries waiting in the batch (warp-uniform)
-  // Sums the batched entries' terms and adds them to their records' gradient slots:
-  // (P, Q, dL/da, dL/db), (dL/dc, o dL/do, dL/dt_z, -), (dL/dr, dL/dg, dL/db, -).
-  auto flush = [&](int count) {
-    __syncwarp();
-    const int e = lane & (kRedBatch - 1), h = lane >> 4;
-    const float2 mu = __ldg(reinterpret_cast<const float2*>(SP + 2 * (size_t)my_rec));   // (a record read before)
-    // w times the image gradient, two pixels at a time
-    const ulonglong2* W = reinterpret_cast<const ulonglong2*>(rw + e * kRedPitch + 16 * h);
-    const ulonglong2* G = reinterpret_cast<const ulonglong2*>(&s_gpix[warp][0][16 * h]);
-    f32x2 gs[4] = {0ull, 0ull, 0ull, 0ull};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const ulonglong2 w = W[k];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const ulonglong2 g = G[8 * c + k];
-        gs[c] = fma2(w.y, g.y, fma2(w.x, g.x, gs[c]));
-      }
-    }
-    // dL/dq times (1, dx, dy, dx^2, dx dy, dy^2), dx = mu_x - pixel centre
-    const ulonglong2* D = reinterpret_cast<const ulonglong2*>(rq + e * kRedPitch + 16 * h);
-    const f32x2 mx = pack2(mu.x, mu.x);
-    f32x2 dx[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) dx[j] = add2(mx, pack2(-(wb.bx0 + (float)(2 * j)), -(wb.bx0 + (float)(2 * j + 1))));
-    f32x2 a2 = 0ull;
-    float sP = 0.f, sQ = 0.f, sB = 0.f, sC = 0.f, s0 = 0.f;
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const ulonglong2 x0 = D[2 * r], x1 = D[2 * r + 1];
-      const f32x2 x[4] = {x0.x, x0.y, x1.x, x1.y};
-      f32x2 o2 = 0ull, p2 = 0ull;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const f32x2 t = mul2(x[j], dx[j]);
-        o2 = add2(o2, x[j]);
-        p2 = add2(p2, t);
-        a2 = fma2(t, dx[j], a2);
-      }
-      const float dy = __fsub_rn(mu.y, wb.by0 + (float)(2 * h + r));
-      const float o = sum2(o2), pr = sum2(p2), q = o * dy;
-      s0 += o;
-      sP += pr;
-      sQ += q;
-      sB = fmaf(pr, dy, sB);
-      sC = fmaf(q, dy, sC);
-    }
-    float v[10] = {sP, sQ, sum2(a2), 2.f * sB, sC, -2.f * s0, sum2(gs[0]), sum2(gs[1]), sum2(gs[2]), sum2(gs[3])};
-#pragma unroll
-    for (int j = 0; j < 10; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 16);
-    if (e < count) {
-      float4* dst = g2d + 3 * (size_t)my_rec;
-      atomicAdd(dst + h, h ? make_float4(v[4], v[5], v[6], 0.f) : make_float4(v[0], v[1], v[2], v[3]));
-      if (h) atomicAdd(dst + 2, make_float4(v[7], v[8], v[9], 0.f));
-    }
-    __syncwarp();
-  };
-  const float ln_amin = __logf(p.alpha_min);
-  const LaneOffsets lo = lane_offsets(lane);
-  const float ccx = wb.bx0 + 3.5f, ccy = wb.by0 + 1.5f;   // centre of the 8x4 block
-  const size_t P = (size_t)ti.W * ti.H;
-  float T = 1.f, gr = 0.f, gg = 0.f, gb = 0.f, gd = 0.f;
-  float S = 0.f;   // sum over the entries behind of w_j (image gradient . x_j)
-  int last = 0;    // 0 outside the image
-  if (wb.px < ti.W && wb.py < ti.H) {
-    const size_t pix = (size_t)wb.py * ti.W + wb.px;
-    const size_t o = (size_t)ti.pix_base + pix;
-    T = fwd.T[o];
-    last = fwd.last[o];
-    if (grad.rgb) {
-      const float* base = grad.rgb + 3 * (size_t)ti.pix_base;
-      gr = base[pix];
-      gg = base[P + pix];
-      gb = base[2 * P + pix];
-    }
-    if (grad.depth) gd = grad.depth[o];
-  }
-  const int wlast = (int)__reduce_max_sync(0xffffffffu, (unsigned)(last > 0 ? last : 0));
-  if (wlast == 0) return;
-  s_gpix[warp][0][lane] = gd;
-  s_gpix[warp][1][lane] = gr;
-  s_gpix[warp][2][lane] = gg;
-  s_gpix[warp][3][lane] = gb;
-  // groups of 32 entries are walked from the last one any lane used back to the
-  // first, with the same four-stage pipeline as the forward kernel (alpha and
-  // colour data of the next group, means of the one after, list indices of the
-  // one after that)
-  const uint32_t* rl = bins.rec + ti.beg;
-  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  int g = ((wlast - 1) >> 5) << 5;
-  uint32_t rA = 0, rB = 0, rC = 0;
-  if (g + lane < wlast) rA = __ldg(rl + g + lane);
-  if (g >= 32) rB = __ldg(rl + g - 32 + lane);
-  if (g >= 64) rC = __ldg(rl + g - 64 + lane);
-  float4 mA = z4, mB = z4;
-  if (g + lane < wlast) mA = __ldg(SP + 2 * (size_t)rA);
-  if (g >= 32) mB = __ldg(SP + 2 * (size_t)rB);
-  bool ovA = g + lane < wlast && box_overlaps(mA, wb);
-  float4 cA = z4, kA = z4;
-  if (ovA) {
-    cA = __ldg(SP + 2 * (size_t)rA + 1);
-    kA = __ldg(CD + rA);
-  }
-  for (; g >= 0; g -= 32) {
-    const bool ovB = g >= 32 && box_overlaps(mB, wb);
-    float4 cB = z4, kB = z4;
-    if (ovB) {
-      cB = __ldg(SP + 2 * (size_t)rB + 1);
-      kB = __ldg(CD + rB);
-    }
-    float4 mC = z4;
-    if (g >= 64) mC = __ldg(SP + 2 * (size_t)rC);
-    uint32_t rD = 0;
-    if (g >= 96) rD = __ldg(rl + g - 96 + lane);
-    ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
-    const uint32_t m = __ballot_sync(0xffffffffu, ovA);
-    if (m) {
-      // the overlapping entries, compacted in list order
-      if (ovA) {
-        const int s = __popc(m & lt);
-        const Exponent e = stage_exponent(mA.x, mA.y, cA, ccx, ccy);
-        sa[s] = make_float4(e.c0, e.cu, e.cv, e.kx);
-        sb[s] = make_float4(e.ky, e.kz, __int_as_float(g + lane), __uint_as_float(rA));
-        sk[s] = kA;
-      }
+  const uint32_t total = item_total(proj, n_views, n_items);
+  // longest tile lists first (usually one round: the grid covers the batch's items, see item_blocks)
+  for (uint64_t i = (uint64_t)blockIdx.x * kBwdWarps + warp; i < total; i += (uint64_t)gridDim.x * kBwdWarps) {
+    const uint32_t item = ordered_item(bins, proj.view_info, n_views, (uint32_t)i);
+    TileInfo ti;
+    if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) continue;
+    WarpBlock wb;
+    warp_block<1>(ti, wb);
+    float4* sa = s_stage[warp][0];
+    float4* sb = s_stage[warp][1];
+    float4* sk = s_stage[warp][2];
+    float* rq = s_red[warp][0];
+    float* rw = s_red[warp][1];
+    const float4* SP = reinterpret_cast<const float4*>(proj.splat);
+    const float4* CD = reinterpret_cast<const float4*>(proj.color_d);
+    uint32_t my_rec = 0;   // record of batched entry `lane & 15`
+    int nb = 0;            // entries waiting in the batch (warp-uniform)
+    // Sums the batched entries' terms and adds them to their records' gradient slots:
+    // (P, Q, dL/da, dL/db), (dL/dc, o dL/do, dL/dt_z, -), (dL/dr, dL/dg, dL/db, -).
+    auto flush = [&](int count) {
       __syncwarp();
-      for (int i = __popc(m) - 1; i >= 0; --i) {
-        const float4 ea = sa[i], eb = sb[i];
-        // the alpha of the forward pass (same staged coefficients, same operations); ar = o G.
-        // A lane that does not contribute runs the same arithmetic with alpha = 0: its T and
-        // suffix sum stay exactly unchanged (T * 1, S + 0) and its terms are zero.
-        const float ar = alpha_raw(ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, lo);
-        float al = fminf(p.alpha_max, ar);
-        const bool contrib = __float_as_int(eb.z) < last && !(al < p.alpha_min);
-        if (!__any_sync(0xffffffffu, contrib)) continue;
-        if (!contrib) al = 0.f;
-        const float4 c = sk[i];
-        const float inv = __fdividef(1.f, 1.f - al);   // 1 - alpha in [1 - alpha_max, 1]: approximate reciprocal
-        T *= inv;
-        const float w = al * T;
-        const float gc = gr * c.x + gg * c.y + gb * c.z + gd * c.w;   // image gradient . x_i
-        const float dalpha = gc * T - S * inv;
-        S += w * gc;
-        // dL/dq = -alpha/2 dL/dalpha where alpha is not clamped (there o dL/do = -2 dL/dq)
-        rq[nb * kRedPitch + lane] = ar < p.alpha_max ? -0.5f * al * dalpha : 0.f;
-        rw[nb * kRedPitch + lane] = w;
-        if ((lane & (kRedBatch - 1)) == nb) my_rec = __float_as_uint(eb.w);
-        if (++nb == kRedBatch) {
-          flush(kRedBatch);
-          nb = 0;
+      const int e = lane & (kRedBatch - 1), h = lane >> 4;
+      const float2 mu = __ldg(reinterpret_cast<const float2*>(SP + 2 * (size_t)my_rec));   // (a record read before)
+      // w times the image gradient, two pixels at a time
+      const ulonglong2* W = reinterpret_cast<const ulonglong2*>(rw + e * kRedPitch + 16 * h);
+      const ulonglong2* G = reinterpret_cast<const ulonglong2*>(&s_gpix[warp][0][16 * h]);
+      f32x2 gs[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const ulonglong2 w = W[k];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const ulonglong2 g = G[8 * c + k];
+          gs[c] = fma2(w.y, g.y, fma2(w.x, g.x, gs[c]));
         }
       }
+      // dL/dq times (1, dx, dy, dx^2, dx dy, dy^2), dx = mu_x - pixel centre
+      const ulonglong2* D = reinterpret_cast<const ulonglong2*>(rq + e * kRedPitch + 16 * h);
+      const f32x2 mx = pack2(mu.x, mu.x);
+      f32x2 dx[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) dx[j] = add2(mx, pack2(-(wb.bx0 + (float)(2 * j)), -(wb.bx0 + (float)(2 * j + 1))));
+      f32x2 a2 = 0ull;
+      float sP = 0.f, sQ = 0.f, sB = 0.f, sC = 0.f, s0 = 0.f;
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const ulonglong2 x0 = D[2 * r], x1 = D[2 * r + 1];
+        const f32x2 x[4] = {x0.x, x0.y, x1.x, x1.y};
+        f32x2 o2 = 0ull, p2 = 0ull;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const f32x2 t = mul2(x[j], dx[j]);
+          o2 = add2(o2, x[j]);
+          p2 = add2(p2, t);
+          a2 = fma2(t, dx[j], a2);
+        }
+        const float dy = __fsub_rn(mu.y, wb.by0 + (float)(2 * h + r));
+        const float o = sum2(o2), pr = sum2(p2), q = o * dy;
+        s0 += o;
+        sP += pr;
+        sQ += q;
+        sB = fmaf(pr, dy, sB);
+        sC = fmaf(q, dy, sC);
+      }
+      float v[10] = {sP, sQ, sum2(a2), 2.f * sB, sC, -2.f * s0, sum2(gs[0]), sum2(gs[1]), sum2(gs[2]), sum2(gs[3])};
+#pragma unroll
+      for (int j = 0; j < 10; ++j) v[j] += __shfl_xor_sync(0xffffffffu, v[j], 16);
+      if (e < count) {
+        float4* dst = g2d + 3 * (size_t)my_rec;
+        atomicAdd(dst + h, h ? make_float4(v[4], v[5], v[6], 0.f) : make_float4(v[0], v[1], v[2], v[3]));
+        if (h) atomicAdd(dst + 2, make_float4(v[7], v[8], v[9], 0.f));
+      }
       __syncwarp();
+    };
+    const float ln_amin = __logf(p.alpha_min);
+    const LaneOffsets lo = lane_offsets(lane);
+    const float ccx = wb.bx0 + 3.5f, ccy = wb.by0 + 1.5f;   // centre of the 8x4 block
+    const size_t P = (size_t)ti.W * ti.H;
+    float T = 1.f, gr = 0.f, gg = 0.f, gb = 0.f, gd = 0.f;
+    float S = 0.f;   // sum over the entries behind of w_j (image gradient . x_j)
+    int last = 0;    // 0 outside the image
+    if (wb.px < ti.W && wb.py < ti.H) {
+      const size_t pix = (size_t)wb.py * ti.W + wb.px;
+      const size_t o = (size_t)ti.pix_base + pix;
+      T = fwd.T[o];
+      last = fwd.last[o];
+      if (grad.rgb) {
+        const float* base = grad.rgb + 3 * (size_t)ti.pix_base;
+        gr = base[pix];
+        gg = base[P + pix];
+        gb = base[2 * P + pix];
+      }
+      if (grad.depth) gd = grad.depth[o];
     }
-    mA = mB; ovA = ovB; cA = cB; kA = kB; rA = rB;
-    rB = rC; mB = mC;
-    rC = rD;
+    const int wlast = (int)__reduce_max_sync(0xffffffffu, (unsigned)(last > 0 ? last : 0));
+    if (wlast == 0) continue;
+    s_gpix[warp][0][lane] = gd;
+    s_gpix[warp][1][lane] = gr;
+    s_gpix[warp][2][lane] = gg;
+    s_gpix[warp][3][lane] = gb;
+    // groups of 32 entries are walked from the last one any lane used back to the
+    // first, with the same four-stage pipeline as the forward kernel (alpha and
+    // colour data of the next group, means of the one after, list indices of the
+    // one after that)
+    const uint32_t* rl = bins.rec + ti.beg;
+    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    int g = ((wlast - 1) >> 5) << 5;
+    uint32_t rA = 0, rB = 0, rC = 0;
+    if (g + lane < wlast) rA = __ldg(rl + g + lane);
+    if (g >= 32) rB = __ldg(rl + g - 32 + lane);
+    if (g >= 64) rC = __ldg(rl + g - 64 + lane);
+    float4 mA = z4, mB = z4;
+    if (g + lane < wlast) mA = __ldg(SP + 2 * (size_t)rA);
+    if (g >= 32) mB = __ldg(SP + 2 * (size_t)rB);
+    bool ovA = g + lane < wlast && box_overlaps(mA, wb);
+    float4 cA = z4, kA = z4;
+    if (ovA) {
+      cA = __ldg(SP + 2 * (size_t)rA + 1);
+      kA = __ldg(CD + rA);
+    }
+    for (; g >= 0; g -= 32) {
+      const bool ovB = g >= 32 && box_overlaps(mB, wb);
+      float4 cB = z4, kB = z4;
+      if (ovB) {
+        cB = __ldg(SP + 2 * (size_t)rB + 1);
+        kB = __ldg(CD + rB);
+      }
+      float4 mC = z4;
+      if (g >= 64) mC = __ldg(SP + 2 * (size_t)rC);
+      uint32_t rD = 0;
+      if (g >= 96) rD = __ldg(rl + g - 96 + lane);
+      ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
+      const uint32_t m = __ballot_sync(0xffffffffu, ovA);
+      if (m) {
+        // the overlapping entries, compacted in list order
+        if (ovA) {
+          const int s = __popc(m & lt);
+          const Exponent e = stage_exponent(mA.x, mA.y, cA, ccx, ccy);
+          sa[s] = make_float4(e.c0, e.cu, e.cv, e.kx);
+          sb[s] = make_float4(e.ky, e.kz, __int_as_float(g + lane), __uint_as_float(rA));
+          sk[s] = kA;
+        }
+        __syncwarp();
+        for (int k = __popc(m) - 1; k >= 0; --k) {
+          const float4 ea = sa[k], eb = sb[k];
+          // the alpha of the forward pass (same staged coefficients, same operations); ar = o G.
+          // A lane that does not contribute runs the same arithmetic with alpha = 0: its T and
+          // suffix sum stay exactly unchanged (T * 1, S + 0) and its terms are zero.
+          const float ar = alpha_raw(ea.x, ea.y, ea.z, ea.w, eb.x, eb.y, lo);
+          float al = fminf(p.alpha_max, ar);
+          const bool contrib = __float_as_int(eb.z) < last && !(al < p.alpha_min);
+          if (!__any_sync(0xffffffffu, contrib)) continue;
+          if (!contrib) al = 0.f;
+          const float4 c = sk[k];
+          const float inv = __fdividef(1.f, 1.f - al);   // 1 - alpha in [1 - alpha_max, 1]: approximate reciprocal
+          T *= inv;
+          const float w = al * T;
+          const float gc = gr * c.x + gg * c.y + gb * c.z + gd * c.w;   // image gradient . x_i
+          const float dalpha = gc * T - S * inv;
+          S += w * gc;
+          // dL/dq = -alpha/2 dL/dalpha where alpha is not clamped (there o dL/do = -2 dL/dq)
+          rq[nb * kRedPitch + lane] = ar < p.alpha_max ? -0.5f * al * dalpha : 0.f;
+          rw[nb * kRedPitch + lane] = w;
+          if ((lane & (kRedBatch - 1)) == nb) my_rec = __float_as_uint(eb.w);
+          if (++nb == kRedBatch) {
+            flush(kRedBatch);
+            nb = 0;
+          }
+        }
+        __syncwarp();
+      }
+      mA = mB; ovA = ovB; cA = cB; kA = kB; rA = rB;
+      rB = rC; mB = mC;
+      rC = rD;
+    }
+    if (nb) flush(nb);   // (synchronises the warp: the next round stages over this one's entries)
+    else __syncwarp();
   }
-  if (nb) flush(nb);
 }
 
 __global__ void k_zero_g2d(float4* __restrict__ g2d, const uint32_t* count, int64_t cap) {
@@ -384,7 +387,7 @@ cudaError_t launch_render_bwd(const gs_map& map, const gs_proj& proj, const gs_b
   launch(k_zero_g2d, (unsigned)zb, 256, 0, st, g2d, proj.count, proj.capacity);
   const int64_t items = bins.tile_capacity * 32;   // upper bound: at most 32 items per tile
   if (items > 0) {
-    launch_spread(k_render_bwd, (unsigned)((items + kBwdWarps - 1) / kBwdWarps), kBwdWarps * 32, 0, st, map, proj,
+    launch_spread(k_render_bwd, item_blocks(bins, items, kBwdWarps), kBwdWarps * 32, 0, st, map, proj,
                   bins, cams, n_views, p, fwd, g, g2d, (uint32_t)items);
   }
   if (map.n > 0) {

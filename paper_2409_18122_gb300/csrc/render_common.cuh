@@ -234,6 +234,22 @@ __device__ __forceinline__ uint32_t ordered_item(const gs_bins& bins, const uint
   return ((int64_t)n <= bins.item_capacity && i < n) ? bins.item_order[i] : i;
 }
 
+// Warp items of the batch, at most n_items (the tile capacity's upper bound).
+__device__ __forceinline__ uint32_t item_total(const gs_proj& proj, int n_views, uint32_t n_items) {
+  const uint32_t n = proj.view_info[kVI * n_views + 2];
+  return n < n_items ? n : n_items;
+}
+
+// Blocks of a compositing launch with `warps` items each.  The host knows an upper bound of the
+// items, 32 for each tile of the capacity, and, when the binning orders them, usually their number
+// (item_capacity): the grid has that many, and the kernels' item loops run again if the batch has
+// more after all.  16x16 tiles have 8 items of the 32: the
+// blocks without one took 70 us of the 1.32 ms mapping iteration of four 640x480 views.
+inline unsigned item_blocks(const gs_bins& bins, int64_t items, int warps) {
+  if (bins.item_order && bins.item_capacity > 0 && bins.item_capacity < items) items = bins.item_capacity;
+  return (unsigned)((items + warps - 1) / warps);
+}
+
 template <int KP>
 __device__ __forceinline__ void warp_block(const TileInfo& ti, WarpBlock& wb) {
   const int lane = threadIdx.x & 31;
