@@ -23,6 +23,8 @@
 // No pair is ever sorted or moved twice, no block waits on another, and the
 // result is deterministic.  Chunks hold equal numbers of pairs: near Gaussians,
 // which come first in depth order, cover many tiles each.
+#include <algorithm>
+
 #include "gs_common.cuh"
 #include "gs_internal.h"
 
@@ -34,11 +36,16 @@ constexpr int kMaxGrid = 4096;
 // warp chunks over all views (256-candidate batch, binning: 49,152 / 65,536 / 98,304 / 131,072
 // chunks 3.45 / 3.40 / 3.35 / 3.35 ms; at 131,072 the 2^24-entry count table bounds K there)
 constexpr int kChunkTarget = 131072;
-constexpr int kPairsPerEntry = 4;     // pairs per (tile, chunk) count entry, at least
+constexpr int kPairsPerEntry = 4;     // pairs per (tile, chunk) count entry, at least ...
+// ... unless that leaves fewer chunks than this, seven warps per SM, and a table of at most 2^21
+// entries holds them: one 640x480 view of 200k Gaussians had 333 chunks of 2,900 pairs, each a
+// serial chain of rounds (placement 48 us; 25 us with 1,024; 4,096 cost as much in the table's scan)
+constexpr int kLeastChunks = 1024;
+constexpr int64_t kLeastTable = (int64_t)1 << 21;
 constexpr int kWin = 1024;            // tile cells of a histogram window (shared memory per warp)
 constexpr int kPlaceWin = 512;        // tile cells of a placement window (running slots per warp)
 constexpr int kWinCols = 256;         // widest window, in tiles
-constexpr int kBinWarps = 8;          // warps (= chunks) per block of the histogram / placement kernels
+constexpr int kBinWarps = 2;          // warps (= chunks) per block of the histogram / placement kernels
 
 inline unsigned grid_for(int64_t n_cap) {
   int64_t b = (n_cap + kBlock - 1) / kBlock;
@@ -57,7 +64,8 @@ int chunks_per_view(int n_views, int64_t tile_cap, int64_t pair_cap) {
     const int64_t by_table = ((int64_t)1 << 24) / tile_cap;
     const int64_t by_pairs = pair_cap / kPairsPerEntry / tile_cap;
     if (k > by_table) k = by_table;
-    if (k > by_pairs) k = by_pairs;
+    const int64_t least = std::min<int64_t>((kLeastChunks + n_views - 1) / n_views, kLeastTable / tile_cap);
+    k = std::min(k, std::max(by_pairs, least));
   }
   if (k < 1) k = 1;
   return (int)k;
@@ -317,7 +325,7 @@ __global__ void k_bin_ranges(const uint32_t* __restrict__ off, const uint32_t* _
 // cell's running slot plus that rank, and the lowest of them advances the running
 // slot for the next round.
 template <bool kTileIds>
-__global__ void __launch_bounds__(kBinWarps * 32, 5) k_bin_place(const gs_proj proj,
+__global__ void __launch_bounds__(kBinWarps * 32, 40 / kBinWarps) k_bin_place(const gs_proj proj,
                                                                  const uint32_t* __restrict__ bounds,
                                                                  const SortedRecords sorted,
                                                                  const ushort4* __restrict__ srect, int n_views, int K,
