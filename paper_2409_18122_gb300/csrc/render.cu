@@ -66,10 +66,14 @@ __device__ __forceinline__ void live_box(uint32_t lm, float x0, float y0, WarpBl
 }
 
 // kPairs: packed pairs per chunk.  kCount: the per-pixel counts are asked for (n_contrib).
-template <int kPairs, bool kCount>
+// kRest = false: block b takes the items 2 b and 2 b + 1.  kRest = true: the blocks share the items
+// from block first_rest on, usually none (launch_items).  One kernel that loops over its items
+// keeps more registers across them: 1,365 instead of 1,324 us for eight 1280x720 views.
+template <int kPairs, bool kCount, bool kRest>
 __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, gs_proj proj, gs_bins bins,
                                                                 const gs_camera* __restrict__ cams, int n_views,
-                                                                gs_params p, gs_image img, uint32_t n_items) {
+                                                                gs_params p, gs_image img, uint32_t n_items,
+                                                                uint32_t first_rest) {
   pdl_begin();
   constexpr int kChunk = 2 * kPairs;
   __shared__ __align__(16) float s_exp[kFwdWarps][kRing / 2 * kPairFloats];   // staged exponents (stage_pair)
@@ -77,10 +81,10 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
   __shared__ float2 s_up[kFwdWarps][kRing];                                   // (u, position in the list + 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t lt = (1u << lane) - 1u;
-  const uint32_t total = item_total(proj, n_views, n_items);
-  // (usually one round: the grid covers the batch's items, see item_blocks)
-  for (uint64_t i = (uint64_t)blockIdx.x * kFwdWarps + warp; i < total; i += (uint64_t)gridDim.x * kFwdWarps) {
-    const uint32_t item = ordered_item(bins, proj.view_info, n_views, (uint32_t)i);
+  uint32_t b = blockIdx.x + (kRest ? first_rest : 0u);
+  if (kRest && !more_items(proj, n_views, n_items, b, kFwdWarps)) return;
+  do {
+    const uint32_t item = ordered_item(bins, proj.view_info, n_views, b * kFwdWarps + warp);
     TileInfo ti;
     if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) continue;
     WarpBlock wb;
@@ -216,7 +220,7 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
     if (img.T) img.T[o] = T;
     if (img.last) img.last[o] = last;
     if (kCount) img.n_contrib[o] = n_contrib;
-  }
+  } while (kRest && more_items(proj, n_views, n_items, b += gridDim.x, kFwdWarps));
 }
 
 // Composites `chunks` whole chunks of kIgBatch staged entries, starting at ring position
@@ -414,11 +418,14 @@ cudaError_t launch_render_fwd(const gs_map& map, const gs_proj& proj, const gs_b
                               int n_views, const gs_params& p, const gs_image& img, cudaStream_t st) {
   const int64_t items = bins.tile_capacity * (32 / kPix);   // upper bound: at most 32 items per tile
   if (items > 0) {
-    const unsigned grid = item_blocks(bins, items, kFwdWarps);
     const int b = p.fwd_batch ? p.fwd_batch : kFwdBatchDefault;
-    auto kern = img.n_contrib ? (b == 4 ? k_render_fwd<2, true> : k_render_fwd<1, true>)
-                              : (b == 4 ? k_render_fwd<2, false> : k_render_fwd<1, false>);
-    launch_spread(kern, grid, kFwdWarps * 32, 0, st, map, proj, bins, cams, n_views, p, img, (uint32_t)items);
+    auto run = [&](auto kern, auto rest) {
+      launch_items(bins, items, kFwdWarps, 12, st, kern, rest, map, proj, bins, cams, n_views, p, img);
+    };
+    if (img.n_contrib && b == 4) run(k_render_fwd<2, true, false>, k_render_fwd<2, true, true>);
+    else if (img.n_contrib) run(k_render_fwd<1, true, false>, k_render_fwd<1, true, true>);
+    else if (b == 4) run(k_render_fwd<2, false, false>, k_render_fwd<2, false, true>);
+    else run(k_render_fwd<1, false, false>, k_render_fwd<1, false, true>);
   }
   return cudaGetLastError();
 }

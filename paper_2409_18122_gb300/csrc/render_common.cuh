@@ -4,6 +4,7 @@
 #pragma once
 
 #include "gs_common.cuh"
+#include "gs_internal.h"
 
 namespace gs {
 
@@ -234,20 +235,34 @@ __device__ __forceinline__ uint32_t ordered_item(const gs_bins& bins, const uint
   return ((int64_t)n <= bins.item_capacity && i < n) ? bins.item_order[i] : i;
 }
 
-// Warp items of the batch, at most n_items (the tile capacity's upper bound).
-__device__ __forceinline__ uint32_t item_total(const gs_proj& proj, int n_views, uint32_t n_items) {
+// Whether block round b of `warps` items each still has one (read anew after each round, so that
+// nothing is held in registers across the item's work; b is the same for the whole block).
+__device__ __forceinline__ bool more_items(const gs_proj& proj, int n_views, uint32_t n_items, uint32_t b, int warps) {
   const uint32_t n = proj.view_info[kVI * n_views + 2];
-  return n < n_items ? n : n_items;
+  return (uint64_t)b * warps < (n < n_items ? n : n_items);
 }
 
-// Blocks of a compositing launch with `warps` items each.  The host knows an upper bound of the
-// items, 32 for each tile of the capacity, and, when the binning orders them, usually their number
-// (item_capacity): the grid has that many, and the kernels' item loops run again if the batch has
-// more after all.  16x16 tiles have 8 items of the 32: the
-// blocks without one took 70 us of the 1.32 ms mapping iteration of four 640x480 views.
-inline unsigned item_blocks(const gs_bins& bins, int64_t items, int warps) {
-  if (bins.item_order && bins.item_capacity > 0 && bins.item_capacity < items) items = bins.item_capacity;
-  return (unsigned)((items + warps - 1) / warps);
+// Launches a compositing kernel with `warps` items per block over a batch of at most `items`.  The
+// host knows this upper bound, 32 items for each tile of the capacity, and, when the binning orders
+// the items, usually their number (item_capacity): `kern` gets the blocks for that many, and `rest`
+// a grid of `per_sm` blocks per multiprocessor that look for what is left of the upper bound and
+// leave when nothing is (1.7 us).  16x16 tiles have 8 items of the 32, and a block for each of the
+// other 24 took 70 us of the 1.32 ms mapping iteration of four 640x480 views.
+template <class K, class... A>
+inline void launch_items(const gs_bins& bins, int64_t items, int warps, int per_sm, cudaStream_t st, K kern, K rest,
+                         const A&... args) {
+  const int64_t all = (items + warps - 1) / warps;
+  int64_t blocks = all;
+  if (bins.item_order && bins.item_capacity > 0) {
+    const int64_t ordered = (bins.item_capacity + warps - 1) / warps;
+    if (ordered < all) blocks = ordered;
+  }
+  launch_spread(kern, dim3((unsigned)blocks), dim3(32 * warps), 0, st, args..., (uint32_t)items, (uint32_t)blocks);
+  if (blocks < all) {
+    const int64_t most = (int64_t)per_sm * device_sm_count();
+    const int64_t n = all - blocks < most ? all - blocks : most;
+    launch(rest, dim3((unsigned)n), dim3(32 * warps), 0, st, args..., (uint32_t)items, (uint32_t)blocks);
+  }
 }
 
 template <int KP>

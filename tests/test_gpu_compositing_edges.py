@@ -72,3 +72,28 @@ def test_padding_adds_nothing_without_an_opacity_floor(n):
     out = images_host(fr, img)[0]
     assert np.isfinite(out["rgb"]).all() and np.isfinite(out["depth"]).all()
     assert (out["last"] <= n).all() and (img["n_contrib"] <= n).all()
+
+
+@pytest.mark.parametrize("capacity", [0, 1, 5, 12])
+def test_items_beyond_the_ordered_capacity(capacity):
+    """The grids are sized by the item order's capacity; a batch with more items (then not ordered)
+    is still rendered and differentiated completely: 4 tiles of 8 items here."""
+    gmap, _ = _stack(50, -1.0)
+    cam = Camera(40.0, 40.0, 14.5, 13.0, 29, 26, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    out = []
+    for cut in (None, capacity):
+        fr = gs.Frame(50, [cam])
+        assert fr.n_items == 32
+        if cut is not None:
+            fr.c_bins.item_capacity = cut
+        img = fr.forward(gm)
+        g = fr.render_bwd(gm, img, torch.ones_like(img["rgb"]), torch.ones_like(img["depth"]))
+        torch.cuda.synchronize()
+        fr.check_status()
+        out.append((img, g))
+    for k in ("rgb", "depth", "unc", "T", "last"):
+        assert torch.equal(out[0][0][k], out[1][0][k])
+    for k in ("dmo", "dsu", "dq", "drgb"):      # (sums of atomics: equal up to their order)
+        a, b = out[0][1][k], out[1][1][k]
+        assert float((a - b).abs().max()) <= 1e-4 * float(a.abs().max())
