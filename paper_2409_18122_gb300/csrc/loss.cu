@@ -19,8 +19,8 @@
 // and the halo are 64, two row quads per thread, 1.19 row blurs per output row.  Eight 1280x720
 // views: pass 1 478 -> 283 us, pass 2 276 -> 184 us, the sum of the partials 57 -> 17 us.
 // A one-CTA kernel sums the partials in FP64 in a fixed order.  Without the SSIM term
-// (w_ssim = 0) the loss is elementwise: one flat kernel over the colour and one over the
-// depth array (contiguous chunks per block, fixed partial slots) replaces both passes.
+// (w_ssim = 0) the loss is elementwise: one flat kernel over the colour and the depth array
+// (contiguous chunks per block, fixed partial slots) replaces both passes.
 #include <math.h>
 
 #include "gs_internal.h"
@@ -313,25 +313,36 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_ssim_bwd(const __grid_con
   }
 }
 
-// Loss without the SSIM term: elementwise over the flat arrays.  Block b takes the
-// contiguous elements [b chunk, (b + 1) chunk) and stores its sum of |x - y| in field
-// `field` of partial slot slot0 + b (other fields zero); g = w sign(x - y) / N_p if g.
-// x == NULL (no depth): differences are zero.
-__global__ void __launch_bounds__(kLossThreads) k_loss_l1(const float* __restrict__ x, const float* __restrict__ y,
-                                                          float* __restrict__ g, int64_t n, int64_t chunk, float w,
-                                                          float inv_n, int field, double* __restrict__ part,
-                                                          int64_t slot0) {
+// Loss without the SSIM term: elementwise over the flat arrays.  The first nb_c blocks take the
+// colour, the others the depth: block b of an array the contiguous elements [b chunk, (b + 1) chunk),
+// storing its sum of |x - y| in its own partial slot (other fields zero) and g = w sign(x - y) / N_p
+// if g.  x == NULL (no depth): differences are zero.
+struct L1Array {
+  const float* x;
+  const float* y;
+  float* g;
+  int64_t n;
+  float w;
+};
+
+__global__ void __launch_bounds__(kLossThreads) k_loss_l1(const L1Array colour, const L1Array depth, int64_t chunk,
+                                                          int nb_c, float inv_n, double* __restrict__ part) {
   pdl_begin();
-  const int64_t b0 = (int64_t)blockIdx.x * chunk;
-  const int64_t b1 = b0 + chunk < n ? b0 + chunk : n;
+  const bool is_c = (int)blockIdx.x < nb_c;
+  const L1Array a = is_c ? colour : depth;
+  const int64_t b0 = (int64_t)(is_c ? blockIdx.x : blockIdx.x - nb_c) * chunk;
+  const int64_t b1 = b0 + chunk < a.n ? b0 + chunk : a.n;
+  const float* __restrict__ x = a.x;
+  const float* __restrict__ y = a.y;
+  float* __restrict__ g = a.g;
   float acc = 0.f;
 #pragma unroll 4
   for (int64_t i = b0 + threadIdx.x; i < b1; i += kLossThreads) {
     const float d = x ? x[i] - y[i] : 0.f;
     acc += fabsf(d);
-    if (g) g[i] = w * sgnf(d) * inv_n;
+    if (g) g[i] = a.w * sgnf(d) * inv_n;
   }
-  block_partial(0.f, field == 1 ? acc : 0.f, field == 2 ? acc : 0.f, part + 3 * (slot0 + blockIdx.x));
+  block_partial(0.f, is_c ? acc : 0.f, is_c ? 0.f : acc, part + 3 * (int64_t)blockIdx.x);
 }
 
 // Sums the partials in a fixed order: thread t takes slots t, t + 1024, ..., then a fixed tree.
@@ -441,10 +452,8 @@ cudaError_t launch_image_loss(const int32_t* sizes, int n_views, const float* rg
     chunk = (chunk + 4 * kLossThreads - 1) / (4 * kLossThreads) * (4 * kLossThreads);
     if (chunk < 4096) chunk = 4096;
     const int64_t nb_c = (3 * lay.P + chunk - 1) / chunk, nb_d = (lay.P + chunk - 1) / chunk;
-    launch(k_loss_l1, (unsigned)nb_c, kLossThreads, 0, st, rgb, rgb_ref, d_rgb, 3 * lay.P, chunk, w.w_rgb, a.inv_n, 1,
-           part, 0);
-    launch(k_loss_l1, (unsigned)nb_d, kLossThreads, 0, st, depth, depth_ref, d_depth, lay.P, chunk, w.w_depth,
-           a.inv_n, 2, part, nb_c);
+    const L1Array colour{rgb, rgb_ref, d_rgb, 3 * lay.P, w.w_rgb}, dep{depth, depth_ref, d_depth, lay.P, w.w_depth};
+    launch(k_loss_l1, (unsigned)(nb_c + nb_d), kLossThreads, 0, st, colour, dep, chunk, (int)nb_c, a.inv_n, part);
     slot = nb_c + nb_d;
   }
   for (int v0 = 0; v0 < n_views && ssim; v0 += kLossViewsPerLaunch) {

@@ -118,6 +118,13 @@ __device__ __forceinline__ void stage_cams(const gs_camera* __restrict__ cams, c
   }
 }
 
+// Records written and the overflow flag, from the scanned offsets.
+__device__ __forceinline__ void record_count(const gs_proj& out, int64_t n_slots) {
+  const uint32_t total = out.grp_base[n_slots];
+  *out.count = (int64_t)total > out.capacity ? (uint32_t)out.capacity : total;
+  if ((int64_t)total > out.capacity) set_flag(out.status, GS_FLAG_RECORD_OVERFLOW);
+}
+
 // One warp = one group of 32 consecutive Gaussians.  For every view the lanes
 // test their Gaussian cheaply (near plane, guard band: frustum_ok; in the write
 // pass, the count pass's visibility bit) and queue the (view, lane) pairs that
@@ -144,6 +151,7 @@ __global__ void __launch_bounds__(kBlock) k_project(gs_map map, const gs_camera*
   const bool active = g < map.n;
   const bool grp_active = __any_sync(0xffffffffu, active);
   const int64_t n_grp = (map.n + 31) >> 5;
+  if (kWrite && g == 0) record_count(out, n_grp * n_views);
   float4 mo = make_float4(0.f, 0.f, 0.f, 0.f), su = mo, q = mo, col = mo;
   GaussPre pre;
   pre.valid = false;
@@ -281,11 +289,9 @@ __global__ void __launch_bounds__(kBlock) k_project(gs_map map, const gs_camera*
   }
 }
 
-__global__ void k_record_count(const gs_proj out, int64_t n_slots) {
+__global__ void k_record_count(const gs_proj out, int64_t n_slots) {   // (an empty map: no write pass)
   pdl_begin();
-  const uint32_t total = out.grp_base[n_slots];
-  *out.count = (int64_t)total > out.capacity ? (uint32_t)out.capacity : total;
-  if ((int64_t)total > out.capacity) set_flag(out.status, GS_FLAG_RECORD_OVERFLOW);
+  record_count(out, n_slots);
 }
 
 }  // namespace
@@ -313,8 +319,9 @@ cudaError_t launch_project(const gs_map& map, const gs_camera* cams, int n_views
   if (blocks > 0) {
     launch_spread(k_project<true>, (unsigned)blocks, kBlock, 0, st, map, cams, n_views, p, out.view_info, counts,
                   out);
+  } else {
+    launch(k_record_count, 1, 1, 0, st, out, slots);
   }
-  launch(k_record_count, 1, 1, 0, st, out, slots);
   return cudaGetLastError();
 }
 

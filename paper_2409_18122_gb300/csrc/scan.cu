@@ -1,9 +1,9 @@
 // scan.cu -- device-wide exclusive prefix sum with a device-side element count.
 //
-// Reduce-then-scan in three launches (per-partition sums, scan of the sums,
-// per-partition scan with carry).  Deterministic, no inter-block waiting, and
-// the element count may live in device memory (known only after an earlier
-// kernel), so the launch configuration depends only on the host-side capacity.
+// Reduce-then-scan in two launches: per-partition sums, and per-partition scans, each of whose
+// blocks adds up the sums before its own (at most 1,024).  Deterministic, no inter-block waiting,
+// and the element count may live in device memory (known only after an earlier kernel), so the
+// launch configuration depends only on the host-side capacity.
 #include "gs_internal.h"
 
 namespace gs {
@@ -79,42 +79,10 @@ __global__ void __launch_bounds__(kBlock) k_scan_reduce(const uint32_t* __restri
   if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_partials(unsigned long long* partial, int g, const uint32_t* n_dev,
-                                                        int64_t n_cap, uint32_t* out, uint32_t* total_out) {
-  pdl_begin();
-  __shared__ unsigned long long sums[32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long v = threadIdx.x < g ? partial[threadIdx.x] : 0, x = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    unsigned long long y = __shfl_up_sync(0xffffffffu, x, d);
-    if (lane >= d) x += y;
-  }
-  if (lane == 31) sums[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    unsigned long long w = sums[lane];
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      unsigned long long y = __shfl_up_sync(0xffffffffu, w, d);
-      if (lane >= d) w += y;
-    }
-    sums[lane] = w;
-  }
-  __syncthreads();
-  unsigned long long incl = (warp > 0 ? sums[warp - 1] : 0) + x;
-  if (threadIdx.x < g) partial[threadIdx.x] = incl - v;
-  if (threadIdx.x == 0) {
-    unsigned long long total = sums[31];
-    int64_t n = count_of(n_dev, n_cap);
-    out[n] = sat32(total);
-    if (total_out) *total_out = sat32(total);
-  }
-}
-
 __global__ void __launch_bounds__(kBlock) k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
                                                        const uint32_t* n_dev, int64_t n_cap,
-                                                       const unsigned long long* partial) {
+                                                       const unsigned long long* partial,
+                                                       uint32_t* __restrict__ total_out) {
   pdl_begin();
   const int64_t n = count_of(n_dev, n_cap);
   const int64_t g = gridDim.x;
@@ -122,7 +90,9 @@ __global__ void __launch_bounds__(kBlock) k_scan_down(const uint32_t* __restrict
   const int64_t beg = (int64_t)blockIdx.x * chunk;
   int64_t end = beg + chunk;
   if (end > n) end = n;
-  unsigned long long carry = partial[blockIdx.x];
+  unsigned long long carry, before = 0;   // carry: sum of the partitions before this one
+  for (int i = threadIdx.x; i < (int)blockIdx.x; i += kBlock) before += partial[i];
+  block_exclusive_scan(before, &carry);
   // 16-byte loads and stores when both arrays allow them (i0 is a multiple of 8 elements)
   const bool vec = (((uintptr_t)in | (uintptr_t)out) & 15u) == 0;
   for (int64_t t0 = beg; t0 < end; t0 += kTile) {
@@ -157,6 +127,10 @@ __global__ void __launch_bounds__(kBlock) k_scan_down(const uint32_t* __restrict
     }
     carry += tot;
   }
+  if (blockIdx.x == g - 1 && threadIdx.x == 0) {   // the partitions end at n: carry is the total
+    out[n] = sat32(carry);
+    if (total_out) *total_out = sat32(carry);
+  }
 }
 
 }  // namespace
@@ -168,8 +142,7 @@ cudaError_t scan_exclusive(const uint32_t* in, uint32_t* out, const uint32_t* n_
   const int g = (int)parts_for(n_cap);
   auto* partial = (unsigned long long*)temp;
   launch(k_scan_reduce, g, kBlock, 0, st, in, n_dev, n_cap, partial);
-  launch(k_scan_partials, 1, 1024, 0, st, partial, g, n_dev, n_cap, out, total_out);
-  launch(k_scan_down, g, kBlock, 0, st, in, out, n_dev, n_cap, partial);
+  launch(k_scan_down, g, kBlock, 0, st, in, out, n_dev, n_cap, partial, total_out);
   return cudaGetLastError();
 }
 
