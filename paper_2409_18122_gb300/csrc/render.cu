@@ -18,8 +18,9 @@ namespace gs {
 namespace {
 
 constexpr int kFwdWarps = 2;   // warps (work items) per CTA: small CTAs free their slot as soon as both finish
-constexpr int kIgWarps = 2;    // the same for the persistent information-gain kernel
+constexpr int kIgWarps = 4;    // the same for the persistent information-gain kernel (which shares out long lists)
 constexpr int kRing = 64;      // staged entries per warp (a ring): a group of 32 and a partial chunk
+constexpr uint32_t kLongList = 1024;   // entries that a list has at least to be shared by a block's warps
 constexpr int kPix = 1;        // pixels per lane of the forward and information-gain kernels
 // Chunk depth: staged entries whose alphas are computed together, a template argument of both
 // compositing kernels chosen per launch by gs_params (forward 1, 2 or 4, default 4; 1 runs as 2,
@@ -223,15 +224,15 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
   } while (kRest && more_items(proj, n_views, n_items, b += gridDim.x, kFwdWarps));
 }
 
-// Composites `chunks` whole chunks of kIgBatch staged entries, starting at ring position
+// Composites `chunks` whole chunks of kIgBatch entries staged in a ring of kSlots, starting at position
 // `head` (a multiple of kIgBatch, so no chunk wraps): the alphas of a chunk are independent
 // and computed together, two to an instruction; the transmittance updates then run in list
 // order.  A lane leaves as soon as its pixel is saturated.
-template <int kIgBatch>
+template <int kIgBatch, int kSlots>
 __device__ __forceinline__ void composite_chunks(const float* sx, const float* su, uint32_t head, uint32_t chunks,
                                                  const LaneOffsets2& lo, const gs_params& p, float& T, float& cu) {
   for (uint32_t c = 0; c < chunks && T != 0.f; ++c) {
-    const uint32_t b0 = (head + c * kIgBatch) & (kRing - 1);
+    const uint32_t b0 = (head + c * kIgBatch) & (kSlots - 1);
     float al[kIgBatch], uu[kIgBatch];
 #pragma unroll
     for (int k = 0; k < kIgBatch; k += 2) {
@@ -261,12 +262,113 @@ __device__ __forceinline__ void composite_chunks(const float* sx, const float* s
   }
 }
 
+// One item by a whole block: warp 0 composites, the others look for the entries that reach the item's
+// live pixels, 32 of the list each and round, and stage them in list order in one ring of the block,
+// while warp 0 composites what earlier rounds staged.  The entries and their order are those of a
+// warp on its own (the live pixels that the others know are a round old, which only keeps entries
+// that add nothing), so the sum is the same bit for bit.  sx, su: the block's rings as one.
+template <int kIgBatch>
+__device__ __forceinline__ void composite_long(const TileInfo& ti, WarpBlock wb, const float4* SP, const gs_bins& bins,
+                                               const gs_params& p, float* sx, float* su, uint32_t (*s_cnt)[kIgWarps],
+                                               uint32_t* s_live, float* out) {
+  constexpr int kSlots = kRing * kIgWarps;
+  constexpr uint32_t kStep = 32u * (kIgWarps - 1);
+  static_assert(kSlots >= 2 * (int)kStep + kIgBatch, "a round's entries beside the round before it");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t lt = (1u << lane) - 1u;
+  const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float x0 = wb.bx0, y0 = wb.by0;
+  const float ccx = x0 + 3.5f, ccy = y0 + 1.5f;   // centre of the 8x4 block
+  const uint32_t n = ti.end - ti.beg;
+  const uint32_t* rl = bins.rec + ti.beg;
+  uint32_t tail = 0;   // entries staged by the rounds before this one
+  if (warp == 0) {
+    const LaneOffsets2 lo = lane_offsets2(lane);
+    float T = (wb.px < ti.W && wb.py < ti.H) ? 1.f : 0.f, cu = 0.f;
+    uint32_t head = 0, r = 0;
+    for (uint32_t g = 0; g < n; g += kStep, r ^= 1u) {
+      const uint32_t chunks = (tail - head) / kIgBatch;
+      composite_chunks<kIgBatch, kSlots>(sx, su, head, chunks, lo, p, T, cu);
+      head += chunks * kIgBatch;
+      const uint32_t lm = __ballot_sync(0xffffffffu, T != 0.f);
+      if (lane == 0) s_live[r] = lm;
+      __syncthreads();
+      for (int w = 1; w < kIgWarps; ++w) tail += s_cnt[r][w];
+      if (!lm) break;
+    }
+    const uint32_t rest = (tail - head) % kIgBatch;
+    if (rest && (uint32_t)lane >= rest && (uint32_t)lane < kIgBatch) {   // pad the last chunk (alpha = 0)
+      const uint32_t s = (tail - rest + lane) & (kSlots - 1);
+      stage_pair(sx, s, Exponent{-INFINITY, 0.f, 0.f, 0.f, 0.f, 0.f});
+      su[s] = 0.f;
+    }
+    __syncwarp();
+    composite_chunks<kIgBatch, kSlots>(sx, su, head, (tail - head + kIgBatch - 1) / kIgBatch, lo, p, T, cu);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) cu += __shfl_down_sync(0xffffffffu, cu, d);
+    if (lane == 0) *out = cu;
+  } else {
+    const float ln_amin = __logf(p.alpha_min);
+    const uint32_t i0 = 32u * (warp - 1) + lane;
+    uint32_t rB = 0, rC = 0, r = 0, lm_prev = 0;
+    float4 mA = z4, mB = z4;
+    if (i0 < n) mA = __ldg(SP + 2 * (size_t)__ldg(rl + i0));
+    float4 cA = z4;
+    bool ovA = i0 < n && box_overlaps(mA, wb);
+    if (ovA) cA = __ldg(SP + 2 * (size_t)__ldg(rl + i0) + 1);
+    if (i0 + kStep < n) rB = __ldg(rl + i0 + kStep);
+    if (i0 + 2 * kStep < n) rC = __ldg(rl + i0 + 2 * kStep);
+    if (i0 + kStep < n) mB = __ldg(SP + 2 * (size_t)rB);
+    for (uint32_t g = 0; g < n; g += kStep, r ^= 1u) {
+      const uint32_t i = g + i0;   // (below 2^32: list positions of one batch)
+      const bool ovB = i + kStep < n && box_overlaps(mB, wb);
+      float4 cB = z4;
+      if (ovB) cB = __ldg(SP + 2 * (size_t)rB + 1);
+      float4 mC = z4;
+      if (i + 2 * kStep < n) mC = __ldg(SP + 2 * (size_t)rC);
+      uint32_t rD = 0;
+      if (i + 3 * kStep < n) rD = __ldg(rl + i + 3 * kStep);
+      ovA = ovA && ellipse_reaches(mA, cA, wb, ln_amin);
+      const uint32_t m = __ballot_sync(0xffffffffu, ovA);
+      if (lane == 0) s_cnt[r][warp] = __popc(m);
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * (kIgWarps - 1)) : "memory");   // the staging warps' counts
+      uint32_t s = tail, all = 0;
+      for (int w = 1; w < kIgWarps; ++w) {
+        const uint32_t c = s_cnt[r][w];
+        if (w < warp) s += c;
+        all += c;
+      }
+      if (ovA) {
+        s = (s + __popc(m & lt)) & (kSlots - 1);
+        stage_pair(sx, s, stage_exponent(mA.x, mA.y, cA, ccx, ccy));
+        su[s] = mA.w;
+      }
+      tail += all;
+      __syncthreads();   // the round's entries are staged, the live pixels are known
+      const uint32_t lm = s_live[r];
+      if (!lm) break;
+      if (lm != lm_prev) live_box(lm, x0, y0, wb);
+      lm_prev = lm;
+      mA = mB; ovA = ovB; cA = cB;
+      rB = rC; mB = mC;
+      rC = rD;
+    }
+  }
+  __syncthreads();   // the rings and counts are free again
+}
+
 // Persistent U-only compositing: every warp takes (tile, pixel block) work items
 // from a device counter, longest tile list first, until the batch is exhausted,
 // and writes the sum of U over its pixels to the item's own slot (fixed shuffle
 // tree), never accumulating, so the result does not depend on scheduling.
+// A list that is long against a warp's share of all the lists is still being walked when the others
+// are done (200k Gaussians, 27 views: multiprocessors busy 42% of the time); such lists, which come
+// first, are composited by the whole block (composite_long).  That kernel 435 -> 172 us, the pass
+// over 1M Gaussians and 6 views 2,395 -> 962 us, 400k and 12 views 1,087 -> 529 us; batches whose
+// share is larger than their lists (256 views) have none and are unchanged.  From a quarter of the
+// share and 1,024 entries on: 64 views of 800k Gaussians 1.70 ms, from the whole share 1.91 ms.
 template <int kIgBatch>
-__global__ void __launch_bounds__(kIgWarps * 32, 12) k_ig_items(gs_proj proj, gs_bins bins,
+__global__ void __launch_bounds__(kIgWarps * 32, 24 / kIgWarps) k_ig_items(gs_proj proj, gs_bins bins,
                                                              const gs_camera* __restrict__ cams, int n_views,
                                                              gs_params p, const uint32_t* __restrict__ order,
                                                              float* __restrict__ item_sum, int64_t item_cap,
@@ -284,10 +386,35 @@ __global__ void __launch_bounds__(kIgWarps * 32, 12) k_ig_items(gs_proj proj, gs
   if ((int64_t)n_items > item_cap) n_items = (uint32_t)item_cap;
   const float4* SP = reinterpret_cast<const float4*>(proj.splat);
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+  // a warp's share of the entries of all items' lists: pairs x items per tile / warps
+  const uint64_t tiles = proj.view_info[kVI * n_views];
+  const uint64_t share = tiles ? (uint64_t)*bins.count * n_items / (tiles * gridDim.x * kIgWarps) : 0ull;
+  const uint32_t long_list = (uint32_t)max((uint64_t)kLongList, min(share / 4, (uint64_t)0xFFFFFFFFu));
+  __shared__ uint32_t s_item, s_cnt[2][kIgWarps], s_live[2];
+  uint32_t next = 0xFFFFFFFFu;   // warp 0: an item taken and not yet done
+  for (;;) {   // long lists, by the block
+    if (threadIdx.x == 0) s_item = atomicAdd(work, 1u);
+    __syncthreads();
+    const uint32_t item = s_item;
+    __syncthreads();
+    if (item >= n_items) return;
+    const uint32_t slot = __ldg(order + item);
+    TileInfo ti;
+    if (!warp_item_setup<kPix>(proj, bins, cams, n_views, slot, ti) || ti.end - ti.beg <= long_list) {
+      if (warp == 0) next = item;
+      break;
+    }
+    WarpBlock wb;
+    warp_block<kPix>(ti, wb);
+    composite_long<kIgBatch>(ti, wb, SP, bins, p, s_exp[0], s_u[0], s_cnt, s_live, item_sum + slot);
+  }
   for (;;) {
-    uint32_t item = 0;
-    if (lane == 0) item = atomicAdd(work, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
+    uint32_t item = next;
+    next = 0xFFFFFFFFu;
+    if (item == 0xFFFFFFFFu) {
+      if (lane == 0) item = atomicAdd(work, 1u);
+      item = __shfl_sync(0xffffffffu, item, 0);
+    }
     if (item >= n_items) break;
     // items are handed out longest tile list first; each writes its own slot
     const uint32_t slot = __ldg(order + item);
@@ -345,7 +472,7 @@ __global__ void __launch_bounds__(kIgWarps * 32, 12) k_ig_items(gs_proj proj, gs
         tail += __popc(m);
         __syncwarp();
         const uint32_t chunks = (tail - head) / kIgBatch;
-        composite_chunks<kIgBatch>(sx, su, head, chunks, lo, p, T, cu);
+        composite_chunks<kIgBatch, kRing>(sx, su, head, chunks, lo, p, T, cu);
         head += chunks * kIgBatch;
         __syncwarp();
       }
@@ -361,7 +488,7 @@ __global__ void __launch_bounds__(kIgWarps * 32, 12) k_ig_items(gs_proj proj, gs
         su[b0 + lane] = 0.f;
       }
       __syncwarp();
-      composite_chunks<kIgBatch>(sx, su, head, 1u, lo, p, T, cu);
+      composite_chunks<kIgBatch, kRing>(sx, su, head, 1u, lo, p, T, cu);
       __syncwarp();
     }
     float sum = cu;

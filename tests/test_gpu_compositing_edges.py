@@ -97,3 +97,22 @@ def test_items_beyond_the_ordered_capacity(capacity):
     for k in ("dmo", "dsu", "dq", "drgb"):      # (sums of atomics: equal up to their order)
         a, b = out[0][1][k], out[1][1][k]
         assert float((a - b).abs().max()) <= 1e-4 * float(a.abs().max())
+
+
+@pytest.mark.parametrize("logit", [-6.5, -2.0])     # nothing saturates; everything does, early in the list
+@pytest.mark.parametrize("n", [1023, 1025, 1120, 1153, 2500, 4099])
+def test_long_lists_of_the_information_gain(n, logit):
+    """Lists long enough to be shared by a block's warps (above 1,024 entries; rounds of 96): the
+    score is the oracle's, and bit for bit that of the same pixels in other tiles and chunk depths."""
+    gmap, cams = _stack(n, logit)
+    gmap.mo[:, 2] = 2.0 + np.arange(n) * np.float32(0.002)
+    gmap.mo[:, 3] = logit
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    prm = gs.RenderParams(alpha_min=1e-3)
+    ref = O.render_images(gmap, cams, O.Params(16, 16, prm.eps2d, prm.near, prm.guard, prm.alpha_min, prm.alpha_max,
+                                               prm.T_min))[0]
+    got = [float(gs.InfoGain(n, cams, gs.RenderParams(alpha_min=1e-3, ig_batch=b))(gm)[0]) for b in gs.IG_BATCH_CANDIDATES]
+    assert got[0] == got[1] == got[2]
+    # a skip or stop decision within rounding moves a pixel by at most alpha_min or T_min times u <= 1
+    slack = ref["knife"].mean() * max(prm.alpha_min, prm.T_min)
+    assert abs(got[0] - ref["unc"].mean()) <= IG_RTOL * abs(ref["unc"].mean()) + 1e-7 + slack
