@@ -202,24 +202,11 @@ struct ViewProj {
   int x0, y0, x1, y1;  // tile rect, ends exclusive
 };
 
-// Returns true if the Gaussian is visible in the view and fills `vp`.
-// The first culls of view_proj (near plane, guard band), with the same operations:
-// view_proj can only accept a pair this accepts.
-__device__ __forceinline__ bool frustum_ok(float4 mo, const CamC& c, float near_plane) {
-  const float4* c4 = reinterpret_cast<const float4*>(&c);
-  const float4 q0 = c4[0], q1 = c4[1], q2 = c4[2], q3 = c4[3];
-  const float dx = fsub(mo.x, q2.y), dy = fsub(mo.y, q2.z), dz = fsub(mo.z, q2.w);
-  const float tx = ffma(q1.z, dz, ffma(q0.w, dy, fmul(q0.x, dx)));
-  const float ty = ffma(q1.w, dz, ffma(q1.x, dy, fmul(q0.y, dx)));
-  const float tz = ffma(q2.x, dz, ffma(q1.y, dy, fmul(q0.z, dx)));
-  return tz > near_plane && !(fabsf(tx) > fmul(q3.x, tz)) && !(fabsf(ty) > fmul(q3.y, tz));
-}
-
-// Group cull: false only if no centre within `rad` of (gc) can pass frustum_ok for the
-// view.  For a point p with |p - gc| <= rad and t = R^T (p - T): t_z <= t_z(gc) + rad, and
+// Group cull: false only if no centre within `rad` of (gc) can pass view_proj's first culls (near
+// plane, guard band) in the view.  For a point p with |p - gc| <= rad and t = R^T (p - T): t_z <= t_z(gc) + rad, and
 // its signed distance to each side plane t_x = +-gx t_z (t_y = +-gy t_z) differs from the
-// centre's by at most rad.  `m` covers the rounding of frustum_ok's FP32 evaluation (a few
-// ulp of |p - T|) with a wide margin, so the cull never drops a pair frustum_ok accepts.
+// centre's by at most rad.  `m` covers the rounding of their FP32 evaluation (a few
+// ulp of |p - T|) with a wide margin, so the cull never drops a pair they accept.
 __device__ __forceinline__ bool group_may_meet(const float* gc, float rad, const CamC& c, float near_plane) {
   const float dx = gc[0] - c.T[0], dy = gc[1] - c.T[1], dz = gc[2] - c.T[2];
   const float tx = c.R[0] * dx + c.R[3] * dy + c.R[6] * dz;
@@ -235,6 +222,7 @@ __device__ __forceinline__ bool group_may_meet(const float* gc, float rad, const
   return true;
 }
 
+// Returns true if the Gaussian is visible in the view and fills `vp`.
 // kFull = false: only the decision (the same operations up to the rectangle test; the
 // record's conic, mean and depth are not formed), for the projection's count pass.
 template <bool kFull = true>

@@ -118,6 +118,41 @@ __device__ __forceinline__ void stage_cams(const gs_camera* __restrict__ cams, c
   }
 }
 
+// view_proj's decision where it is clear without the covariance: 0 not visible, 1 visible, 2 take
+// view_proj.  The near plane and guard band are decided with its own operations; the rest has margins
+// far above the rounding of either side:
+//  - the covariance's diagonal without the low-pass is at most ax = tr(Sigma) (f_x / t_z)^2 (1 + u^2)
+//    (ay alike), so a mean further outside the image than sqrt(Q (ax + eps2d)) reaches no pixel;
+//  - for a mean inside the image, rx, ry >= 0.51 px (Q eps2d 0.9 >= 0.27) reach the nearest pixel
+//    centre; and det > 0 holds for ax, ay <= 1e4 eps2d: the exact det is at least eps2d (a + c -
+//    eps2d), the rounding of a, b, c at most about 5e-6 of ax, ay, so that of det is below a tenth.
+// trS: trace of the 3D covariance.  Non-finite values satisfy no comparison and give 2.
+// Count pass: 436 -> 350 us (1M Gaussians, 256 views), 2,025 -> 1,263 us (3M, 384 views).
+__device__ __forceinline__ int quick_vis(float4 mo, float trS, float Q, const CamC& c, float near_plane,
+                                         float eps2d) {
+  const float4* c4 = reinterpret_cast<const float4*>(&c);
+  const float4 q0 = c4[0], q1 = c4[1], q2 = c4[2], q3 = c4[3];
+  const float dx = fsub(mo.x, q2.y), dy = fsub(mo.y, q2.z), dz = fsub(mo.z, q2.w);
+  const float tx = ffma(q1.z, dz, ffma(q0.w, dy, fmul(q0.x, dx)));
+  const float ty = ffma(q1.w, dz, ffma(q1.x, dy, fmul(q0.y, dx)));
+  const float tz = ffma(q2.x, dz, ffma(q1.y, dy, fmul(q0.z, dx)));
+  if (!(tz > near_plane) || fabsf(tx) > fmul(q3.x, tz) || fabsf(ty) > fmul(q3.y, tz)) return 0;
+  const float iz = __fdividef(1.f, tz);
+  const float u = tx * iz, v = ty * iz, jx = q3.z * iz, jy = q3.w * iz;
+  const float mx = q3.z * u + c.cx, my = q3.w * v + c.cy;
+  const float ax = trS * jx * jx * (1.f + u * u), ay = trS * jy * jy * (1.f + v * v);
+  const float W = (float)c.W, H = (float)c.H;
+  if (!(tz < 1e30f)) return 2;   // (the reciprocal may be flushed)
+  const float ex = 0.05f + 2e-6f * W, ey = 0.05f + 2e-6f * H;
+  if (mx >= ex && mx <= W - ex && my >= ey && my <= H - ey && Q * (0.9f * eps2d) >= 0.27f &&
+      fmaxf(ax, ay) <= 1e4f * eps2d)
+    return 1;
+  const float rx = sqrtf(Q * (ax + eps2d)) * 1.01f + 1.f + 1e-6f * fabsf(c.cx);
+  const float ry = sqrtf(Q * (ay + eps2d)) * 1.01f + 1.f + 1e-6f * fabsf(c.cy);
+  if (mx + rx < 0.f || mx - rx > W || my + ry < 0.f || my - ry > H) return 0;
+  return 2;
+}
+
 // Records written and the overflow flag, from the scanned offsets.
 __device__ __forceinline__ void record_count(const gs_proj& out, int64_t n_slots) {
   const uint32_t total = out.grp_base[n_slots];
@@ -126,9 +161,9 @@ __device__ __forceinline__ void record_count(const gs_proj& out, int64_t n_slots
 }
 
 // One warp = one group of 32 consecutive Gaussians.  For every view the lanes
-// test their Gaussian cheaply (near plane, guard band: frustum_ok; in the write
-// pass, the count pass's visibility bit) and queue the (view, lane) pairs that
-// pass in shared memory; whenever 32 are queued, each lane takes one and runs the
+// test their Gaussian cheaply (quick_vis: near plane, guard band, and the pairs that are clear
+// without the covariance; in the write pass, the count pass's visibility bit) and queue the
+// (view, lane) pairs that are left in shared memory; whenever 32 are queued, each lane takes one and runs the
 // full projection, so the expensive EWA path runs with every lane busy whatever
 // the fraction of Gaussians a view sees.  Count pass: the visible lanes of each
 // (view, group) become a ballot mask (grp_mask, entry view * G + group) and its
@@ -169,6 +204,7 @@ __global__ void __launch_bounds__(kBlock) k_project(gs_map map, const gs_camera*
   s_g[warp][2][lane] = make_float4(pre.S[4], pre.S[5], pre.Q, pre.o);
   s_g[warp][3][lane] = make_float4(col.x, col.y, col.z, su.w);
   const bool usable = active && pre.valid;
+  const float trS = usable ? pre.S[0] + pre.S[3] + pre.S[5] : 0.f;
   uint32_t* queue = s_q[warp];
   uint32_t* vmask = s_mask[warp];
   // count pass: a sphere holding the centres of the group's usable Gaussians, for the group
@@ -260,8 +296,15 @@ __global__ void __launch_bounds__(kBlock) k_project(gs_map map, const gs_camera*
         const int i = vb + __ffs(cm) - 1;
         cm &= cm - 1u;
         bool take;
-        if (kWrite) take = (vmask[i] >> lane) & 1u;
-        else take = usable && frustum_ok(mo, s_cam[i], p.near_plane);
+        if (kWrite) {
+          take = (vmask[i] >> lane) & 1u;
+        } else {
+          const int d = usable ? quick_vis(mo, trS, pre.Q, s_cam[i], p.near_plane, p.eps2d) : 0;
+          const uint32_t sure = __ballot_sync(0xffffffffu, d == 1);
+          if (lane == 0 && sure) vmask[i] |= sure;   // (drain adds to other lanes' bits only between these)
+          __syncwarp();
+          take = d == 2;
+        }
         const uint32_t m = __ballot_sync(0xffffffffu, take);
         if (take) queue[qn + __popc(m & lt)] = ((uint32_t)i << 5) | (uint32_t)lane;
         qn += __popc(m);
