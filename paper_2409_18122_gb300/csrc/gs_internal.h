@@ -9,6 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "../../include/gs.h"
+#include "smem_limit.h"
 
 namespace gs {
 

@@ -436,13 +436,10 @@ cudaError_t launch_image_loss(const int32_t* sizes, int n_views, const float* rg
     for (int j = 0; j < kWin; ++j) a.g[j] = (float)(gw[j] / sum);
   }
 
-  static bool attr_set = false;
-  if (ssim && !attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_loss_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_loss_ssim_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwdSmem);
+  if (ssim) {
+    cudaError_t e = allow_smem<k_loss_fwd>(kFwdSmem);
+    if (e == cudaSuccess) e = allow_smem<k_loss_ssim_bwd>(kBwdSmem);
     if (e != cudaSuccess) return e;
-    attr_set = true;
   }
   int64_t pix = 0, slot = 0;
   if (!ssim) {

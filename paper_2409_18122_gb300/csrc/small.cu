@@ -295,13 +295,8 @@ __global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_
 
 cudaError_t launch_render_small(const gs_map& map, const gs_camera* cams, int n_views, const gs_params& p,
                                 const gs_image& img, uint32_t* status, cudaStream_t st) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(k_render_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSmem));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  const cudaError_t e = allow_smem<k_render_small>(sizeof(SmallSmem));
+  if (e != cudaSuccess) return e;
   // one CTA per SM walks the tiles of all views with a fixed stride (the number of tiles
   // lives in the cameras, in device memory)
   launch(k_render_small, (unsigned)device_sm_count(), kThreads, sizeof(SmallSmem), st, map, cams, n_views, p, img,

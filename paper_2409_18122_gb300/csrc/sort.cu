@@ -445,13 +445,8 @@ struct SortArgs {
 template <int kPass, int kItems>
 cudaError_t sort_pass(const SortArgs& a, const uint32_t* keys_in, const uint32_t* vals_in, uint32_t* keys_out,
                       uint32_t* vals_out, const SortRectEpilogue& epi) {
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e = cudaFuncSetAttribute(k_downsweep<kPass, kItems>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)down_smem(kItems));
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  const cudaError_t e = allow_smem<k_downsweep<kPass, kItems>>(down_smem(kItems));
+  if (e != cudaSuccess) return e;
   launch(k_upsweep<kPass>, a.g, kBlock, 0, a.st, keys_in, a.seg, a.n_seg, a.pmap, a.ctl, a.hist);
   launch(k_scan_hist<kPass>, dim3(a.n_seg, kRadix / 32), 1024, 0, a.st, a.hist, a.g, a.pmap, a.ctl, a.tot);
   launch(k_downsweep<kPass, kItems>, a.g, kBlock, down_smem(kItems), a.st, keys_in, vals_in, a.seg, a.n_seg, a.pmap,
