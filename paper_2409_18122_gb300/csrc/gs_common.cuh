@@ -43,11 +43,11 @@ struct __align__(16) CamC {
   float fx, fy;
   float cx, cy;
   int W, H;
-  int tw, th;            // this view's tile size (powers of two)
-  int sx, sy;            // log2 of tw, th
+  int sx, sy;            // log2 of this view's tile width and height
   int tiles_x, tiles_y;
   uint32_t tile_base;
   uint32_t pix_base;
+  float stretch;         // bound of |R^T x| / |x| (rotation_stretch): 1 up to rounding for a rotation
 };
 
 // ---------------------------------------------------------------- float math
@@ -202,18 +202,34 @@ struct ViewProj {
   int x0, y0, x1, y1;  // tile rect, ends exclusive
 };
 
+// Bound of |R^T x| / |x|, at least 1: the root of the largest row sum of |R^T R|.  The culls that
+// bound lengths in the camera's frame scale by it, so that they hold for every matrix a camera may
+// carry, not for rotations alone (a scaled pose is taken as its arithmetic says).
+__device__ __forceinline__ float rotation_stretch(const float* R) {
+  float most = 1.f;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    float s = 0.f;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) s += fabsf(R[i] * R[j] + R[3 + i] * R[3 + j] + R[6 + i] * R[6 + j]);
+    most = fmaxf(most, s);
+  }
+  return sqrtf(most);
+}
+
 // Group cull: false only if no centre within `rad` of (gc) can pass view_proj's first culls (near
-// plane, guard band) in the view.  For a point p with |p - gc| <= rad and t = R^T (p - T): t_z <= t_z(gc) + rad, and
-// its signed distance to each side plane t_x = +-gx t_z (t_y = +-gy t_z) differs from the
-// centre's by at most rad.  `m` covers the rounding of their FP32 evaluation (a few
-// ulp of |p - T|) with a wide margin, so the cull never drops a pair they accept.
+// plane, guard band) in the view.  For a point p with |p - gc| <= rad and t = R^T (p - T), t differs
+// from the centre's by at most r = stretch * rad: t_z <= t_z(gc) + r, and its signed distance to each
+// side plane t_x = +-gx t_z (t_y = +-gy t_z) differs from the centre's by at most r.  `m` covers the
+// rounding of their FP32 evaluation (a few ulp of |p - T|) with a wide margin, so the cull never
+// drops a pair they accept.
 __device__ __forceinline__ bool group_may_meet(const float* gc, float rad, const CamC& c, float near_plane) {
   const float dx = gc[0] - c.T[0], dy = gc[1] - c.T[1], dz = gc[2] - c.T[2];
   const float tx = c.R[0] * dx + c.R[3] * dy + c.R[6] * dz;
   const float ty = c.R[1] * dx + c.R[4] * dy + c.R[7] * dz;
   const float tz = c.R[2] * dx + c.R[5] * dy + c.R[8] * dz;
   const float m = 1e-4f * (fabsf(dx) + fabsf(dy) + fabsf(dz) + rad) + 1e-4f;
-  const float r = rad + m;
+  const float r = (rad + m) * c.stretch;
   if (tz + r <= near_plane) return false;
   const float kx = r * sqrtf(1.f + c.gx * c.gx) * 1.0001f;
   const float ky = r * sqrtf(1.f + c.gy * c.gy) * 1.0001f;
@@ -300,8 +316,6 @@ __device__ __forceinline__ void view_tile(const gs_camera& g, int def_w, int def
 __device__ __forceinline__ void load_cam(const gs_camera& g, float guard, int def_tw, int def_th, CamC& c) {
   int tile_w, tile_h;
   view_tile(g, def_tw, def_th, tile_w, tile_h);
-  c.tw = tile_w;
-  c.th = tile_h;
   c.sx = __ffs(tile_w) - 1;
   c.sy = __ffs(tile_h) - 1;
   c.fx = g.fx; c.fy = g.fy; c.cx = g.cx; c.cy = g.cy;
@@ -311,6 +325,7 @@ __device__ __forceinline__ void load_cam(const gs_camera& g, float guard, int de
   for (int i = 0; i < 3; ++i) c.T[i] = g.T[i];
   c.W = g.width;
   c.H = g.height;
+  c.stretch = 1.f;   // (set by the projection, whose culls use it)
   c.gx = fdiv(fmul(guard, fmul(0.5f, (float)g.width)), g.fx);
   c.gy = fdiv(fmul(guard, fmul(0.5f, (float)g.height)), g.fy);
   c.tiles_x = (g.width + tile_w - 1) / tile_w;

@@ -108,7 +108,10 @@ __device__ __forceinline__ void stage_cams(const gs_camera* __restrict__ cams, c
     const gs_camera g = cams[v0 + i];
     CamC c;
     load_cam(g, p.guard, p.tile_w, p.tile_h, c);
-    if (!camera_ok(g, c.tw, c.th)) {
+    c.stretch = rotation_stretch(c.R);
+    int tw, th;
+    view_tile(g, p.tile_w, p.tile_h, tw, th);
+    if (!camera_ok(g, tw, th)) {
       c.W = 0;  // marks the view unusable
       c.H = 0;
     }
@@ -121,11 +124,12 @@ __device__ __forceinline__ void stage_cams(const gs_camera* __restrict__ cams, c
 // view_proj's decision where it is clear without the covariance: 0 not visible, 1 visible, 2 take
 // view_proj.  The near plane and guard band are decided with its own operations; the rest has margins
 // far above the rounding of either side:
-//  - the covariance's diagonal without the low-pass is at most ax = tr(Sigma) (f_x / t_z)^2 (1 + u^2)
-//    (ay alike), so a mean further outside the image than sqrt(Q (ax + eps2d)) reaches no pixel;
+//  - the covariance's diagonal without the low-pass is at most ax = stretch^2 tr(Sigma) (f_x / t_z)^2
+//    (1 + u^2) (ay alike), so a mean further outside the image than sqrt(Q (ax + eps2d)) reaches no pixel;
 //  - for a mean inside the image, rx, ry >= 0.51 px (Q eps2d 0.9 >= 0.27) reach the nearest pixel
 //    centre; and det > 0 holds for ax, ay <= 1e4 eps2d: the exact det is at least eps2d (a + c -
-//    eps2d), the rounding of a, b, c at most about 5e-6 of ax, ay, so that of det is below a tenth.
+//    eps2d), the rounding of a, b, c at most about 5e-6 of ax, ay, so that of det is below a tenth;
+//  - f_x u of a mean near the image is of the size of c_x + W, and so is the mean's rounding.
 // trS: trace of the 3D covariance.  Non-finite values satisfy no comparison and give 2.
 // Count pass: 436 -> 350 us (1M Gaussians, 256 views), 2,025 -> 1,263 us (3M, 384 views).
 __device__ __forceinline__ int quick_vis(float4 mo, float trS, float Q, const CamC& c, float near_plane,
@@ -140,10 +144,11 @@ __device__ __forceinline__ int quick_vis(float4 mo, float trS, float Q, const Ca
   const float iz = __fdividef(1.f, tz);
   const float u = tx * iz, v = ty * iz, jx = q3.z * iz, jy = q3.w * iz;
   const float mx = q3.z * u + c.cx, my = q3.w * v + c.cy;
-  const float ax = trS * jx * jx * (1.f + u * u), ay = trS * jy * jy * (1.f + v * v);
+  const float tr = trS * c.stretch * c.stretch;
+  const float ax = tr * jx * jx * (1.f + u * u), ay = tr * jy * jy * (1.f + v * v);
   const float W = (float)c.W, H = (float)c.H;
   if (!(tz < 1e30f)) return 2;   // (the reciprocal may be flushed)
-  const float ex = 0.05f + 2e-6f * W, ey = 0.05f + 2e-6f * H;
+  const float ex = 0.05f + 2e-6f * (W + fabsf(c.cx)), ey = 0.05f + 2e-6f * (H + fabsf(c.cy));
   if (mx >= ex && mx <= W - ex && my >= ey && my <= H - ey && Q * (0.9f * eps2d) >= 0.27f &&
       fmaxf(ax, ay) <= 1e4f * eps2d)
     return 1;

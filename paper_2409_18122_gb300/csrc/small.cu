@@ -217,10 +217,10 @@ __global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_
     // 2. depth order (ties keep the Gaussian-id order)
     sort_list(s, n_all);
     // 3. front-to-back compositing of the tile's 8x4 pixel blocks, one warp per block
-    const int wpr = cam.tw >> 3, nb = (cam.tw * cam.th) >> 5;
+    const int wpr = (1 << cam.sx) >> 3, nb = (1 << (cam.sx + cam.sy)) >> 5;
     const float amax = p.alpha_max;
     for (int b = warp; b < nb; b += kWarps) {
-      const int x0 = tx * cam.tw + (b % wpr) * 8, y0 = ty * cam.th + (b / wpr) * 4;
+      const int x0 = (tx << cam.sx) + (b % wpr) * 8, y0 = (ty << cam.sy) + (b / wpr) * 4;
       WarpBlock wb;
       wb.px = x0 + (lane & 7);
       wb.py = y0 + (lane >> 3);

@@ -54,3 +54,46 @@ def test_visible_sets(seed, eps2d, alpha_min):
     # every counted record was written by the write pass: ids in order, per view the visible ones
     for v in range(len(cams)):
         np.testing.assert_array_equal(rec["gid"][rec["view"] == v], np.flatnonzero(vis[v]))
+
+
+def _check_visible(gmap, cams, prm):
+    n = gmap.n
+    fr = gs.Frame(n, cams, prm)
+    fr.project(gs.GaussianMapTensors.from_numpy(gmap))
+    torch.cuda.synchronize()
+    rec = gpu_records(fr)
+    vis = O.project(gmap, cams, oparams(prm))["vis"].astype(bool)
+    n_grp = (n + 31) // 32
+    masks = rec["grp_mask"].reshape(len(cams), n_grp)
+    got = ((masks[:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(len(cams), -1)[:, :n].astype(bool)
+    np.testing.assert_array_equal(got, vis)
+    return vis
+
+
+@pytest.mark.parametrize("scale", [0.25, 1.5, 6.0])
+def test_visible_sets_of_scaled_and_sheared_cameras(scale):
+    """R is used as it is given: lengths in the camera's frame are those of R^T, also where R is not
+    a rotation (a pose with a scale, a shear), so the culls that bound them must follow it."""
+    gmap = _map(20_011, 7)
+    shear = np.array([[1.0, 0.4, -0.2], [0.0, 1.0, 0.3], [0.0, 0.1, 1.0]])
+    cams = [Camera(97.0, 97.0, 48.5, 30.5, 97, 61, (scale * m).astype(np.float32), np.zeros(3, np.float32))
+            for m in (np.eye(3), shear, np.diag([1.0, 1.0, 1.0 / scale]), np.diag([1.0 / scale, 1.0, 1.0]))]
+    vis = _check_visible(gmap, cams, gs.RenderParams())
+    assert vis[:2].sum(axis=1).min() > 1000
+
+
+def test_visible_sets_with_a_far_principal_point():
+    """A guard band of 1e5 and an image four million pixels off the optical axis: the means are
+    rounded to quarters of a pixel, of which the half-pixel supports are not independent."""
+    rng = np.random.default_rng(5)
+    n = 20_011
+    tz = rng.uniform(20.0, 60.0, n)
+    px = np.where(rng.random(n) < 0.5, rng.uniform(-1.5, 1.5, n), 97.0 + rng.uniform(-1.5, 1.5, n))
+    mo = np.stack([(px + 4.0e6) / 100.0 * tz, rng.uniform(-0.25, 0.25, n) * tz, tz, rng.uniform(-5.05, -4.9, n)], 1)
+    q = rng.standard_normal((n, 4))
+    q /= np.linalg.norm(q, axis=1, keepdims=True)
+    su = np.full((n, 4), -13.0)
+    gmap = GaussianMap(*(a.astype(np.float32) for a in (mo, su, q, np.zeros((n, 4)))))
+    cam = Camera(100.0, 100.0, -4.0e6, 30.5, 97, 61, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
+    vis = _check_visible(gmap, [cam], gs.RenderParams(guard=1.0e5))
+    assert 0.05 < vis.mean() < 0.95
