@@ -174,7 +174,7 @@ __device__ inline int64_t lower_bound_u32(const uint32_t* __restrict__ poff, int
 // first pair lies at or past P_v k / K (bounds[v (K + 1) + K] = the view's end).  One thread
 // per bound, so the binary searches run side by side instead of at the start of every warp
 // of the histogram and placement kernels.
-__global__ void k_chunk_bounds(const uint32_t* __restrict__ seg, const uint32_t* __restrict__ poff, int n_views,
+__global__ void k_chunk_bounds(const uint32_t* seg, const uint32_t* poff, int n_views,
                                int K, uint32_t* __restrict__ bounds) {
   pdl_begin();
   const int64_t nb = (int64_t)n_views * (K + 1);
@@ -284,9 +284,9 @@ __global__ void __launch_bounds__(kBinWarps * 32) k_bin_hist(const gs_proj proj,
 
 // Step 5b: ranges of every global tile from the scanned counts, the pair total
 // and the overflow flags.  Empty tiles, and tiles past the scanned range, get [0, 0).
-__global__ void k_bin_ranges(const uint32_t* __restrict__ off, const uint32_t* __restrict__ scan_n,
-                             const uint32_t* __restrict__ total, int K, int64_t pair_cap, int64_t tile_cap,
-                             const uint32_t* __restrict__ view_info, int n_views, uint32_t* __restrict__ ranges,
+__global__ void k_bin_ranges(const uint32_t* off, const uint32_t* scan_n,
+                             const uint32_t* total, int K, int64_t pair_cap, int64_t tile_cap,
+                             const uint32_t* view_info, int n_views, uint32_t* __restrict__ ranges,
                              uint32_t* __restrict__ bins_count, uint32_t* status,
                              uint32_t* __restrict__ order_cnt) {
   pdl_begin();
@@ -502,8 +502,8 @@ __device__ inline int64_t order_items(const uint32_t* __restrict__ view_info, in
 }
 
 // Items per bucket.
-__global__ void __launch_bounds__(kBlock) k_order_count(const uint32_t* __restrict__ view_info, int n_views,
-                                                        const uint32_t* __restrict__ ranges, int64_t tile_cap,
+__global__ void __launch_bounds__(kBlock) k_order_count(const uint32_t* view_info, int n_views,
+                                                        const uint32_t* ranges, int64_t tile_cap,
                                                         int64_t item_cap, bool clamp, uint32_t* __restrict__ cnt) {
   pdl_begin();
   __shared__ uint32_t s_cnt[kOrderBuckets];
@@ -518,10 +518,10 @@ __global__ void __launch_bounds__(kBlock) k_order_count(const uint32_t* __restri
 }
 
 // Every item to its bucket's next free position; one atomic per (warp, bucket).
-__global__ void __launch_bounds__(kBlock) k_order_place(const uint32_t* __restrict__ view_info, int n_views,
-                                                        const uint32_t* __restrict__ ranges, int64_t tile_cap,
+__global__ void __launch_bounds__(kBlock) k_order_place(const uint32_t* view_info, int n_views,
+                                                        const uint32_t* ranges, int64_t tile_cap,
                                                         int64_t item_cap, bool clamp,
-                                                        const uint32_t* __restrict__ cnt, uint32_t* __restrict__ cur,
+                                                        const uint32_t* cnt, uint32_t* __restrict__ cur,
                                                         uint32_t* __restrict__ order) {
   pdl_begin();
   __shared__ uint32_t s_base[kOrderBuckets];

@@ -55,6 +55,10 @@ uint64_t launch_count();
 // between kernels, which small calls are made of (some 38 launches for one view): one 640x480 view of 200k
 // Gaussians 288 -> 232 us, 27 scored candidates 750 -> 685 us, 3M Gaussians and eight 1280x720 views
 // 5.91 -> 5.85 ms.
+// Its lifetime begins before the wait, while kernels before it still write, so nothing that they may
+// write is read-only "for the lifetime of the kernel": a kernel launched this way takes no input
+// through the non-coherent path (no __ldg, no `const ... __restrict__` parameter, which the compiler
+// reads the same way and may read early).  A kernel launched plainly may.
 template <class... P, class... A>
 inline void launch_as(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                       A&&... args) {

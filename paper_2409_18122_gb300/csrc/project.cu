@@ -31,7 +31,7 @@ __device__ __forceinline__ unsigned long long view_pixels(const gs_camera& c) {
 
 // Per-view table: tile, pixel and warp-item offsets (prefix sums over views), tile
 // sizes, camera checks.
-__global__ void __launch_bounds__(1024) k_view_info(const gs_camera* __restrict__ cams, int n_views, int def_tw,
+__global__ void __launch_bounds__(1024) k_view_info(const gs_camera* cams, int n_views, int def_tw,
                                                     int def_th, uint32_t n_groups, uint32_t* __restrict__ view_info,
                                                     uint32_t* status) {
   pdl_begin();

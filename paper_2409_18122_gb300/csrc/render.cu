@@ -499,9 +499,9 @@ __global__ void __launch_bounds__(kIgWarps * 32, 24 / kIgWarps) k_ig_items(gs_pr
 }
 
 // IG_v = (1 / P_v) * sum over the view's warp items, in a fixed order.
-__global__ void __launch_bounds__(256) k_ig_views(const uint32_t* __restrict__ view_info,
-                                                   const gs_camera* __restrict__ cams, int n_views,
-                                                   const float* __restrict__ item_sum, int64_t item_cap,
+__global__ void __launch_bounds__(256) k_ig_views(const uint32_t* view_info,
+                                                   const gs_camera* cams, int n_views,
+                                                   const float* item_sum, int64_t item_cap,
                                                    float* __restrict__ ig) {
   pdl_begin();
   __shared__ float s_red[32];

@@ -247,7 +247,9 @@ __device__ __forceinline__ bool more_items(const gs_proj& proj, int n_views, uin
 // the items, usually their number (item_capacity): `kern` gets the blocks for that many, and `rest`
 // a grid of `per_sm` blocks per multiprocessor that look for what is left of the upper bound and
 // leave when nothing is (1.7 us).  16x16 tiles have 8 items of the 32, and a block for each of the
-// other 24 took 70 us of the 1.32 ms mapping iteration of four 640x480 views.
+// other 24 took 70 us of the 1.32 ms mapping iteration of four 640x480 views.  (`rest` reads its
+// inputs as read-only although its start is overlapped: it is only overlapped with `kern`, which
+// starts plainly, after all that wrote them, and writes none of them.)
 template <class K, class... A>
 inline void launch_items(const gs_bins& bins, int64_t items, int warps, int per_sm, cudaStream_t st, K kern, K rest,
                          const A&... args) {

@@ -63,7 +63,7 @@ __device__ unsigned long long block_exclusive_scan(unsigned long long v, unsigne
   return before + x - v;
 }
 
-__global__ void __launch_bounds__(kBlock) k_scan_reduce(const uint32_t* __restrict__ in, const uint32_t* n_dev,
+__global__ void __launch_bounds__(kBlock) k_scan_reduce(const uint32_t* in, const uint32_t* n_dev,
                                                          int64_t n_cap, unsigned long long* partial) {
   pdl_begin();
   const int64_t n = count_of(n_dev, n_cap);
@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kBlock) k_scan_reduce(const uint32_t* __restri
   if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
-__global__ void __launch_bounds__(kBlock) k_scan_down(const uint32_t* __restrict__ in, uint32_t* __restrict__ out,
+__global__ void __launch_bounds__(kBlock) k_scan_down(const uint32_t* in, uint32_t* __restrict__ out,
                                                        const uint32_t* n_dev, int64_t n_cap,
                                                        const unsigned long long* partial,
                                                        uint32_t* __restrict__ total_out) {

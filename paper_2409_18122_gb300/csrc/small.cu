@@ -138,7 +138,7 @@ __device__ void sort_list(SmallSmem& s, int n) {
   }
 }
 
-__global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_camera* __restrict__ cams,
+__global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_camera* cams,
                                                            int n_views, gs_params p, gs_image img,
                                                            uint32_t* __restrict__ status) {
   pdl_begin();
@@ -178,9 +178,9 @@ __global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_
       GaussPre pre;
       ViewProj vp;
       if (g < map.n) {
-        mo = __ldg(MO + g);
-        su = __ldg(SU + g);
-        const float4 q = __ldg(Q + g);
+        mo = MO[g];
+        su = SU[g];
+        const float4 q = Q[g];
         pre = gauss_pre(mo, su, q, p.alpha_min);
         if (t == blockIdx.x && blockIdx.x == 0 &&
             !(finite4(mo) && isfinite(su.x) && isfinite(su.y) && isfinite(su.z) && finite4(q)))
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kThreads) k_render_small(gs_map map, const gs_
       int pos = s.n_list + __popc(m & lt);
       for (int w = 0; w < warp; ++w) pos += s.wsum[w];
       if (take && pos < kList) {
-        const float4 c = __ldg(RGB + g);
+        const float4 c = RGB[g];
         s.m[pos] = make_float4(vp.mx, vp.my, pack_ext(vp.rx, vp.ry), su.w);
         s.co[pos] = make_float4(vp.ca, vp.cb, vp.cc, pre.o);
         s.cd[pos] = make_float4(c.x, c.y, c.z, vp.depth);

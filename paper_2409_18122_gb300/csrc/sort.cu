@@ -67,7 +67,7 @@ __device__ inline int64_t count_of(const uint32_t* n_dev, int64_t n_cap) {
 // Partition map: pmap[0] = partition size, pmap[1 + s] = first
 // partition of segment s (s = 0 .. n_seg).  Segment s of n_s elements gets
 // ceil(n_s / size) partitions; size is chosen so that all fit in the grid.
-__global__ void __launch_bounds__(1024) k_part_map(const uint32_t* __restrict__ seg, int n_seg, const uint32_t* n_dev,
+__global__ void __launch_bounds__(1024) k_part_map(const uint32_t* seg, int n_seg, const uint32_t* n_dev,
                                                    int64_t n_cap, int grid, int tile, uint32_t* __restrict__ pmap,
                                                    uint32_t* __restrict__ ctl) {
   pdl_begin();
@@ -146,9 +146,9 @@ __device__ __forceinline__ uint32_t digit_of(uint32_t key, uint32_t base) {
 // (1) digit counts of each partition: hist[part][digit]; the first pass also finds the smallest
 // and largest key.
 template <int kPass>
-__global__ void __launch_bounds__(kBlock) k_upsweep(const uint32_t* __restrict__ keys,
-                                                    const uint32_t* __restrict__ seg, int n_seg,
-                                                    const uint32_t* __restrict__ pmap, uint32_t* __restrict__ ctl,
+__global__ void __launch_bounds__(kBlock) k_upsweep(const uint32_t* keys,
+                                                    const uint32_t* seg, int n_seg,
+                                                    const uint32_t* pmap, uint32_t* __restrict__ ctl,
                                                     uint32_t* __restrict__ hist) {
   pdl_begin();
   constexpr int kCopies = kWarps / 2;   // two warps share a copy of the counts
@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(kBlock) k_upsweep(const uint32_t* __restrict__
 // takes 14 us.
 template <int kPass>
 __global__ void __launch_bounds__(1024) k_scan_hist(uint32_t* __restrict__ hist, int g,
-                                                    const uint32_t* __restrict__ pmap,
-                                                    const uint32_t* __restrict__ ctl, uint32_t* __restrict__ tot) {
+                                                    const uint32_t* pmap,
+                                                    const uint32_t* ctl, uint32_t* __restrict__ tot) {
   pdl_begin();
   __shared__ uint32_t s_sum[32][33];
   if (kPass == 3 && sorted_in_three(ctl)) return;
@@ -265,15 +265,15 @@ __device__ __forceinline__ uint32_t block_exclusive(uint32_t v, uint32_t* wsum) 
 // (3) stable scatter of each partition's tiles.  The last pass writes the record indices, their
 // rectangles and pair counts (SortRectEpilogue) instead of keys and values.
 template <int kPass, int kItems>
-__global__ void __launch_bounds__(kBlock, kItems > 8 ? 2 : 4) k_downsweep(const uint32_t* __restrict__ keys_in,
-                                                          const uint32_t* __restrict__ vals_in,
-                                                          const uint32_t* __restrict__ seg, int n_seg,
-                                                          const uint32_t* __restrict__ pmap,
-                                                          const uint32_t* __restrict__ ctl,
+__global__ void __launch_bounds__(kBlock, kItems > 8 ? 2 : 4) k_downsweep(const uint32_t* keys_in,
+                                                          const uint32_t* vals_in,
+                                                          const uint32_t* seg, int n_seg,
+                                                          const uint32_t* pmap,
+                                                          const uint32_t* ctl,
                                                           uint32_t* __restrict__ keys_out,
                                                           uint32_t* __restrict__ vals_out,
-                                                          const uint32_t* __restrict__ hist,
-                                                          const uint32_t* __restrict__ tot,
+                                                          const uint32_t* hist,
+                                                          const uint32_t* tot,
                                                           const SortRectEpilogue epi) {
   pdl_begin();
   constexpr int kTile = kBlock * kItems;

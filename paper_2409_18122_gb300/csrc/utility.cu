@@ -100,7 +100,7 @@ __device__ __forceinline__ bool group_may_see(float gx, float gy, float gz, floa
 }
 
 // u_i = |mu_cur - mu_prev| (or its square); unchanged means keep their u.
-__global__ void k_uncertainty_update(const float4* __restrict__ mo_prev, const float4* __restrict__ mo_cur,
+__global__ void k_uncertainty_update(const float4* mo_prev, const float4* mo_cur,
                                      float4* __restrict__ su, int64_t n, int squared) {
   pdl_begin();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kMomThreads) k_u_moments(const float4* __restr
 }
 
 // stats = (mean, sigma, t_high = mean + sigma/2, t_low = mean - sigma/2, count); 96 threads
-__global__ void __launch_bounds__(96) k_u_finish(const double* __restrict__ part, int g, double* __restrict__ stats) {
+__global__ void __launch_bounds__(96) k_u_finish(const double* part, int g, double* __restrict__ stats) {
   pdl_begin();
   __shared__ double s[3];
   const int warp = threadIdx.x >> 5;
@@ -322,8 +322,8 @@ __global__ void __launch_bounds__(kBlock) k_view_utility(const float4* __restric
 // One warp per view adds the g blocks' partials (lanes take every 32nd, then a fixed tree).
 // One thread per view, walking all partials by itself, took 41 us for 256 views.
 template <bool kSum>
-__global__ void __launch_bounds__(kBlock) k_view_utility_finish(const uint32_t* __restrict__ cnt_part,
-                                                                const float* __restrict__ sum_part, int g,
+__global__ void __launch_bounds__(kBlock) k_view_utility_finish(const uint32_t* cnt_part,
+                                                                const float* sum_part, int g,
                                                                 int n_views, float lambda, float* __restrict__ xi,
                                                                 uint32_t* __restrict__ counts) {
   pdl_begin();
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(kBlock) k_regions(const float4* __restrict__ m
   if (lane < n_tab) atomicAdd(&count[tab], cnt);
 }
 
-__global__ void k_region_mean(const double* __restrict__ sum, const uint32_t* __restrict__ count, int64_t n_reg,
+__global__ void k_region_mean(const double* sum, const uint32_t* count, int64_t n_reg,
                               float* __restrict__ omega) {
   pdl_begin();
   for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n_reg; r += (int64_t)gridDim.x * blockDim.x)
@@ -453,7 +453,7 @@ __global__ void k_region_mean(const double* __restrict__ sum, const uint32_t* __
 
 // Trajectory information (Eq. traj_utility): per trajectory the sum over its states
 // of xi (states l = 0..L in order, FP64), and the first trajectory with the largest sum.
-__global__ void k_traj_sum(const float* __restrict__ xi, int n_traj, int n_states, float* __restrict__ out,
+__global__ void k_traj_sum(const float* xi, int n_traj, int n_states, float* __restrict__ out,
                            int32_t* __restrict__ best) {
   pdl_begin();
   __shared__ double s_best[256];
@@ -669,9 +669,9 @@ __global__ void __launch_bounds__(kBlock) k_collision(const float4* __restrict__
 constexpr int kColSamples = 2048;
 constexpr int kSeedThreads = 512;
 
-__global__ void __launch_bounds__(kSeedThreads) k_collision_seed(const float4* __restrict__ mo,
-                                                                 const float4* __restrict__ su, int64_t n,
-                                                                 const float4* __restrict__ pts, float r_robot,
+__global__ void __launch_bounds__(kSeedThreads) k_collision_seed(const float4* mo,
+                                                                 const float4* su, int64_t n,
+                                                                 const float4* pts, float r_robot,
                                                                  float lambda_g, float ground_z,
                                                                  float* __restrict__ margin,
                                                                  uint32_t* __restrict__ hit) {
