@@ -503,6 +503,12 @@ __device__ __forceinline__ bool pair_collides(const float4& p, const float4& mu,
 constexpr int kColChunk = 2048;               // Gaussians per block of the collision kernel
 constexpr int kColGroups = kColChunk / 32;    // groups of 32, each with a bounding sphere
 static_assert(kColGroups == 64, "two groups per lane below");
+// A point to which more groups than this still matter after its nearest one takes the whole chunk
+// instead.  Whole, a group of 32 costs about 17 instructions (the pair test; every lane keeps its own
+// minimum), chosen group by group about 50 (the test, a vote, five exchanges with minima, the bounds
+// again), so the line lies near 64 x 17 / 50 = 22; 12 and 20 measure alike, 32 is slower by up to a
+// quarter.
+constexpr int kColAll = 12;
 
 // Each block stages a chunk of Gaussians (mu, gamma) with a sphere (centre, radius + largest
 // gamma) around every 32 of them and one around the chunk.  |p - c| - radius - gamma bounds
@@ -513,9 +519,11 @@ static_assert(kColGroups == 64, "two groups per lane below");
 // first, one Gaussian per lane.  The results are the minimum margin over all Gaussians and
 // whether some Gaussian has |p - mu|^2 < gamma^2 (separately rounded FP32), whatever the
 // order, because what is skipped can change neither.
+// A map in random order has wide spheres, so most groups matter to most points, which then take whole
+// chunks (kColAll): 3M shuffled Gaussians and 129 points 1,200 -> 316 us, 1,000 points 9,050 -> 2,260
+// us (every pair with one point per thread: 466 and 2,640 us); in patches 60 -> 45 us and 183 -> 134.
 // Bound: the staging (32 B and an exponential per Gaussian) and the latency of the chain of
-// evaluations near the points.  A map in random order has wide spheres and evaluates most
-// groups.  3M Gaussians, 129 points: 453 us with every pair evaluated (one point per thread),
+// evaluations near the points.  3M Gaussians, 129 points: 453 us with every pair evaluated (one point per thread),
 // 153 us with groups of 32 only, 96 us with first bounds, 64 us with the chunk test (and 7 us for the
 // first bounds).
 __global__ void __launch_bounds__(kBlock) k_collision(const float4* __restrict__ mo, const float4* __restrict__ su,
@@ -533,13 +541,12 @@ __global__ void __launch_bounds__(kBlock) k_collision(const float4* __restrict__
 #pragma unroll 2
   for (int q = warp; q < kColGroups; q += kWarps) {   // warp-uniform
     const int64_t gi = g0 + q * 32 + lane;
-    float4 e = make_float4(0.f, 0.f, 0.f, -1.f);
+    float4 e = make_float4(INFINITY, 0.f, 0.f, -1.f);   // (infinitely far: no pair with it counts)
     if (gi < n) {
       const float4 m = mo[gi];
       const float4 s = su[gi];
-      if (m.z >= ground_z) {
-        e = make_float4(m.x, m.y, m.z, col_gamma(s, r_robot, lambda_g));
-      }
+      const float gamma = col_gamma(s, r_robot, lambda_g);
+      if (m.z >= ground_z && gamma >= 0.f) e = make_float4(m.x, m.y, m.z, gamma);
     }
     s_g[q * 32 + lane] = e;
     const bool use = e.w >= 0.f;
@@ -647,6 +654,24 @@ __global__ void __launch_bounds__(kBlock) k_collision(const float4* __restrict__
         if (lane == (q & 31)) (q < 32 ? wa : wb) = false;
         na = __ballot_sync(0xffffffffu, wa && matters(la));
         nb = __ballot_sync(0xffffffffu, wb && matters(lb));
+      }
+      if (__popc(na) + __popc(nb) > kColAll) {
+        na = nb = 0u;
+        float low = best;    // of this lane's Gaussians
+        bool in = false;
+#pragma unroll 4
+        for (int q = 0; q < kColGroups; ++q) {
+          const float4 g = s_g[q * 32 + lane];
+          const float dx = __fsub_rn(p.x, g.x), dy = __fsub_rn(p.y, g.y), dz = __fsub_rn(p.z, g.z);
+          const float d2 = __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
+          in |= d2 < __fmul_rn(g.w, g.w);
+          const float lim = fmaxf(__fadd_ru(g.w, low), 0.f);   // a smaller margin needs |p - mu| < gamma + low
+          if (d2 < lim * lim * 1.0001f) low = fminf(low, sqrtf(d2) - g.w);
+        }
+        col |= __any_sync(0xffffffffu, in) != 0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) low = fminf(low, __shfl_xor_sync(0xffffffffu, low, d));
+        best = low;
       }
       while (na | nb) {
         const int q = na ? __ffs(na) - 1 : 31 + __ffs(nb);

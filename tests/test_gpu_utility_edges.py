@@ -86,3 +86,33 @@ def test_collision_edges(n, points, order):
         np.testing.assert_array_equal(hit.cpu().numpy().astype(bool), ref_h)
         # |p - mu| - gamma in FP32: a few units in the last place of |p - mu| and gamma
         np.testing.assert_allclose(margin.cpu().numpy(), ref_m, rtol=1e-5, atol=2e-6)
+
+
+@pytest.mark.parametrize("points", [9, 33, 129, 257, 1000])
+@pytest.mark.parametrize("order", ["random", "half"])
+def test_collision_of_maps_in_random_order(order, points):
+    """Maps whose neighbours in memory are not neighbours in space: most groups matter to most
+    points, which then take whole chunks."""
+    n = 40_003
+    g = _map(n, "random" if order == "random" else "patches")
+    if order == "half":      # chunks of both kinds
+        p = np.arange(n)
+        p[n // 2:] = np.random.default_rng(1).permutation(p[n // 2:])
+        g = g.subset(p)
+    g.mo[n // 2, 0], g.mo[n // 3, 1] = np.nan, np.inf
+    rng = np.random.default_rng(points)
+    pts = np.zeros((points, 4), np.float32)
+    pts[:, :3] = rng.uniform([-1, -1, 0.0], [11, 11, 3], (points, 3))
+    pts[0, :3] = g.mo[7, :3]
+    gm = gs.GaussianMapTensors.from_numpy(g)
+    for r_robot, lam, gz in ((0.2, 3.0, float("-inf")), (0.0, 0.0, 0.5)):
+        margin, hit = gs.collision_check(gm, torch.from_numpy(pts).cuda(), r_robot, lam, gz)
+        keep = np.isfinite(g.mo[:, :3]).all(1)
+        ref_m, ref_h = O.collision_check(g.mo[keep], g.su[keep], pts, r_robot, lam, gz)
+        np.testing.assert_array_equal(hit.cpu().numpy().astype(bool), ref_h)
+        np.testing.assert_allclose(margin.cpu().numpy(), ref_m, rtol=1e-5, atol=2e-6)
+        # what the other points are does not matter
+        some = rng.choice(points, min(points, 9), replace=False)
+        for i in some:
+            m1, h1 = gs.collision_check(gm, torch.from_numpy(pts[i:i + 1]).cuda(), r_robot, lam, gz)
+            assert float(m1[0]) == float(margin[i]) and int(h1[0]) == int(hit[i])
