@@ -332,15 +332,21 @@ __global__ void __launch_bounds__(kLossThreads) k_loss_l1(const L1Array colour, 
   const L1Array a = is_c ? colour : depth;
   const int64_t b0 = (int64_t)(is_c ? blockIdx.x : blockIdx.x - nb_c) * chunk;
   const int64_t b1 = b0 + chunk < a.n ? b0 + chunk : a.n;
-  const float* __restrict__ x = a.x;
-  const float* __restrict__ y = a.y;
-  float* __restrict__ g = a.g;
   float acc = 0.f;
-#pragma unroll 4
-  for (int64_t i = b0 + threadIdx.x; i < b1; i += kLossThreads) {
-    const float d = x ? x[i] - y[i] : 0.f;
-    acc += fabsf(d);
-    if (g) g[i] = a.w * sgnf(d) * inv_n;
+  // four elements' loads in flight at a time (the compiler cannot know that the stores leave x and y alone)
+  for (int64_t i0 = b0 + threadIdx.x; i0 < b1; i0 += 4 * kLossThreads) {
+    float d[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t i = i0 + k * kLossThreads;
+      d[k] = a.x && i < b1 ? a.x[i] - a.y[i] : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t i = i0 + k * kLossThreads;
+      acc += fabsf(d[k]);
+      if (a.g && i < b1) a.g[i] = a.w * sgnf(d[k]) * inv_n;
+    }
   }
   block_partial(0.f, is_c ? acc : 0.f, is_c ? 0.f : acc, part + 3 * (int64_t)blockIdx.x);
 }
