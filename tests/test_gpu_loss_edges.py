@@ -33,3 +33,15 @@ def test_flat_images(x, y):
     torch.cuda.synchronize()
     L = O.mapping_loss_views(rgbs, d, rrefs, d, *gs.EQ3_WEIGHTS)[0]
     np.testing.assert_allclose(float(loss[0]), L, rtol=2e-5, atol=2e-6)
+
+
+@pytest.mark.parametrize("h", [2, 6, 7, 8, 14, 43, 44, 45, 47, 49, 50, 61, 62, 108 + 43, 108 + 44])
+def test_heights_that_end_inside_a_tile(h):
+    """Only the input rows that some output row of the view takes are blurred (height of the last
+    tile + 10, at most 64), seven output rows per warp: heights on both sides of each."""
+    sizes = [(35, h), (70, h + 1)]
+    loss, g_rgb, g_depth, ref, (rgbs, rrefs) = _run(sizes, gs.EQ3_WEIGHTS, seed=h)
+    L, l1d, l1c, ss, gr, gd = ref
+    np.testing.assert_allclose(loss, [L, l1d, l1c, ss], rtol=2e-5)
+    _check_grad(g_rgb, gr, _ssim_part(rgbs, rrefs, sizes, 0.1))
+    np.testing.assert_allclose(g_depth, np.concatenate([g.reshape(-1) for g in gd]), rtol=1e-6, atol=0)
