@@ -32,9 +32,13 @@ constexpr int kWarps = kBlock / 32;
 // keys, 8 keys or 32 bytes per digit and store on average, and few open output lines; 128
 // registers, two blocks per SM): with 8 the sort of 209M records takes 10.6 instead of 6.5 ms.
 // Small ones (up to kSmallSort records): 4, more blocks on a chip they leave idle anyway (one
-// 640x480 view of 200k Gaussians: 286 instead of 306 us); equal at 2M records.
+// 640x480 view of 200k Gaussians: 286 instead of 306 us); equal at 2M records.  Segments of at most
+// kSmallSegs records, a tile and a half, also 4, however many they are: they fill no larger tile (512
+// rendered views of a 5,000-Gaussian map 2,949 -> 2,851 us, 16,384 views of 1,000 9,013 -> 8,281; at
+// 8,000 Gaussians the larger tile is 1% faster).
 constexpr int kItemsLarge = 16, kItemsSmall = 4;
 constexpr int64_t kSmallSort = 1 << 20;
+constexpr int64_t kSmallSegs = 6144;
 constexpr int kBits = 9;
 constexpr int kRadix = 1 << kBits;
 constexpr int kLastShift = 2 * kBits;    // the third digit's first bit
@@ -48,11 +52,14 @@ constexpr int kPitch = kRadix + 2;       // a warp's counts and one slot for abs
 constexpr int kFewParts = 8192, kMaxParts = 16384;
 constexpr int64_t kPartKeys = 16384;
 
-inline bool small_sort(int64_t n_cap) { return n_cap <= kSmallSort; }
-inline int tile_keys(int64_t n_cap) { return kBlock * (small_sort(n_cap) ? kItemsSmall : kItemsLarge); }
 
-inline int64_t parts_for(int64_t n_cap) {
-  const int64_t t = tile_keys(n_cap);
+inline bool small_sort(int64_t n_cap, int n_seg) { return n_cap <= kSmallSort || n_cap / n_seg <= kSmallSegs; }
+inline int tile_keys(int64_t n_cap, int n_seg) {
+  return kBlock * (small_sort(n_cap, n_seg) ? kItemsSmall : kItemsLarge);
+}
+
+inline int64_t parts_for(int64_t n_cap, int n_seg) {
+  const int64_t t = tile_keys(n_cap, n_seg);
   int64_t g = (n_cap + t - 1) / t;
   if (g < 1) g = 1;
   if (g > kFewParts) g = n_cap <= kFewParts * kPartKeys ? kFewParts : kMaxParts;
@@ -197,7 +204,10 @@ __global__ void __launch_bounds__(kBlock) k_upsweep(const uint32_t* keys,
 // the warps' sums are scanned in shared memory.  (The scatter adds the digits' bases itself.)
 // One block per segment with a thread per digit took 194 us of the 3M-Gaussian mapping
 // iteration's four passes (eight segments: eight blocks); this
-// takes 14 us.
+// takes 14 us.  At least kEachSegs segments with at most kEachParts partitions each on average are
+// blocks enough with one each (k_scan_hist_each), and sixteen of 1,024 threads for a handful of
+// partitions are a waste: 4,096 views of a 20k map 5,743 -> 4,904 us, 128 of a 100k map 609 -> 585.
+constexpr int kEachSegs = 32, kEachParts = 64;
 template <int kPass>
 __global__ void __launch_bounds__(1024) k_scan_hist(uint32_t* __restrict__ hist, int g,
                                                     const uint32_t* pmap,
@@ -244,6 +254,29 @@ __global__ void __launch_bounds__(1024) k_scan_hist(uint32_t* __restrict__ hist,
       run += c[k];
     }
   }
+}
+
+// The same with one block per segment and a thread per digit, for many segments of few partitions.
+template <int kPass>
+__global__ void __launch_bounds__(kRadix) k_scan_hist_each(uint32_t* __restrict__ hist, int g, const uint32_t* pmap,
+                                                           const uint32_t* ctl, uint32_t* __restrict__ tot) {
+  pdl_begin();
+  if (kPass == 3 && sorted_in_three(ctl)) return;
+  const int s = blockIdx.x, d = threadIdx.x;
+  const int64_t p0 = pmap[1 + s] < (uint32_t)g ? pmap[1 + s] : g;
+  const int64_t p1 = pmap[2 + s] < (uint32_t)g ? pmap[2 + s] : g;
+  uint32_t run = 0;
+  for (int64_t p = p0; p < p1; p += 8) {
+    uint32_t c[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) c[k] = p + k < p1 ? hist[(size_t)(p + k) * kRadix + d] : 0u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (p + k < p1) hist[(size_t)(p + k) * kRadix + d] = run;
+      run += c[k];
+    }
+  }
+  tot[(size_t)s * kRadix + d] = run;
 }
 
 // Exclusive prefix over the block of one value per thread (wsum: kWarps words; ends unsynchronised).
@@ -438,6 +471,7 @@ constexpr size_t down_smem(int items) {
 struct SortArgs {
   const uint32_t* seg;
   int n_seg, g;
+  bool each;   // k_scan_hist_each
   uint32_t *pmap, *ctl, *hist, *tot;
   cudaStream_t st;
 };
@@ -448,7 +482,10 @@ cudaError_t sort_pass(const SortArgs& a, const uint32_t* keys_in, const uint32_t
   const cudaError_t e = allow_smem<k_downsweep<kPass, kItems>>(down_smem(kItems));
   if (e != cudaSuccess) return e;
   launch(k_upsweep<kPass>, a.g, kBlock, 0, a.st, keys_in, a.seg, a.n_seg, a.pmap, a.ctl, a.hist);
-  launch(k_scan_hist<kPass>, dim3(a.n_seg, kRadix / 32), 1024, 0, a.st, a.hist, a.g, a.pmap, a.ctl, a.tot);
+  if (a.each)
+    launch(k_scan_hist_each<kPass>, a.n_seg, kRadix, 0, a.st, a.hist, a.g, a.pmap, a.ctl, a.tot);
+  else
+    launch(k_scan_hist<kPass>, dim3(a.n_seg, kRadix / 32), 1024, 0, a.st, a.hist, a.g, a.pmap, a.ctl, a.tot);
   launch(k_downsweep<kPass, kItems>, a.g, kBlock, down_smem(kItems), a.st, keys_in, vals_in, a.seg, a.n_seg, a.pmap,
          a.ctl, keys_out, vals_out, a.hist, a.tot, epi);
   return cudaSuccess;
@@ -466,7 +503,7 @@ cudaError_t sort_passes(const SortArgs& a, const uint32_t* keys, const SortBufs&
 }  // namespace
 
 size_t record_sort_temp_bytes(int64_t n_cap, int n_seg) {
-  const int64_t g = parts_for(n_cap) + n_seg;
+  const int64_t g = parts_for(n_cap, n_seg) + n_seg;
   return align_up(sizeof(uint32_t) * kRadix * g, 256) + align_up(sizeof(uint32_t) * kRadix * n_seg, 256) +
          align_up(sizeof(uint32_t) * (n_seg + 2), 256);
 }
@@ -477,15 +514,16 @@ cudaError_t record_sort(const uint32_t* keys, SortBufs b, const uint32_t* n_dev,
   SortArgs a;
   a.seg = seg;
   a.n_seg = n_seg;
-  a.g = (int)(parts_for(n_cap) + n_seg);
+  a.g = (int)(parts_for(n_cap, n_seg) + n_seg);
+  a.each = n_seg >= kEachSegs && parts_for(n_cap, n_seg) / n_seg <= kEachParts;
   Carver c(temp);
   a.hist = c.take<uint32_t>((size_t)kRadix * a.g);
   a.tot = c.take<uint32_t>((size_t)kRadix * n_seg);
   a.pmap = c.take<uint32_t>(n_seg + 2);
   a.ctl = ctl;
   a.st = st;
-  launch(k_part_map, 1, 1024, 0, st, seg, n_seg, n_dev, n_cap, a.g, tile_keys(n_cap), a.pmap, ctl);
-  const cudaError_t e = small_sort(n_cap) ? sort_passes<kItemsSmall>(a, keys, b, epi) : sort_passes<kItemsLarge>(a, keys, b, epi);
+  launch(k_part_map, 1, 1024, 0, st, seg, n_seg, n_dev, n_cap, a.g, tile_keys(n_cap, n_seg), a.pmap, ctl);
+  const cudaError_t e = small_sort(n_cap, n_seg) ? sort_passes<kItemsSmall>(a, keys, b, epi) : sort_passes<kItemsLarge>(a, keys, b, epi);
   if (e != cudaSuccess) return e;
   *out = SortedRecords{b.vals_b, b.vals_a, ctl};
   return cudaGetLastError();

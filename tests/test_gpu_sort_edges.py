@@ -33,3 +33,29 @@ def test_tile_and_span_edges(n, top, base, large):
     assert (fr.rec_capacity > 1 << 20) == large
     _check_bins(fr, rec, cams)
     fr.check_status()
+
+
+@pytest.mark.parametrize("views", [31, 32, 200])
+@pytest.mark.parametrize("n_cap", [3000, 6144, 6145, 40_000])
+def test_many_views(n_cap, views):
+    """Many segments of few partitions (one scan block per view), of at most a tile and a half or
+    more records (the two tile sizes), one view holding most of the records and some none."""
+    cams = [Camera(40, 40, 20, 10, 40 + 3 * (i % 5), 20) for i in range(views)]
+    rng = np.random.default_rng(n_cap + views)
+    most = int(rng.integers(0, views))
+    gid, view, rect = [], [], []
+    for v, c in enumerate(cams):
+        k = min(n_cap, 12_000) if v == most else int(rng.choice([0, 1, 33, 150]))
+        gid.append(np.sort(rng.choice(n_cap, k, replace=False)).astype(np.uint32))
+        view.append(np.full(k, v, np.uint32))
+        tx, ty = -(-c.width // 16), -(-c.height // 16)
+        x0, y0 = rng.integers(0, tx, k), rng.integers(0, ty, k)
+        rect.append(np.stack([x0, y0, x0 + 1 + rng.integers(0, tx - x0), y0 + 1 + rng.integers(0, ty - y0)], 1))
+    rec = dict(gid=np.concatenate(gid), view=np.concatenate(view), rect=np.concatenate(rect).astype(np.int32))
+    rec["dkey"] = rng.uniform(0.2, 30.0, len(rec["gid"])).astype(np.float32).view(np.uint32)
+    rec["dkey"][::3] = rec["dkey"][0]
+    rec["gid"][-1] = n_cap - 1        # (the frame's Gaussians)
+    fr = _bin_only(rec, cams)
+    assert fr.rec_capacity == n_cap * views
+    _check_bins(fr, rec, cams)
+    fr.check_status()
