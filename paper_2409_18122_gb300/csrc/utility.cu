@@ -366,7 +366,8 @@ __global__ void __launch_bounds__(kBlock) k_view_utility_finish(const uint32_t* 
 // warp keeps a table of the first kRegSlots regions it meets in its stretch of the map, with
 // one FP64 sum per slot and lane in shared memory: one addition per 32 Gaussians, and one
 // reduction and one global atomic per slot at the end.  Lanes whose region finds no slot (a
-// map in random order) add for themselves, and then meet few others on an address.
+// map in random order) add for themselves, and then meet few others on an address; a full table is
+// looked through slot by slot (region by region, 81,920 regions took 64 us instead of 60).
 // 1M Gaussians, 32 regions: 702 us with one atomic per Gaussian, now 25 us.
 constexpr int kRegSlots = 8;
 
@@ -410,6 +411,15 @@ __global__ void __launch_bounds__(kBlock) k_regions(const float4* __restrict__ m
     }
     uint32_t left = __ballot_sync(0xffffffffu, r >= 0);
     int slot = -1;
+    if (n_tab == kRegSlots) {   // a full table is looked through once, whatever the number of regions here
+#pragma unroll
+      for (int k = 0; k < kRegSlots; ++k) {
+        const uint32_t same = __ballot_sync(0xffffffffu, r == __shfl_sync(0xffffffffu, tab, k));
+        if (lane == k) cnt += __popc(same);
+        if ((same >> lane) & 1u) slot = k;
+      }
+      left = 0u;
+    }
     while (left) {
       const int rr = __shfl_sync(0xffffffffu, r, __ffs(left) - 1);
       const uint32_t same = __ballot_sync(0xffffffffu, r == rr);

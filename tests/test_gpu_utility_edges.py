@@ -116,3 +116,21 @@ def test_collision_of_maps_in_random_order(order, points):
         for i in some:
             m1, h1 = gs.collision_check(gm, torch.from_numpy(pts[i:i + 1]).cuda(), r_robot, lam, gz)
             assert float(m1[0]) == float(margin[i]) and int(h1[0]) == int(hit[i])
+
+
+@pytest.mark.parametrize("regions", [7, 8, 9, 33])
+def test_region_tables(regions):
+    """A warp's table of eight regions: not full, exactly full, overflowing, and regions that come
+    back after the table is full (in rounds of all regions, and then the first ones again)."""
+    n = 64 * 40
+    rng = np.random.default_rng(regions)
+    g = _map(n, "random")
+    r = np.arange(n) // 5 % regions
+    r[n // 2:] = rng.integers(0, regions, n - n // 2)
+    g.mo[:, 0] = r + rng.uniform(0.1, 0.9, n)
+    g.mo[:, 1:3] = 0.5
+    g.mo[::97, 0] = -1.0       # outside the grid
+    omega, count = gs.region_uncertainty(gs.GaussianMapTensors.from_numpy(g), (0.0, 0.0, 0.0), 1.0, (regions, 1, 1))
+    ref, ref_cnt = O.region_uncertainty(g.mo, g.su[:, 3], (0.0, 0.0, 0.0), 1.0, (regions, 1, 1))
+    np.testing.assert_array_equal(count.cpu().numpy(), ref_cnt)
+    np.testing.assert_allclose(omega.cpu().numpy(), ref, rtol=1e-6, atol=0)
