@@ -134,3 +134,25 @@ def test_region_tables(regions):
     ref, ref_cnt = O.region_uncertainty(g.mo, g.su[:, 3], (0.0, 0.0, 0.0), 1.0, (regions, 1, 1))
     np.testing.assert_array_equal(count.cpu().numpy(), ref_cnt)
     np.testing.assert_allclose(omega.cpu().numpy(), ref, rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("views", [1, 31, 100, 257])
+@pytest.mark.parametrize("n", [1, 65, 19_456, 19_457, 38_913, 77_825, 155_648, 155_649])
+def test_view_counts_of_maps_with_fewer_groups_than_warps(n, views):
+    """Groups shared by eight, four and two warps, one each, and more than one per warp (4,864 warps
+    on 152 multiprocessors), with view counts that do not divide; both modes."""
+    g = _map(n, "random")
+    rng = np.random.default_rng(n + views)
+    cams = [scenes.yaw_camera(*rng.uniform([0, 0, 0.5], [10, 10, 2.5]), rng.uniform(0, 6.28), 80, 60, 65.6)
+            for _ in range(views)]
+    gm = gs.GaussianMapTensors.from_numpy(g)
+    vu = gs.ViewUtility(cams)
+    st = vu.thresholds(gm).cpu().numpy()
+    vu(gm)
+    ref_xi, ref_cnt = O.view_utility(g.mo, g.su[:, 3], cams, thresholds=tuple(float(x) for x in st))
+    np.testing.assert_array_equal(vu.counts.cpu().numpy().astype(np.int64), ref_cnt)
+    np.testing.assert_array_equal(vu.xi.cpu().numpy(), ref_xi.astype(np.float32))
+    sums = vu(gm, 1).cpu().numpy()
+    ref = O.view_utility(g.mo, g.su[:, 3], cams, mode="sum")[0]
+    # positive terms through about 40 roundings to FP32 (5 + 2 per warp, 8 per block, 19 + 5 over blocks)
+    np.testing.assert_allclose(sums, ref, rtol=3e-6, atol=0)
