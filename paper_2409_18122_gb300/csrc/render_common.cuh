@@ -247,7 +247,9 @@ __device__ __forceinline__ bool more_items(const gs_proj& proj, int n_views, uin
 // the items, usually their number (item_capacity): `kern` gets the blocks for that many, and `rest`
 // a grid of `per_sm` blocks per multiprocessor that look for what is left of the upper bound and
 // leave when nothing is (1.7 us).  16x16 tiles have 8 items of the 32, and a block for each of the
-// other 24 took 70 us of the 1.32 ms mapping iteration of four 640x480 views.  (`rest` reads its
+// other 24 took 70 us of the 1.32 ms mapping iteration of four 640x480 views.  An upper bound of one
+// wave gets all its blocks at once, which costs less than a second launch (one 32x24 view, backward:
+// 28.5 -> 26.5 us, most of it the host's).  (`rest` reads its
 // inputs as read-only although its start is overlapped: it is only overlapped with `kern`, which
 // starts plainly, after all that wrote them, and writes none of them.)
 template <class K, class... A>
@@ -255,14 +257,14 @@ inline void launch_items(const gs_bins& bins, int64_t items, int warps, int per_
                          const A&... args) {
   const int64_t all = (items + warps - 1) / warps;
   int64_t blocks = all;
-  if (bins.item_order && bins.item_capacity > 0) {
+  const int64_t wave = (int64_t)per_sm * device_sm_count();
+  if (bins.item_order && bins.item_capacity > 0 && all > wave) {
     const int64_t ordered = (bins.item_capacity + warps - 1) / warps;
     if (ordered < all) blocks = ordered;
   }
   launch_spread(kern, dim3((unsigned)blocks), dim3(32 * warps), 0, st, args..., (uint32_t)items, (uint32_t)blocks);
   if (blocks < all) {
-    const int64_t most = (int64_t)per_sm * device_sm_count();
-    const int64_t n = all - blocks < most ? all - blocks : most;
+    const int64_t n = all - blocks < wave ? all - blocks : wave;
     launch(rest, dim3((unsigned)n), dim3(32 * warps), 0, st, args..., (uint32_t)items, (uint32_t)blocks);
   }
 }

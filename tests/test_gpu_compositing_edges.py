@@ -116,3 +116,28 @@ def test_long_lists_of_the_information_gain(n, logit):
     # a skip or stop decision within rounding moves a pixel by at most alpha_min or T_min times u <= 1
     slack = ref["knife"].mean() * max(prm.alpha_min, prm.T_min)
     assert abs(got[0] - ref["unc"].mean()) <= IG_RTOL * abs(ref["unc"].mean()) + 1e-7 + slack
+
+
+@pytest.mark.parametrize("capacity", [0, 1, 5, 100, 1023])
+def test_items_beyond_the_ordered_capacity_of_large_images(capacity):
+    """The same for more possible items than one wave of blocks has (128 tiles, 4,096 of 3,648),
+    where a second launch looks for the items beyond the capacity."""
+    gmap, _ = _stack(50, -1.0)
+    cam = Camera(400.0, 400.0, 125.0, 60.0, 250, 120, np.eye(3, dtype=np.float32), np.zeros(3, np.float32))
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    out = []
+    for cut in (None, capacity):
+        fr = gs.Frame(50, [cam])
+        assert fr.n_items == 1024 and fr.n_tiles == 128
+        if cut is not None:
+            fr.c_bins.item_capacity = cut
+        img = fr.forward(gm)
+        g = fr.render_bwd(gm, img, torch.ones_like(img["rgb"]), torch.ones_like(img["depth"]))
+        torch.cuda.synchronize()
+        fr.check_status()
+        out.append((img, g))
+    for k in ("rgb", "depth", "unc", "T", "last"):
+        assert torch.equal(out[0][0][k], out[1][0][k])
+    for k in ("dmo", "dsu", "dq", "drgb"):      # (sums of atomics: equal up to their order)
+        a, b = out[0][1][k], out[1][1][k]
+        assert float((a - b).abs().max()) <= 1e-4 * float(a.abs().max())
