@@ -811,7 +811,7 @@ def autotune_tiles(gmap: GaussianMapTensors, cams: Sequence, params: RenderParam
 
 
 IG_BATCH_CANDIDATES = (4, 8, 16)     # RenderParams.ig_batch
-FWD_BATCH_CANDIDATES = (1, 2, 4)     # RenderParams.fwd_batch
+FWD_BATCH_CANDIDATES = (2, 4)        # RenderParams.fwd_batch (1 is accepted and runs as 2)
 
 
 L2_FLUSH_BYTES = 256 << 20     # more than the GPU's L2: written between timed calls of the autotuners

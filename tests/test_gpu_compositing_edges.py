@@ -141,3 +141,11 @@ def test_items_beyond_the_ordered_capacity_of_large_images(capacity):
     for k in ("dmo", "dsu", "dq", "drgb"):      # (sums of atomics: equal up to their order)
         a, b = out[0][1][k], out[1][1][k]
         assert float((a - b).abs().max()) <= 1e-4 * float(a.abs().max())
+
+
+def test_chunk_depth_one_is_depth_two():
+    gmap, cams = _stack(33, 0.0)
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    a, b = (gs.Frame(33, cams, gs.RenderParams(fwd_batch=k)).forward(gm) for k in (1, 2))
+    for k in ("rgb", "depth", "unc", "T", "last"):
+        assert torch.equal(a[k], b[k])

@@ -260,3 +260,9 @@ def test_invalid_cameras_keep_their_pixels_and_lose_their_tiles():
     assert list(tx * ty) == [8 * 5, 0, 0, 0]
     assert list(np.diff(pix_base)) == [120 * 80, 64 * 48, 0, 40 * 30]
     assert tile_base[-1] == 40
+
+
+def test_autotuner_times_no_depth_twice():
+    """fwd_batch 1 runs the kernel of depth 2: timing both would choose between them on noise."""
+    assert gs.FWD_BATCH_CANDIDATES == tuple(sorted({max(b, 2) for b in (1, 2, 4)}))
+    assert len(set(gs.IG_BATCH_CANDIDATES)) == len(gs.IG_BATCH_CANDIDATES)
