@@ -21,7 +21,6 @@ constexpr int kFwdWarps = 2;   // warps (work items) per CTA: small CTAs free th
 constexpr int kIgWarps = 4;    // the same for the persistent information-gain kernel (which shares out long lists)
 constexpr int kRing = 64;      // staged entries per warp (a ring): a group of 32 and a partial chunk
 constexpr uint32_t kLongList = 1024;   // entries that a list has at least to be shared by a block's warps
-constexpr int kPix = 1;        // pixels per lane of the forward and information-gain kernels
 // Chunk depth: staged entries whose alphas are computed together, a template argument of both
 // compositing kernels chosen per launch by gs_params (forward 1, 2 or 4, default 4; 1 runs as 2,
 // the pair of one packed evaluation; information gain 4, 8 or 16, default 8)
@@ -87,9 +86,9 @@ __global__ void __launch_bounds__(kFwdWarps * 32, 12) k_render_fwd(gs_map map, g
   do {
     const uint32_t item = ordered_item(bins, proj.view_info, n_views, b * kFwdWarps + warp);
     TileInfo ti;
-    if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) continue;
+    if (!warp_item_setup(proj, bins, cams, n_views, item, ti)) continue;
     WarpBlock wb;
-    warp_block<1>(ti, wb);
+    warp_block(ti, wb);
     float* sx = s_exp[warp];
     float4* sk = s_col[warp];
     float2* su = s_up[warp];
@@ -382,7 +381,7 @@ __global__ void __launch_bounds__(kIgWarps * 32, 24 / kIgWarps) k_ig_items(gs_pr
   const uint32_t lt = (1u << lane) - 1u;
   float* sx = s_exp[warp];
   float* su = s_u[warp];
-  uint32_t n_items = proj.view_info[kVI * n_views + 2] / kPix;
+  uint32_t n_items = proj.view_info[kVI * n_views + 2];
   if ((int64_t)n_items > item_cap) n_items = (uint32_t)item_cap;
   const float4* SP = reinterpret_cast<const float4*>(proj.splat);
   const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -400,12 +399,12 @@ __global__ void __launch_bounds__(kIgWarps * 32, 24 / kIgWarps) k_ig_items(gs_pr
     if (item >= n_items) return;
     const uint32_t slot = __ldg(order + item);
     TileInfo ti;
-    if (!warp_item_setup<kPix>(proj, bins, cams, n_views, slot, ti) || ti.end - ti.beg <= long_list) {
+    if (!warp_item_setup(proj, bins, cams, n_views, slot, ti) || ti.end - ti.beg <= long_list) {
       if (warp == 0) next = item;
       break;
     }
     WarpBlock wb;
-    warp_block<kPix>(ti, wb);
+    warp_block(ti, wb);
     composite_long<kIgBatch>(ti, wb, SP, bins, p, s_exp[0], s_u[0], s_cnt, s_live, item_sum + slot);
   }
   for (;;) {
@@ -419,13 +418,12 @@ __global__ void __launch_bounds__(kIgWarps * 32, 24 / kIgWarps) k_ig_items(gs_pr
     // items are handed out longest tile list first; each writes its own slot
     const uint32_t slot = __ldg(order + item);
     TileInfo ti;
-    if (!warp_item_setup<kPix>(proj, bins, cams, n_views, slot, ti)) {
+    if (!warp_item_setup(proj, bins, cams, n_views, slot, ti)) {
       if (lane == 0) item_sum[slot] = 0.f;
       continue;
     }
     WarpBlock wb;
-    warp_block<kPix>(ti, wb);
-    static_assert(kPix == 1, "one pixel per lane: the staged exponent and the live-pixel box assume it");
+    warp_block(ti, wb);
     const float ln_amin = __logf(p.alpha_min);
     const float bx_full = wb.bx0, by_full = wb.by0;   // centre of the block's first pixel
     const float ccx = bx_full + 3.5f, ccy = by_full + 1.5f;   // centre of the 8x4 block
@@ -506,8 +504,8 @@ __global__ void __launch_bounds__(256) k_ig_views(const uint32_t* view_info,
   pdl_begin();
   __shared__ float s_red[32];
   const int v = blockIdx.x;
-  const uint32_t i0 = view_info[kVI * v + 2] / kPix;
-  uint32_t i1 = view_info[kVI * (v + 1) + 2] / kPix;
+  const uint32_t i0 = view_info[kVI * v + 2];
+  uint32_t i1 = view_info[kVI * (v + 1) + 2];
   if ((int64_t)i1 > item_cap) i1 = (uint32_t)item_cap;
   const int W = cams[v].width, H = cams[v].height;
   float s = 0.f;
@@ -543,7 +541,7 @@ cudaError_t launch_ig_items(const gs_proj& proj, const gs_bins& bins, const gs_c
 
 cudaError_t launch_render_fwd(const gs_map& map, const gs_proj& proj, const gs_bins& bins, const gs_camera* cams,
                               int n_views, const gs_params& p, const gs_image& img, cudaStream_t st) {
-  const int64_t items = bins.tile_capacity * (32 / kPix);   // upper bound: at most 32 items per tile
+  const int64_t items = bins.tile_capacity * 32;   // upper bound: at most 32 items per tile
   if (items > 0) {
     const int b = p.fwd_batch ? p.fwd_batch : kFwdBatchDefault;
     auto run = [&](auto kern, auto rest) {

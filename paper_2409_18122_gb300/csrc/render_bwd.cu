@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 12) k_render_bwd(gs_map map, g
   do {   // longest tile lists first
     const uint32_t item = ordered_item(bins, proj.view_info, n_views, b * kBwdWarps + warp);
     TileInfo ti;
-    if (!warp_item_setup<1>(proj, bins, cams, n_views, item, ti)) continue;
+    if (!warp_item_setup(proj, bins, cams, n_views, item, ti)) continue;
     WarpBlock wb;
-    warp_block<1>(ti, wb);
+    warp_block(ti, wb);
     float4* sa = s_stage[warp][0];
     float4* sb = s_stage[warp][1];
     float4* sk = s_stage[warp][2];

@@ -151,42 +151,40 @@ __device__ __forceinline__ float2 alpha_raw2(const float* pairs, uint32_t i, con
   return make_float2(ex2_approx(e.x), ex2_approx(e.y));
 }
 
-// Work item of the compositing kernels: one warp renders one 8 x (4 KP) pixel
-// block of one screen tile, KP pixels per lane (KP = 1 in every kernel: a larger
-// block per warp culls less finely, which costs more than it saves).  Block b of a tile covers columns
-// 8 (b mod (tile_w/8)) .. +7 and rows 4 KP (b div (tile_w/8)) .. +4 KP - 1;
-// lane l owns pixels (l mod 8, l div 8 + 4 q), q < KP.  Warps never wait for
-// each other: each walks its tile's list on its own and stops as soon as all of
-// its pixels are saturated.
+// Work item of the compositing kernels: one warp renders one 8x4 pixel block of one
+// screen tile, one pixel per lane (a larger block per warp culls less finely, which
+// costs more than it saves).  Block b of a tile covers columns 8 (b mod (tile_w/8)) .. +7
+// and rows 4 (b div (tile_w/8)) .. +3; lane l owns pixel (l mod 8, l div 8).  Warps
+// rarely wait for each other: each walks its tile's list on its own and stops as soon as
+// all of its pixels are saturated (long lists of the information gain are shared).
 struct WarpBlock {
-  int px, py;                   // this lane's first pixel; the others are (px, py + 4 q)
+  int px, py;                   // this lane's pixel
   float bx0, bx1, by0, by1;     // pixel-centre bounds of the warp's block
 };
 
 // Decodes warp item `item` (numbered view by view, tile by tile, block by block,
-// with tile_w * tile_h / (32 KP) items per tile) into its tile and block; lane 0
+// with tile_w * tile_h / 32 items per tile) into its tile and block; lane 0
 // computes and broadcasts.  Returns false (warp-uniform) if the item does not exist.
-template <int KP>
 __device__ __forceinline__ bool warp_item_setup(const gs_proj& proj, const gs_bins& bins, const gs_camera* cams,
                                                 int n_views, uint32_t item, TileInfo& ti) {
   const int lane = threadIdx.x & 31;
   int f[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   uint32_t pix_base = 0;
   if (lane == 0) {
-    const uint32_t total = proj.view_info[kVI * n_views + 2] / KP;
+    const uint32_t total = proj.view_info[kVI * n_views + 2];
     if (item < total) {
-      // largest v with first_item(v) / KP <= item
+      // largest v with first_item(v) <= item
       int lo = 0, hi = n_views - 1;
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (proj.view_info[kVI * mid + 2] / KP <= item) lo = mid; else hi = mid - 1;
+        if (proj.view_info[kVI * mid + 2] <= item) lo = mid; else hi = mid - 1;
       }
       const int v = lo;
       const uint32_t code = proj.view_info[kVI * v + 3];
       const int tw = (int)(code & 0xffu), th = (int)((code >> 8) & 0xffu);
       const uint32_t tx = code >> 16;
-      const uint32_t wpt = (uint32_t)(tw * th / (32 * KP));
-      const uint32_t local = item - proj.view_info[kVI * v + 2] / KP;
+      const uint32_t wpt = (uint32_t)(tw * th / 32);
+      const uint32_t local = item - proj.view_info[kVI * v + 2];
       const uint32_t lt = wpt ? local / wpt : 0u;
       const uint32_t tile = proj.view_info[kVI * v] + lt;
       if (code != 0u && wpt != 0u && (int64_t)tile < bins.tile_capacity) {
@@ -269,36 +267,17 @@ inline void launch_items(const gs_bins& bins, int64_t items, int warps, int per_
   }
 }
 
-template <int KP>
 __device__ __forceinline__ void warp_block(const TileInfo& ti, WarpBlock& wb) {
   const int lane = threadIdx.x & 31;
   const int wpr = ti.tw >> 3;
   const int blk = ti.blk;
-  const int wx = (blk % wpr) * 8, wy = (blk / wpr) * 4 * KP;
+  const int wx = (blk % wpr) * 8, wy = (blk / wpr) * 4;
   wb.px = ti.x0 + wx + (lane & 7);
   wb.py = ti.y0 + wy + (lane >> 3);
   wb.bx0 = (float)(ti.x0 + wx) + 0.5f;
   wb.bx1 = wb.bx0 + 7.f;
   wb.by0 = (float)(ti.y0 + wy) + 0.5f;
-  wb.by1 = wb.by0 + (float)(4 * KP - 1);
-}
-
-template <int KP>
-__device__ __forceinline__ bool all_done(const bool* done) {
-  bool r = true;
-#pragma unroll
-  for (int q = 0; q < KP; ++q) r = r && done[q];
-  return r;
-}
-
-// Some pixel of the lane is not saturated (the information-gain kernel keeps T = 0 for
-// saturated pixels and for pixels outside the image).
-template <int KP>
-__device__ __forceinline__ bool live(const float* T) {
-  bool r = false;
-#pragma unroll
-  for (int q = 0; q < KP; ++q) r = r || T[q] != 0.f;
-  return r;
+  wb.by1 = wb.by0 + 3.f;
 }
 
 // Can the support box of an entry contain a pixel centre of the warp's block?

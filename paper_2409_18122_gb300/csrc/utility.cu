@@ -788,7 +788,7 @@ cudaError_t launch_uncertainty_update(const float* mo_prev, const float* mo_cur,
 }
 
 size_t thresholds_ws_bytes() {
-  return align_up(sizeof(double) * 1024, 256) + align_up(sizeof(unsigned long long) * 2, 256);
+  return align_up(sizeof(double) * 1024, 256);
 }
 
 cudaError_t launch_uncertainty_thresholds(const float* mo, const float* su, int64_t n, float ground_z, double* stats,
