@@ -149,3 +149,38 @@ def test_chunk_depth_one_is_depth_two():
     a, b = (gs.Frame(33, cams, gs.RenderParams(fwd_batch=k)).forward(gm) for k in (1, 2))
     for k in ("rgb", "depth", "unc", "T", "last"):
         assert torch.equal(a[k], b[k])
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 9, 33, 61])
+def test_staged_leftovers_never_count_without_an_opacity_floor(n):
+    """alpha_min = 0 again, with infinite colours and uncertainties staged beforehand in every slot of
+    the rings (a longer stack): the forward with and without counts and the information gain at
+    every chunk depth give the oracle's values."""
+    gmap, cams = _stack(n, -1.0)
+    long, _ = _stack(200, -6.0)          # transparent: its 200 entries all pass through the ring
+    su = long.su.copy()
+    su[:, 3] = np.inf
+    hot = gs.GaussianMapTensors.from_numpy(GaussianMap(long.mo, su, long.q, np.full_like(long.rgb, np.inf)))
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    P = O.Params(16, 16, 0.3, 0.2, 1.3, 0.0, 0.99, 1e-4)
+    ref = O.render_images(gmap, cams, P)[0]
+    ok = ~ref["knife"]
+    for b in gs.FWD_BATCH_CANDIDATES:
+        prm = gs.RenderParams(alpha_min=0.0, fwd_batch=b)
+        for counts in (False, True):
+            for _ in range(3):
+                gs.Frame(200, cams, prm).forward(hot)
+            fr = gs.Frame(n, cams, prm)
+            h = images_host(fr, fr.forward(gm, fr.new_images(with_counts=counts)))[0]
+            for k in ("rgb", "unc", "T"):
+                np.testing.assert_allclose(h[k][ok], ref[k][ok], rtol=0, atol=IMG_ATOL, err_msg=k)
+            np.testing.assert_allclose(h["depth"][ok], ref["depth"][ok], rtol=0, atol=DEPTH_RTOL * (2.0 + 0.01 * n))
+            assert (h["last"] <= n).all()
+    # a pixel of a knife-edge decision moves by at most T_min times u <= 1
+    slack = ref["knife"].mean() * 1e-4
+    for b in gs.IG_BATCH_CANDIDATES:
+        prm = gs.RenderParams(alpha_min=0.0, ig_batch=b)
+        for _ in range(3):
+            gs.InfoGain(200, cams, prm)(hot)
+        ig = float(gs.InfoGain(n, cams, prm)(gm)[0])
+        assert abs(ig - ref["unc"].mean()) <= IG_RTOL * abs(ref["unc"].mean()) + 1e-7 + slack
