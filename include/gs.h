@@ -275,7 +275,7 @@ gs_status gs_render_fwd(const gs_map* map, const gs_proj* proj, const gs_bins* b
 /* gs_render_small -- the forward render of gs_render_fwd (Sec. III), from the map
  * directly, in one kernel launch and without records, bins or workspace: for maps of
  * up to a few thousand Gaussians, whose tiled render (gs_project + gs_bin_sort +
- * gs_render_fwd, about 35 kernels) is bound by launch latency.  Every CTA takes screen
+ * gs_render_fwd, 32 kernels) is bound by launch latency.  Every CTA takes screen
  * tiles, projects the whole map for the tile's view with gs_project's decision
  * arithmetic, sorts the Gaussians whose tile rectangle covers the tile by depth key
  * (ties by Gaussian id) in shared memory and composites the tile; the outputs are bit
@@ -316,10 +316,10 @@ typedef struct {
 
 /* gs_render_bwd -- Eq. (2): the adjoint of gs_render_fwd and gs_project.
  * Each tile is replayed back to front from the saved final transmittance and
- * last index (T_i = T_{i+1} / (1 - alpha_i)), keeping suffix sums
- * S = sum_{j>i} w_j x_j; dL/dalpha_i = sum_ch g_ch (x_i T_i - S_ch / (1 - alpha_i)).
- * Screen-space gradients are reduced per Gaussian with warp shuffles before one
- * atomic add per warp, then mapped through the projection to dmu, dlog s, dq
+ * last index (T_i = T_{i+1} / (1 - alpha_i)), keeping the suffix sum
+ * S = sum_{j>i} w_j (g . x_j); dL/dalpha_i = (g . x_i) T_i - S / (1 - alpha_i).
+ * Screen-space gradients are summed per Gaussian over each warp's pixels before they
+ * are added atomically, then mapped through the projection to dmu, dlog s, dq
  * (through the normalisation), dlogit and dc.  Float atomics make the last bits
  * of the result depend on scheduling.
  * ws: DEVICE workspace of gs_workspace_size(GS_OP_RENDER_BWD, ...) bytes.

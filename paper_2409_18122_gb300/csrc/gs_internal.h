@@ -52,7 +52,7 @@ uint64_t launch_count();
 // library begins with pdl_begin, which lets the next one be placed in turn (once all blocks of this
 // one have started) and then waits until everything before it in the stream has finished and its
 // writes are visible.  So the order of the work is that of plain launches; what is saved is the gap
-// between kernels, which small calls are made of (some 38 launches for one view): one 640x480 view of 200k
+// between kernels, which small calls are made of (some 32 launches for one view): one 640x480 view of 200k
 // Gaussians 288 -> 232 us, 27 scored candidates 750 -> 685 us, 3M Gaussians and eight 1280x720 views
 // 5.91 -> 5.85 ms.
 // Its lifetime begins before the wait, while kernels before it still write, so nothing that they may

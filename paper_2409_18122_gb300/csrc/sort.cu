@@ -10,7 +10,7 @@
 // shape depends only on the host-side capacity.
 //
 // Digits have 9 bits, so three passes cover 27.  Depth keys are the bits of positive floats, and
-// a batch whose depths lie within a factor of about 2^8 (0.2 m to 56 m: 2^26 keys apart) differs
+// a batch whose depths lie within a factor of about 2^16 (0.2 m to 13 km: 2^27 keys apart) differs
 // in no more: the low two digits are taken as they are, the third is the rest of the key minus the
 // rest of the smallest key, which fits in 9 bits when the rests differ by less than 512.  The device
 // finds the smallest and largest key during the first counts; only a batch with a wider span runs
