@@ -10,7 +10,7 @@ from oracle import oracle as O
 from paper_2409_18122_gb300 import gs
 from paper_2409_18122_gb300.scenes import Camera, GaussianMap
 
-from gpu_helpers import DEPTH_RTOL, IG_RTOL, IMG_ATOL, images_host
+from gpu_helpers import DEPTH_RTOL, GRAD_RTOL, IG_RTOL, IMG_ATOL, images_host
 
 pytestmark = pytest.mark.gpu
 
@@ -184,3 +184,31 @@ def test_staged_leftovers_never_count_without_an_opacity_floor(n):
             gs.InfoGain(200, cams, prm)(hot)
         ig = float(gs.InfoGain(n, cams, prm)(gm)[0])
         assert abs(ig - ref["unc"].mean()) <= IG_RTOL * abs(ref["unc"].mean()) + 1e-7 + slack
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 31, 33, 50])
+def test_last_and_gradients_without_an_opacity_floor(n):
+    """alpha_min = 0: every entry of the list counts and the padding of a last chunk does not, so
+    `last` is the one-launch render's (it indexes the tile's list) and the adjoint, which replays
+    the list from it, gives the oracle's gradients."""
+    gmap, cams = _stack(n, -2.0)
+    gm = gs.GaussianMapTensors.from_numpy(gmap)
+    ref = O.render_images(gmap, cams, O.Params(16, 16, 0.3, 0.2, 1.3, 0.0, 0.99, 1e-4))[0]
+    rng = np.random.default_rng(n)
+    d = rng.normal(size=(9, 13, 4))
+    d[ref["knife"]] = 0.0
+    gref = O.grad(gmap, cams, [d], O.Params(16, 16, 0.3, 0.2, 1.3, 0.0, 0.99, 1e-4))
+    d_rgb = torch.from_numpy(np.ascontiguousarray(d[..., :3].transpose(2, 0, 1)).reshape(-1)).float().cuda()
+    d_dep = torch.from_numpy(np.ascontiguousarray(d[..., 3]).reshape(-1)).float().cuda()
+    for b in gs.FWD_BATCH_CANDIDATES:
+        prm = gs.RenderParams(alpha_min=0.0, fwd_batch=b)
+        fr = gs.Frame(n, cams, prm)
+        img = fr.forward(gm, fr.new_images(with_counts=True))
+        small, status = gs.render_small(gm, cams, prm)
+        assert int(status) == 0 and torch.equal(img["last"], small["last"])
+        np.testing.assert_array_equal(img["n_contrib"].cpu().numpy().reshape(9, 13)[~ref["knife"]],
+                                      ref["n_contrib"][~ref["knife"]])
+        out = fr.render_bwd(gm, img, d_rgb, d_dep)
+        for k in ("dmo", "dsu", "dq", "drgb"):
+            a, g = out[k].cpu().numpy().astype(np.float64), gref[k]
+            np.testing.assert_allclose(a, g, rtol=0, atol=GRAD_RTOL * np.abs(g).max() + 1e-7, err_msg=k)
